@@ -262,14 +262,14 @@ PTQTP_API ptqtp_status ptqtp_gemm_skinny_static(const ptqtp_shape *shape /* host
  * iterate is (alpha_t, T_t) of the last sweep, without a refit.  canonicalize != 0: afterwards, per group-row and
  * without changing alpha1 T1 + alpha2 T2, both scales are made non-negative (flipping plane and scale) and ordered
  * alpha1 >= alpha2 (exchanging the planes).  The scales are rounded to fp16 once, at the end.
- * Arithmetic: IEEE double precision, every operation rounded on its own, sums in column order: a run is
- * reproducible bit for bit.  group: 1..PTQTP_DECOMPOSE_MAX_GROUP, k % group == 0 (ptqtp_pack needs group = 128);
+ * Arithmetic: IEEE double precision, every operation rounded on its own, sums in column order wherever an order can
+ * matter: planes, scales, sweeps and changes are reproducible bit for bit.  group: 1..PTQTP_DECOMPOSE_MAX_GROUP, k % group == 0 (ptqtp_pack needs group = 128);
  * t_max: 1..PTQTP_DECOMPOSE_MAX_SWEEPS (the paper uses 50, eps = 1e-4).
  * workspace: device, 16-byte aligned, ptqtp_decompose_workspace_size bytes, contents irrelevant on entry.  On
  * return (after syncing) it holds, at the offsets given by ptqtp_decompose_layout: int32 sweeps run; per sweep
  * t = 1..sweeps the largest change of a scale pair (f64 at delta_offset + 8 t) and the total squared error after the
  * sweep (f64 at error_offset + 8 (t - 1)); per group-row the unrounded scales and lambda (f64).
- * 2 t_max + 2 small kernels are enqueued on `stream`; no synchronisation. */
+ * Five kernels are enqueued on `stream`; no synchronisation. */
 #define PTQTP_DECOMPOSE_MAX_GROUP 256
 #define PTQTP_DECOMPOSE_MAX_SWEEPS 1000
 typedef struct {

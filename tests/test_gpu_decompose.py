@@ -89,6 +89,32 @@ def test_degenerate_groups():
     assert np.array_equal(run(W[:16])["T1"], sub["T1"])
 
 
+def _special(kind, rng):
+    """Weights at which the sorted sums, the runs of the quantiser or the second pass can go wrong."""
+    W = (rng.standard_normal((70, 640)) * 0.02).astype(np.float32)
+    if kind == "inexact sums":          # magnitudes too far apart for exact sums, in every group of half of the rows
+        W[::2] *= np.exp2(rng.integers(-40, 3, W[::2].shape)).astype(np.float32)
+    elif kind == "few values":          # ties everywhere: multiples of 1/8, zeros of both signs among them
+        W = (rng.integers(-4, 5, W.shape) / 8).astype(np.float32)
+        W[3:9] *= -1.0
+    elif kind == "short mantissas":     # as from a 16-bit checkpoint
+        W = torch.from_numpy(W).bfloat16().float().numpy()
+    elif kind == "one plane":           # W = c * sign: the second scale is nothing but rounding
+        W = (np.where(rng.random(W.shape) < 0.5, 1.0, -1.0) * 0.3).astype(np.float32)
+    elif kind == "extremes":
+        W[:20] *= np.float32(1e-41)     # subnormal
+        W[20:40] *= np.float32(1e36)
+    return W
+
+
+@pytest.mark.parametrize("kind", ["inexact sums", "few values", "short mantissas", "one plane", "extremes"])
+@pytest.mark.parametrize("G,kw,okw", [(128, {}, {}), (20, {}, {}), (160, {"eps": 1e-2}, {"eps": 1e-2}),
+                                      (5, {"t_max": 2}, {"T_max": 2}), (64, {"eps": 0.0, "t_max": 30}, {"eps": 0.0, "T_max": 30})])
+def test_sorted_sweeps_match_the_oracle(kind, G, kw, okw):
+    W = _special(kind, np.random.default_rng(70 + G))
+    assert_same(run(W, group=G, **kw), decompose_c(W, G=G, **okw), "%s G=%d" % (kind, G))
+
+
 def test_decompose_pack_gemv_pipeline_on_the_gpu():
     # W -> planes on the GPU -> pack -> GEMV, never leaving the device; checked against the oracle's layer product
     # on the same planes and against the dense product at the level of the reconstruction error
