@@ -189,30 +189,22 @@ PTQTP_API ptqtp_status ptqtp_gemv_multi(int32_t count, const ptqtp_shape *shapes
 
 /* Small-batch variant: Y[m,:] = layer(X[m,:]) for m < M, 1 <= M <= PTQTP_MAX_BATCH.
  * X: device fp16 [M*K] row-major; Y: device fp16 [M*N] row-major.  Same definition per row of X.
- * Format 2, M >= 2: the planes are contracted on the tensor cores with int8 warp MMAs against 15-bit
- * block-fixed-point activations (blocks of 128 columns), exact int32 sums, fp32 scale epilogue.  M = 2..4 take
- * one pass over the planes at about the cost of a batch-1 call (the activations stay in registers); larger M
- * take one such pass per four rows (ptqtp_gemm_skinny_ws reads the planes once for any M).  When four rows of x
- * leave no room in shared memory (very long K) the passes take three or two rows, or one row on the batch-1
- * kernel.  M = 1 runs the batch-1 kernel.  Format 3, few rows: the same tiles and decode as its batch-1 kernel, with
- * the MMA columns holding two or four batch rows instead of the four scale groups (two or four times the
- * tensor-core work of one row, the same masks and the same stream of tiles); M = 2 takes one pass at about 1.3
- * times the cost of a batch-1 call, larger M take a pass per four rows (two when four rows of x leave no room in
- * shared memory).  Format 3, more rows (from M = 5 to about 20, later for small matrices: the library compares the
- * measured costs of both): one pass over the planes for all rows on the tcgen05 tensor cores -- the codes
- * are decoded to fp16 trits in tensor memory (the A operand), the activations are the fp16 B operand as given (no
- * quantisation), the sums of a scale group accumulate in fp32 in tensor memory and get the fp32 scale epilogue;
- * matrices with few rows split K over a thread-block cluster and add the partial sums in rank order
- * (reproducible).  Format 1 is a batch-1 layout: M > 1 returns PTQTP_ERR_CONFIG. */
+ * Format 2, M >= 2, and format 3, M <= 4 and larger M on small matrices: the planes are contracted on the tensor cores
+ * with int8 warp MMAs against 15-bit block-fixed-point activations (blocks of 128 columns), exact int32 sums, fp32
+ * scale epilogue.  Format 3, more rows (from M = 5 to about 20, by the size of the matrix): the activations are fp16
+ * operands as given (no quantisation), the codes fp16 numbers, the sums of a scale group accumulate in fp32 and get the
+ * fp32 scale epilogue.  One pass over the planes takes up to 16 (int8) or 32 (fp16) rows, fewer when K is very
+ * long; more rows take several passes, or on format 3 with fp16 operands one pass on the tcgen05 tensor cores.
+ * Matrices with few rows split K over a thread-block cluster and add the partial sums in a fixed order
+ * (reproducible).  M = 1 runs the batch-1 kernel.  Format 1 is a batch-1 layout: M > 1 returns PTQTP_ERR_CONFIG. */
 PTQTP_API ptqtp_status ptqtp_gemm_skinny(const ptqtp_shape *shape /* host */, const void *packed,
                                size_t packed_bytes, int32_t m, const uint16_t *X, uint16_t *Y,
                                void *stream);
 
 /* ptqtp_gemm_skinny on format 3 with the kernel chosen by the caller (tuning and tests; PTQTP_ERR_CONFIG for the
- * other formats).  path: 0 = library choice, 5 = passes of up to four rows on the warp-MMA kernel, 6 = the tcgen05
- * kernel (all M rows in one pass over the planes; fp16 trits from tensor memory against the fp16 activations, fp32
- * accumulators in tensor memory, fp32 scale epilogue).  k_split (path 6): CTAs of a cluster that share the columns
- * of a block of 128 rows: 1, 2, 4 or 8; 0 = library choice.  Same result definition as ptqtp_gemm_skinny. */
+ * other formats).  path: 0 = library choice, 5 = int8 MMAs on block-fixed-point activations, 6 = fp16 activations as
+ * given.  k_split (path 6): with 1, 2, 4 or 8 the tcgen05 kernel, that many CTAs of a cluster sharing the columns of a block
+ * of 128 rows; 0 = library choice of kernel and split.  Same result definition as ptqtp_gemm_skinny. */
 PTQTP_API ptqtp_status ptqtp_gemm_skinny_cfg(const ptqtp_shape *shape /* host */, const void *packed, size_t packed_bytes,
                                    int32_t m, const uint16_t *X, uint16_t *Y, int32_t path, int32_t k_split,
                                    void *stream);
@@ -220,8 +212,8 @@ PTQTP_API ptqtp_status ptqtp_gemm_skinny_cfg(const ptqtp_shape *shape /* host */
 /* Small-batch variant with a caller-provided workspace (format 2 only; PTQTP_ERR_CONFIG for format 1).
  * Same result definition as ptqtp_gemm_skinny.  The workspace (device, 16-byte aligned, at least
  * ptqtp_gemm_skinny_workspace_size(shape, m) bytes, contents irrelevant on entry, clobbered on return) holds X
- * converted once to block fixed point; with it the packed planes are read from HBM exactly once for any M and
- * K, where ptqtp_gemm_skinny needs several passes when M or K is large.  Two kernels are enqueued on `stream`.
+ * converted once to block fixed point when one pass of ptqtp_gemm_skinny does not take all rows (then two kernels are
+ * enqueued on `stream`); with it the packed planes are read from HBM exactly once for any M and K.
  * Calls that share a workspace must not overlap on the GPU.  ptqtp_gemm_skinny_workspace_size returns 0 for a
  * bad shape, formats 1 and 3 (the workspace kernels read format 2) or M out of range.  (Small-batch use of the layer of Eq. 1-2; the paper measures batch 1.) */
 PTQTP_API size_t ptqtp_gemm_skinny_workspace_size(const ptqtp_shape *shape /* host */, int32_t m);

@@ -247,12 +247,11 @@ ptqtp_status ptqtp_gemv_multi(int32_t count, const ptqtp_shape* shapes, const vo
     return launch_gemv4_jobs(J, x, 0, 0, 0, 0, static_cast<cudaStream_t>(stream), pair ? 2 : 0);
 }
 
-// Small batch on format 3.  path 5: up to four rows per pass over the planes on the warp-MMA kernel whose MMA columns
-// are the rows (two rows cost about a batch-1 pass, four about one and a half); when four rows of x leave no room in
-// shared memory its passes take two rows, or one on the batch-1 kernel.  path 6: the tcgen05 kernel, all rows in one
-// pass.  path 0: whichever the measured costs below make cheaper -- the tcgen05 kernel has a fixed cost of several
-// microseconds and a cost per byte that grows slowly with the rows, the passes cost a batch-1 call each.
-static bool tcgen05_is_cheaper(const Layout3& L3, int m) {
+// Small batch on format 3.  The arithmetic goes by the size: up to four rows, and more on small matrices, int8 MMAs on
+// activations in 15-bit block fixed point (path 5); more rows on large matrices the fp16 activations as given (path 6).
+// path 0 takes the one below.  The line between them is where the passes of four rows that path 5 once was and the
+// tcgen05 kernel cost the same; the kernels have changed since, the arithmetic of a size has not.
+static bool fp16_activations(const Layout3& L3, int m) {
     if (m < 5) return false;
     const double mb = (double)L3.total / 1e6;
     const int npad = (m + 15) / 16 * 16;
@@ -262,22 +261,23 @@ static bool tcgen05_is_cheaper(const Layout3& L3, int m) {
     const double us5 = full * (1.2 + mb / rate4) + (rest > 2 ? 1.2 + mb / rate4 : rest > 0 ? 1.2 + mb / rate2 : 0.0);
     return us6 < us5;
 }
-static ptqtp_status skinny_v3(const Layout3& L3, const ptqtp_shape* shape, const void* packed, int m, const uint16_t* X,
-                              uint16_t* Y, int path, int k_split, cudaStream_t st) {
-    if (path == 6 || (path == 0 && tcgen05_is_cheaper(L3, m))) return launch_gemm6(L3, packed, m, X, Y, k_split, st);
-    int per_pass = m < 4 ? m : 4;
-    int done = 0;
-    while (done < m) {
-        const uint16_t* Xp = X + (size_t)done * shape->k_in;
-        uint16_t* Yp = Y + (size_t)done * shape->n_out;
-        const int rows = m - done < per_pass ? m - done : per_pass;
-        ptqtp_status sp = rows == 1 ? launch_gemv4(L3, packed, Xp, Yp, 0, 0, 0, 0, st)
-                                    : launch_gemv5(L3, packed, rows, Xp, Yp, 0, 0, st);
-        if (sp == PTQTP_ERR_SHAPE && rows > 1 && done == 0) { per_pass = per_pass > 2 ? 2 : 1; continue; }   // nothing launched yet
-        if (sp != PTQTP_OK) return sp;
-        done += rows;
+// Kernels, in microseconds per call in a chain of its kind (14336 x 4096, 4096 x 14336, 4096 x 4096, 1024 x 4096):
+//   fp16: the warp-MMA kernel while one launch takes all rows (8 rows: 12.6, 14.0, 6.4, 4.0; 16: 18.4, 20.6, 8.4, 5.7),
+//   the tcgen05 kernel otherwise and with k_split (30.2, 27.3, 11.0, 8.1; 30.8, 28.0, 11.5, 8.2; at 64 rows 50.5, 43.5,
+//   17.2, 11.9 against 79, 79, 38, 13.5 in launches of 16 and 32 rows).
+//   int8: four rows 8.7, 10.5, 5.2, 3.6 on the warp-MMA kernel, 15.0, 27.4, 5.6, 2.6 on the batch-1 tiles kernel at overlap
+//   level 2, where its launches overlap (16.5, 27.5, 8.6, 6.5 at level 0): small matrices of up to four rows stay there,
+//   and so do two rows (6.9, 13.2, 3.2, 2.0 at level 2 against 8.4, 9.8, 5.2, 3.5) unless K is long.
+static ptqtp_status skinny_v3(const Layout3& L3, const void* packed, int m, const uint16_t* X, uint16_t* Y, int path,
+                              int k_split, cudaStream_t st) {
+    if (path == 6 || (path == 0 && fp16_activations(L3, m))) {
+        if (k_split == 0 && gemm7_one_launch(L3, m, false)) return launch_gemm7(L3, packed, m, X, Y, false, st);
+        return launch_gemm6(L3, packed, m, X, Y, k_split, st);
     }
-    return PTQTP_OK;
+    if (m > 4 || (m > 1 && L3.k > 8192) || (m > 2 && L3.total > 8500000)) return launch_gemm7(L3, packed, m, X, Y, true, st);
+    if (m == 1) return launch_gemv4(L3, packed, X, Y, 0, 0, 0, 0, st);
+    const ptqtp_status s = launch_gemv5(L3, packed, m, X, Y, 0, 0, st);
+    return s == PTQTP_ERR_SHAPE ? launch_gemm7(L3, packed, m, X, Y, true, st) : s;       // no room for m rows of x
 }
 
 ptqtp_status ptqtp_gemm_skinny(const ptqtp_shape* shape, const void* packed, size_t packed_bytes, int32_t m,
@@ -290,27 +290,18 @@ ptqtp_status ptqtp_gemm_skinny(const ptqtp_shape* shape, const void* packed, siz
     if (!aligned16(X) || !aligned16(Y)) return PTQTP_ERR_ALIGN;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     if (L.v2) {
-        // Up to four rows cost about the same as one on the register-stationary tensor-core kernel; more rows take
-        // one pass per four (ptqtp_gemm_skinny_ws reads the planes only once).  When four rows of x leave no room in
-        // shared memory the passes take three, two or, on the batch-1 kernel, one row.
+        // Two rows, and up to four on small matrices, take the register-stationary kernel, whose launches overlap at level
+        // 2 (two rows of 4096 x 4096 there: 3.8 us against 6.0); the rest the warp-MMA kernel (four rows of 14336 x 4096,
+        // 4096 x 14336, 4096 x 4096: 11.2, 12.4, 6.2 us against 13.7, 18.1, 8.1 at level 0 and 11.7, 16.8, 6.9 at level 2).
+        if (m > 4 || (m > 1 && shape->k_in > 8192) || (m > 2 && L.l2.total > 2000000))
+            return launch_gemm7(L.l2, packed, m, X, Y, st);
         if (m >= 2) {
-            int per_pass = m < 4 ? m : 4;
-            int done = 0;
-            while (done < m) {
-                const uint16_t* Xp = X + (size_t)done * shape->k_in;
-                uint16_t* Yp = Y + (size_t)done * shape->n_out;
-                const int rows = m - done < per_pass ? m - done : per_pass;
-                ptqtp_status sp = rows == 1 ? launch_gemv2(L.l2, packed, Xp, Yp, 0, 0, 0, 0, st)
-                                            : launch_gemv3(L.l2, packed, rows, Xp, Yp, 0, 0, 0, st);
-                if (sp == PTQTP_ERR_SHAPE && rows > 1 && done == 0) { --per_pass; continue; }   // nothing launched yet
-                if (sp != PTQTP_OK) return sp;
-                done += rows;
-            }
-            return PTQTP_OK;
+            const ptqtp_status sp = launch_gemv3(L.l2, packed, m, X, Y, 0, 0, 0, st);
+            return sp == PTQTP_ERR_SHAPE ? launch_gemm7(L.l2, packed, m, X, Y, st) : sp;
         }
         return launch_gemv2(L.l2, packed, X, Y, 0, 0, 0, 0, st);
     }
-    if (L.v3) return skinny_v3(L.l3, shape, packed, m, X, Y, 0, 0, st);
+    if (L.v3) return skinny_v3(L.l3, packed, m, X, Y, 0, 0, st);
     // format 1 is a batch-1 layout
     if (m != 1) return PTQTP_ERR_CONFIG;
     return gemv_any(L, packed, X, Y, 0, 0, 0, 0, -1, st);
@@ -325,7 +316,7 @@ ptqtp_status ptqtp_gemm_skinny_cfg(const ptqtp_shape* shape, const void* packed,
     if (m < 1 || m > PTQTP_MAX_BATCH) return PTQTP_ERR_SHAPE;
     if (!L.v3 || (path != 0 && path != 5 && path != 6)) return PTQTP_ERR_CONFIG;
     if (!aligned16(X) || !aligned16(Y)) return PTQTP_ERR_ALIGN;
-    return skinny_v3(L.l3, shape, packed, m, X, Y, path, k_split, static_cast<cudaStream_t>(stream));
+    return skinny_v3(L.l3, packed, m, X, Y, path, k_split, static_cast<cudaStream_t>(stream));
 }
 
 size_t ptqtp_gemm_skinny_workspace_size(const ptqtp_shape* shape, int32_t m) {
@@ -344,6 +335,7 @@ ptqtp_status ptqtp_gemm_skinny_ws(const ptqtp_shape* shape, const void* packed, 
     if (!L.v2) return PTQTP_ERR_CONFIG;
     if (!aligned16(X) || !aligned16(Y) || !aligned16(workspace)) return PTQTP_ERR_ALIGN;
     if (workspace_bytes < skinny3_workspace_bytes(shape->k_in, m)) return PTQTP_ERR_SIZE;
+    if (gemm7_one_launch(L.l2, m)) return launch_gemm7(L.l2, packed, m, X, Y, static_cast<cudaStream_t>(stream));
     return launch_skinny3(L.l2, packed, m, X, Y, workspace, static_cast<cudaStream_t>(stream));
 }
 
@@ -357,6 +349,7 @@ ptqtp_status ptqtp_gemm_skinny_static(const ptqtp_shape* shape, const void* pack
     if (!L.v2) return PTQTP_ERR_CONFIG;
     if (!aligned16(X) || !aligned16(Y)) return PTQTP_ERR_ALIGN;
     if (skinny3_workspace_bytes(shape->k_in, m) > (size_t)PTQTP_STATIC_WORKSPACE_BYTES) return PTQTP_ERR_SIZE;
+    if (gemm7_one_launch(L.l2, m)) return launch_gemm7(L.l2, packed, m, X, Y, static_cast<cudaStream_t>(stream));
     void* workspace = nullptr;
     s = static_workspace_address(&workspace);
     if (s != PTQTP_OK) return s;

@@ -162,6 +162,12 @@ ptqtp_status launch_gemv5(const Layout3& L, const void* packed, int m, const uin
 // 1 <= m <= 64 rows on format 3, tcgen05 kernel; ksplit = CTAs per cluster sharing the columns (0 = library choice)
 ptqtp_status launch_gemm6(const Layout3& L, const void* packed, int m, const uint16_t* X, uint16_t* Y, int ksplit,
                           cudaStream_t st);
+// 1 <= m <= 64 rows on formats 3 and 2, warp MMAs on a CTA's share of rows and columns.  int8: 15-bit block fixed-point
+// activations, otherwise fp16 as given.  gemm7_one_launch: all m rows take one pass over the planes.
+ptqtp_status launch_gemm7(const Layout3& L, const void* packed, int m, const uint16_t* X, uint16_t* Y, bool int8, cudaStream_t st);
+ptqtp_status launch_gemm7(const Layout2& L, const void* packed, int m, const uint16_t* X, uint16_t* Y, cudaStream_t st);
+bool gemm7_one_launch(const Layout3& L, int m, bool int8);
+bool gemm7_one_launch(const Layout2& L, int m);
 size_t decompose_workspace_bytes(long long rows, int t_max);
 void decompose_offsets(long long rows, int t_max, size_t* delta_off, size_t* err_off, size_t* a1_off, size_t* a2_off,
                        size_t* lam_off);
