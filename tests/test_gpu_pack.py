@@ -145,3 +145,23 @@ def test_guard_bands_untouched(fmt):
     host = buf.cpu().numpy()
     assert np.all(host[:256] == 0xA5) and np.all(host[256 + size:] == 0xA5)
     assert np.array_equal(host[256:256 + size], reference_blob(c, fmt))
+
+
+@pytest.mark.parametrize("fmt", [binding.FORMAT_V2, binding.FORMAT_V3])
+@pytest.mark.parametrize("N,K", [(16, 512), (3, 640), (2049, 4096)])
+def test_every_byte_value_next_to_valid_trits(fmt, N, K):
+    # bytes outside {-1, 0, 1} are stored as trit 0 and reported; the trits beside them in the same word are untouched
+    rng = np.random.default_rng(N + K)
+    planes = [rng.integers(-1, 2, (N, K)).astype(np.int8) for _ in range(2)]
+    for T in planes:
+        where = rng.choice(N * K, 1024, replace=False)
+        T.reshape(-1)[where] = np.tile(np.arange(-128, 128), 4).astype(np.int8)
+    a = [np.abs(rng.standard_normal((N, K // 128)) * 0.02).astype(np.float16) for _ in range(2)]
+    packed, st = binding.ptqtp_pack(*[torch.from_numpy(v).cuda() for v in planes + a], fmt=fmt)
+    U1, U2, b1, b2, st2 = binding.ptqtp_unpack(packed, N, K, fmt=fmt)
+    torch.cuda.synchronize()
+    assert int(st.item()) == binding.ERR_TRIT and int(st2.item()) == 0
+    for T, U in zip(planes, (U1, U2)):
+        assert np.array_equal(U.cpu().numpy(), np.where(np.abs(T.astype(np.int32)) <= 1, T, 0))
+    assert np.array_equal(b1.cpu().numpy().view(np.uint16), a[0].view(np.uint16))
+    assert np.array_equal(b2.cpu().numpy().view(np.uint16), a[1].view(np.uint16))
