@@ -175,8 +175,9 @@ gemv2_kernel(Layout2 L, const unsigned char* __restrict__ packed, const __half* 
     constexpr int kSlot = RU * kUnit2;                 // a ring slot holds the RU units of one copy
     unsigned char* ring = smem + sm.ring_off + (size_t)warp * D * kSlot;
 
-    // Let the next kernel on the stream start while this one runs.
-    asm volatile("griddepcontrol.launch_dependents;");
+    // Speculative: let the next kernel on the stream start while this one runs; otherwise once everything before this one is
+    // complete.
+    if (speculate) asm volatile("griddepcontrol.launch_dependents;");
 
     // this CTA's row pairs, and this warp's share of their slice units
     // balanced partition computed on the host: the first rp_rem CTAs take rp_base + 1 row pairs, the rest rp_base
@@ -236,6 +237,7 @@ gemv2_kernel(Layout2 L, const unsigned char* __restrict__ packed, const __half* 
         if (!spec && !waited) {
             asm volatile("griddepcontrol.wait;" ::: "memory");
             waited = true;
+            if (!speculate) asm volatile("griddepcontrol.launch_dependents;");
         }
         pt = n_rp > 0 ? 0 : n_sl;
         pleft = n_rp;
@@ -424,7 +426,8 @@ ptqtp_status launch_d(const Layout2& L, const void* packed, const uint16_t* x, u
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = overlap_enabled() && !consume_pack(st) ? 1 : 0;   // plain right after a pack on this stream
+    // level 0: a dependent launch that touches nothing before its wait; otherwise plain right after a pack on this stream
+    cfg.numAttrs = !overlap_enabled() || !consume_pack(st) ? 1 : 0;
     cudaError_t e = cudaLaunchKernelEx(&cfg, kern, L, static_cast<const unsigned char*>(packed),
                                        reinterpret_cast<const __half*>(x), reinterpret_cast<__half*>(y), rows_cap,
                                        L.nrp / grid, L.nrp % grid, speculate, gated);

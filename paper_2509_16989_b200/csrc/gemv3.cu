@@ -199,8 +199,9 @@ gemv3_kernel(Layout2 L, const unsigned char* __restrict__ packed, const __half* 
     uint64_t* empty = full + depth;
     unsigned char* ring = rings + (size_t)team * depth * kStage3;
 
-    // Let the next kernel on the stream start while this one runs.
-    asm volatile("griddepcontrol.launch_dependents;");
+    // Speculative: let the next kernel on the stream start while this one runs; otherwise once everything before this one is
+    // complete.
+    if (speculate) asm volatile("griddepcontrol.launch_dependents;");
 
     // this CTA's quads (balanced partition from the host); team tm takes tasks [tm T / teams, (tm + 1) T / teams)
     // of the (slice, quad) list
@@ -262,6 +263,7 @@ gemv3_kernel(Layout2 L, const unsigned char* __restrict__ packed, const __half* 
         if (!spec && !waited) {
             asm volatile("griddepcontrol.wait;" ::: "memory");
             waited = true;
+            if (!speculate) asm volatile("griddepcontrol.launch_dependents;");
         }
         // The packed planes do not depend on earlier work of the stream: two stages are requested first, the
         // rest of the ring while the first reads of x are in flight.
@@ -459,7 +461,8 @@ ptqtp_status launch_gemv3(const Layout2& L, const void* packed, int m, const uin
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = overlap_enabled() && !consume_pack(st) ? 1 : 0;   // plain right after a pack on this stream
+    // level 0: a dependent launch that touches nothing before its wait; otherwise plain right after a pack on this stream
+    cfg.numAttrs = !overlap_enabled() || !consume_pack(st) ? 1 : 0;
     cudaError_t e = cudaLaunchKernelEx(&cfg, gemv3_kernel, L, static_cast<const unsigned char*>(packed),
                                        reinterpret_cast<const __half*>(X), reinterpret_cast<__half*>(Y), m, rows_cap,
                                        nquads / grid, nquads % grid, teams, depth, speculate, status_word);

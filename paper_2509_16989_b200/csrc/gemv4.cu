@@ -178,7 +178,7 @@ __device__ __forceinline__ Share4 share_of(const Jobs4& J, int j, int wi, int m,
 // kMulti = false is the same kernel for a single matrix with the job loops folded away.
 template <int D, int RU, bool kMulti>
 __global__ void __launch_bounds__(kRegBound4, 1)
-gemv4_kernel(const __grid_constant__ Jobs4 J, const __half* __restrict__ x, int rows_cap, int speculate, int overlap,
+gemv4_kernel(const __grid_constant__ Jobs4 J, const __half* __restrict__ x, int rows_cap, int speculate,
              int gated, int spin_limit, int inject, int* __restrict__ status_word) {
     extern __shared__ __align__(128) unsigned char smem[];
     const int S = J.sbs;
@@ -196,8 +196,9 @@ gemv4_kernel(const __grid_constant__ Jobs4 J, const __half* __restrict__ x, int 
     constexpr int kSlot = RU * kTile3;                 // a ring slot holds the RU tiles of one copy
     unsigned char* ring = smem + sm.ring_off + (size_t)warp * D * kSlot;
 
-    // Let the next kernel on the stream start while this one runs.
-    asm volatile("griddepcontrol.launch_dependents;");
+    // Speculative: let the next kernel on the stream start while this one runs.  Otherwise only once everything before this
+    // one is complete, see the wait below.
+    if (speculate) asm volatile("griddepcontrol.launch_dependents;");
 
     const int Wc = min(S, warps);                       // superblock lanes among the warps
     const int m = warps / Wc;                           // warps sharing a superblock lane
@@ -295,29 +296,25 @@ gemv4_kernel(const __grid_constant__ Jobs4 J, const __half* __restrict__ x, int 
         const bool spec = speculate && attempt == 0;
         // x as it is, by one bulk copy (through L2, the point of coherence): one round trip whatever K is.  It is
         // requested before the ring is filled (copies complete in the order they were requested: behind a full
-        // ring x would arrive microseconds later), except under a dependent launch without speculative execution,
-        // where the planes, which do not depend on earlier work of the stream, are requested before the wait.
+        // ring x would arrive microseconds later).  Without speculative execution nothing is read before earlier work of
+        // the stream is complete: tiles requested ahead of that delay x, and tiles prefetched into L2 meanwhile delay
+        // what the kernel before still streams (four-launch layer of LLaMA-3-8B, two layers: 65.5 us as it is, 71 with one
+        // tile per warp, 80 with a prefetch of eight).
         pt = 0;
         pj = 0;
         seek();
-        const bool fill_first = !spec && !waited && overlap;
-        if (fill_first) {
-#pragma unroll
-            for (int d = 0; d < D; ++d) issue();
-        }
         if (!spec && !waited) {
             asm volatile("griddepcontrol.wait;" ::: "memory");
             waited = true;
+            if (!speculate) asm volatile("griddepcontrol.launch_dependents;");
         }
         if (threadIdx.x == 0) {
             mbar_expect_tx(xbar_a, xbytes);
             bulk_copy_g2s(smem_u32(raw), x, xbytes, xbar_a);
         }
         __syncthreads();                                // the mbarrier of x is initialised and armed before anyone polls it
-        if (!fill_first) {                              // (and x has been requested before any tile)
 #pragma unroll
-            for (int d = 0; d < D; ++d) issue();
-        }
+        for (int d = 0; d < D; ++d) issue();            // (x has been requested before any tile)
         if (!mbar_try_wait(xbar_a, (uint32_t)attempt)) {
             const int limit = failed ? kSpinAfterFailure4 : spin_limit;
             int spins = 0;
@@ -502,9 +499,12 @@ ptqtp_status launch_d4(const Jobs4& J, const uint16_t* x, int grid, int warps, i
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = overlap_enabled() && !consume_pack(st) ? 1 : 0;   // plain right after a pack on this stream
+    // Always a dependent launch: without speculative execution it sets itself up while the kernel before it drains and touches
+    // nothing before the wait (a layer of LLaMA-3-8B in seven plain launches: 48.3 us, 41.0 like this); with it the planes
+    // and x are read at once, so plain right after a pack on this stream.
+    cfg.numAttrs = !speculate || !consume_pack(st) ? 1 : 0;
     cudaError_t e = cudaLaunchKernelEx(&cfg, gemv4_kernel<D, RU, kMulti>, J, reinterpret_cast<const __half*>(x), rows_cap, speculate,
-                                       overlap_enabled() ? 1 : 0, gated, wait_poll_limit(),
+                                       gated, wait_poll_limit(),
                                        take_injected_wait_failure() ? 1 : 0, status_word);
     if (e != cudaSuccess) { set_last_cuda_error(e); (void)cudaGetLastError(); return PTQTP_ERR_CUDA; }
     return PTQTP_OK;
@@ -543,7 +543,7 @@ ptqtp_status launch_gemv4_jobs(Jobs4& J, const uint16_t* x, int warps, int ctas_
         rb_cap += J.rb_base[j] + (J.rb_rem[j] ? 1 : 0);
     }
     const int rows_cap = 16 * rb_cap;
-    const bool alone = warps == -1 || (warps == 0 && !overlap_enabled());   // plain launches never share an SM
+    const bool alone = warps == -1 || (warps == 0 && !speculation_enabled());   // nothing to gain from sharing an SM with the next launch
     if (warps <= 0) {
         if (alone) {
             // one CTA has the SM to itself: as many warps as have tiles to stream

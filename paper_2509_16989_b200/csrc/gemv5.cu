@@ -144,8 +144,8 @@ gemv5_kernel(Layout3 L, const unsigned char* __restrict__ packed, const __half* 
     uint64_t* xbar = reinterpret_cast<uint64_t*>(smem + sm.bar_off) + warps * D;
     unsigned char* ring = smem + sm.ring_off + (size_t)warp * D * kTile3;
 
-    // Let the next kernel on the stream start while this one runs.
-    asm volatile("griddepcontrol.launch_dependents;");
+    // Let the next kernel on the stream start while this one runs (without overlap: once everything before this one is complete).
+    if (overlap) asm volatile("griddepcontrol.launch_dependents;");
 
     // this CTA's row blocks (balanced partition from the host) and this warp's share of their tiles
     const int rb0 = (int)blockIdx.x * rb_base + min((int)blockIdx.x, rb_rem);
@@ -220,6 +220,7 @@ gemv5_kernel(Layout3 L, const unsigned char* __restrict__ packed, const __half* 
         if (!spec && !waited) {
             asm volatile("griddepcontrol.wait;" ::: "memory");
             waited = true;
+            if (!overlap) asm volatile("griddepcontrol.launch_dependents;");
         }
         if (threadIdx.x == 0) {                         // X by one bulk copy, requested before any tile
             mbar_expect_tx(xbar_a, xbytes);
@@ -428,7 +429,8 @@ ptqtp_status launch_d5(const Layout3& L, const void* packed, int m, const uint16
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = overlap_enabled() && !consume_pack(st) ? 1 : 0;   // plain right after a pack on this stream
+    // level 0: a dependent launch that touches nothing before its wait; otherwise plain right after a pack on this stream
+    cfg.numAttrs = !overlap_enabled() || !consume_pack(st) ? 1 : 0;
     cudaError_t e = cudaLaunchKernelEx(&cfg, gemv5_kernel<D, MB>, L, static_cast<const unsigned char*>(packed),
                                        reinterpret_cast<const __half*>(X), reinterpret_cast<__half*>(Y), m, rows_cap,
                                        L.nrb / grid, L.nrb % grid, speculation_enabled() ? 1 : 0, overlap_enabled() ? 1 : 0,
