@@ -116,6 +116,22 @@ def status_string(status):
     return lib().ptqtp_status_string(int(status)).decode()
 
 
+# Shapes already marshalled, by value, with the reference that the foreign calls take: building one costs half a microsecond
+# of the few that a call takes on the host.  Read only; bounded.
+_shapes = {}
+
+
+def _shape_ref(N, K, fmt):
+    key = (int(N), int(K), int(DEFAULT_FORMAT if fmt is None else fmt))
+    ref = _shapes.get(key)
+    if ref is None:
+        ref = ctypes.byref(make_shape(N, K, fmt=fmt))
+        if len(_shapes) >= 1024:
+            _shapes.clear()
+        _shapes[key] = ref
+    return ref
+
+
 def make_shape(N, K, group=GROUP, fmt=None):
     if fmt is None:
         fmt = DEFAULT_FORMAT
@@ -123,19 +139,18 @@ def make_shape(N, K, group=GROUP, fmt=None):
 
 
 def packed_size(N, K, fmt=None):
-    return int(lib().ptqtp_packed_size(ctypes.byref(make_shape(N, K, fmt=fmt))))
+    return int(lib().ptqtp_packed_size(_shape_ref(N, K, fmt)))
 
 
 def _stream_ptr(stream):
-    if stream is None:
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream)
+    # the address as a plain int: no Stream object is made for the current stream
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()) if stream is None else stream.cuda_stream
 
 
 def _dev(t, dtype, what):
-    if not (isinstance(t, torch.Tensor) and t.is_cuda and t.is_contiguous() and t.dtype == dtype):
+    if not (isinstance(t, torch.Tensor) and t.is_cuda and t.dtype == dtype and t.is_contiguous()):
         raise TypeError("%s must be a contiguous CUDA tensor of dtype %s" % (what, dtype))
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 def _check(status, what):
@@ -146,7 +161,7 @@ def _check(status, what):
 def ptqtp_pack(T1, T2, alpha1, alpha2, packed=None, dev_status=None, stream=None, fmt=None):
     """Pack int8 planes [N,K] and fp16 scales [N,K/128] (CUDA tensors).  Returns (packed uint8 tensor, dev_status)."""
     N, K = T1.shape
-    shape = make_shape(N, K, fmt=fmt)
+    shape = _shape_ref(N, K, fmt)
     nbytes = packed_size(N, K, fmt=fmt)
     if nbytes == 0:
         raise PtqtpError(ERR_SHAPE, "ptqtp_packed_size")
@@ -154,7 +169,7 @@ def ptqtp_pack(T1, T2, alpha1, alpha2, packed=None, dev_status=None, stream=None
         packed = torch.empty(nbytes, dtype=torch.uint8, device=T1.device)
     if dev_status is None:
         dev_status = torch.zeros(1, dtype=torch.int32, device=T1.device)
-    st = lib().ptqtp_pack(ctypes.byref(shape), _dev(T1, torch.int8, "T1"), _dev(T2, torch.int8, "T2"),
+    st = lib().ptqtp_pack(shape, _dev(T1, torch.int8, "T1"), _dev(T2, torch.int8, "T2"),
                           _dev(alpha1, torch.float16, "alpha1"), _dev(alpha2, torch.float16, "alpha2"),
                           _dev(packed, torch.uint8, "packed"), packed.numel(),
                           _dev(dev_status, torch.int32, "dev_status"), _stream_ptr(stream))
@@ -164,7 +179,7 @@ def ptqtp_pack(T1, T2, alpha1, alpha2, packed=None, dev_status=None, stream=None
 
 def ptqtp_unpack(packed, N, K, dev_status=None, stream=None, fmt=None):
     """Inverse of ptqtp_pack.  Returns (T1, T2, alpha1, alpha2, dev_status) as CUDA tensors."""
-    shape = make_shape(N, K, fmt=fmt)
+    shape = _shape_ref(N, K, fmt)
     dev = packed.device
     T1 = torch.empty((N, K), dtype=torch.int8, device=dev)
     T2 = torch.empty((N, K), dtype=torch.int8, device=dev)
@@ -172,7 +187,7 @@ def ptqtp_unpack(packed, N, K, dev_status=None, stream=None, fmt=None):
     a2 = torch.empty((N, K // GROUP), dtype=torch.float16, device=dev)
     if dev_status is None:
         dev_status = torch.zeros(1, dtype=torch.int32, device=dev)
-    st = lib().ptqtp_unpack(ctypes.byref(shape), _dev(packed, torch.uint8, "packed"), packed.numel(),
+    st = lib().ptqtp_unpack(shape, _dev(packed, torch.uint8, "packed"), packed.numel(),
                             _dev(T1, torch.int8, "T1"), _dev(T2, torch.int8, "T2"),
                             _dev(a1, torch.float16, "alpha1"), _dev(a2, torch.float16, "alpha2"),
                             _dev(dev_status, torch.int32, "dev_status"), _stream_ptr(stream))
@@ -182,10 +197,10 @@ def ptqtp_unpack(packed, N, K, dev_status=None, stream=None, fmt=None):
 
 def ptqtp_gemv(packed, N, K, x, y=None, stream=None, fmt=None):
     """y[N] = layer(x[K]) from a packed blob; fp16 CUDA tensors."""
-    shape = make_shape(N, K, fmt=fmt)
+    shape = _shape_ref(N, K, fmt)
     if y is None:
         y = torch.empty(N, dtype=torch.float16, device=x.device)
-    st = lib().ptqtp_gemv(ctypes.byref(shape), _dev(packed, torch.uint8, "packed"), packed.numel(),
+    st = lib().ptqtp_gemv(shape, _dev(packed, torch.uint8, "packed"), packed.numel(),
                           _dev(x, torch.float16, "x"), _dev(y, torch.float16, "y"), _stream_ptr(stream))
     _check(st, "ptqtp_gemv")
     return y
@@ -193,10 +208,10 @@ def ptqtp_gemv(packed, N, K, x, y=None, stream=None, fmt=None):
 
 def ptqtp_gemv_cfg(packed, N, K, x, y=None, rows_per_warp=0, k_split=0, ctas_per_sm=0, depth=0, arith=-1,
                    stream=None, fmt=None):
-    shape = make_shape(N, K, fmt=fmt)
+    shape = _shape_ref(N, K, fmt)
     if y is None:
         y = torch.empty(N, dtype=torch.float16, device=x.device)
-    st = lib().ptqtp_gemv_cfg(ctypes.byref(shape), _dev(packed, torch.uint8, "packed"), packed.numel(),
+    st = lib().ptqtp_gemv_cfg(shape, _dev(packed, torch.uint8, "packed"), packed.numel(),
                               _dev(x, torch.float16, "x"), _dev(y, torch.float16, "y"),
                               int(rows_per_warp), int(k_split), int(ctas_per_sm), int(depth), int(arith),
                               _stream_ptr(stream))
@@ -206,10 +221,10 @@ def ptqtp_gemv_cfg(packed, N, K, x, y=None, rows_per_warp=0, k_split=0, ctas_per
 
 def ptqtp_gemv_swiglu(packed, N, K, x, y=None, stream=None, fmt=FORMAT_V2):
     """y[N/2] = silu(row 2i) * row 2i+1 of the layer applied to x; packed holds gate/up rows interleaved (format 2 or 3)."""
-    shape = make_shape(N, K, fmt=fmt)
+    shape = _shape_ref(N, K, fmt)
     if y is None:
         y = torch.empty(N // 2, dtype=torch.float16, device=x.device)
-    st = lib().ptqtp_gemv_swiglu(ctypes.byref(shape), _dev(packed, torch.uint8, "packed"), packed.numel(),
+    st = lib().ptqtp_gemv_swiglu(shape, _dev(packed, torch.uint8, "packed"), packed.numel(),
                                  _dev(x, torch.float16, "x"), _dev(y, torch.float16, "y"), _stream_ptr(stream))
     _check(st, "ptqtp_gemv_swiglu")
     return y
@@ -260,9 +275,9 @@ def ptqtp_gemv_multi(packed_list, N_list, K, x, ys=None, epilogue=EPILOGUE_NONE,
     n_out = 1 if epilogue == EPILOGUE_GATED_PAIR else count
     if ys is None:
         ys = [torch.empty(N_list[j], dtype=torch.float16, device=x.device) for j in range(n_out)]
-    ptrs = (ctypes.c_void_p * count)(*[_dev(p, torch.uint8, "packed").value for p in packed_list])
+    ptrs = (ctypes.c_void_p * count)(*[_dev(p, torch.uint8, "packed") for p in packed_list])
     sizes = (ctypes.c_size_t * count)(*[p.numel() for p in packed_list])
-    yp = (ctypes.c_void_p * count)(*([_dev(y, torch.float16, "y").value for y in ys] + [None] * (count - len(ys))))
+    yp = (ctypes.c_void_p * count)(*([_dev(y, torch.float16, "y") for y in ys] + [None] * (count - len(ys))))
     st = lib().ptqtp_gemv_multi(count, shapes, ptrs, sizes, _dev(x, torch.float16, "x"), yp, int(epilogue),
                                 _stream_ptr(stream))
     _check(st, "ptqtp_gemv_multi")
@@ -271,11 +286,11 @@ def ptqtp_gemv_multi(packed_list, N_list, K, x, ys=None, epilogue=EPILOGUE_NONE,
 
 def ptqtp_gemm_skinny(packed, N, K, X, Y=None, stream=None, fmt=None):
     """Y[M,N] = layer applied to each row of X[M,K]; fp16 CUDA tensors, 1 <= M <= 64."""
-    shape = make_shape(N, K, fmt=fmt)
+    shape = _shape_ref(N, K, fmt)
     M = X.shape[0]
     if Y is None:
         Y = torch.empty((M, N), dtype=torch.float16, device=X.device)
-    st = lib().ptqtp_gemm_skinny(ctypes.byref(shape), _dev(packed, torch.uint8, "packed"), packed.numel(),
+    st = lib().ptqtp_gemm_skinny(shape, _dev(packed, torch.uint8, "packed"), packed.numel(),
                                  int(M), _dev(X, torch.float16, "X"), _dev(Y, torch.float16, "Y"),
                                  _stream_ptr(stream))
     _check(st, "ptqtp_gemm_skinny")
@@ -284,11 +299,11 @@ def ptqtp_gemm_skinny(packed, N, K, X, Y=None, stream=None, fmt=None):
 
 def ptqtp_gemm_skinny_cfg(packed, N, K, X, Y=None, path=0, k_split=0, stream=None):
     """ptqtp_gemm_skinny on format 3 with the kernel chosen by the caller (path 0 / 5 / 6, k_split 0 / 1 / 2 / 4 / 8)."""
-    shape = make_shape(N, K, fmt=FORMAT_V3)
+    shape = _shape_ref(N, K, FORMAT_V3)
     M = X.shape[0]
     if Y is None:
         Y = torch.empty((M, N), dtype=torch.float16, device=X.device)
-    st = lib().ptqtp_gemm_skinny_cfg(ctypes.byref(shape), _dev(packed, torch.uint8, "packed"), packed.numel(),
+    st = lib().ptqtp_gemm_skinny_cfg(shape, _dev(packed, torch.uint8, "packed"), packed.numel(),
                                      int(M), _dev(X, torch.float16, "X"), _dev(Y, torch.float16, "Y"), int(path),
                                      int(k_split), _stream_ptr(stream))
     _check(st, "ptqtp_gemm_skinny_cfg")
@@ -296,18 +311,18 @@ def ptqtp_gemm_skinny_cfg(packed, N, K, X, Y=None, path=0, k_split=0, stream=Non
 
 
 def gemm_skinny_workspace_size(N, K, M, fmt=None):
-    return int(lib().ptqtp_gemm_skinny_workspace_size(ctypes.byref(make_shape(N, K, fmt=fmt)), int(M)))
+    return int(lib().ptqtp_gemm_skinny_workspace_size(_shape_ref(N, K, fmt), int(M)))
 
 
 def ptqtp_gemm_skinny_ws(packed, N, K, X, Y=None, workspace=None, stream=None, fmt=None):
     """ptqtp_gemm_skinny with a caller-provided workspace (uint8 CUDA tensor; allocated here if None)."""
-    shape = make_shape(N, K, fmt=fmt)
+    shape = _shape_ref(N, K, fmt)
     M = X.shape[0]
     if Y is None:
         Y = torch.empty((M, N), dtype=torch.float16, device=X.device)
     if workspace is None:
         workspace = torch.empty(gemm_skinny_workspace_size(N, K, M, fmt=fmt), dtype=torch.uint8, device=X.device)
-    st = lib().ptqtp_gemm_skinny_ws(ctypes.byref(shape), _dev(packed, torch.uint8, "packed"), packed.numel(), int(M),
+    st = lib().ptqtp_gemm_skinny_ws(shape, _dev(packed, torch.uint8, "packed"), packed.numel(), int(M),
                                     _dev(X, torch.float16, "X"), _dev(Y, torch.float16, "Y"),
                                     _dev(workspace, torch.uint8, "workspace"), workspace.numel(), _stream_ptr(stream))
     _check(st, "ptqtp_gemm_skinny_ws")
@@ -323,8 +338,8 @@ def ptqtp_gemm_skinny_static(packed, N, K, X, Y, stream=None, fmt=None):
     Y must be passed in (this wrapper allocates nothing either).  Raises PtqtpError(ERR_SIZE) when
     gemm_skinny_workspace_size(N, K, M) exceeds STATIC_WORKSPACE_BYTES.  Calls share one array per device:
     do not let two of them overlap on the GPU."""
-    shape = make_shape(N, K, fmt=fmt)
-    st = lib().ptqtp_gemm_skinny_static(ctypes.byref(shape), _dev(packed, torch.uint8, "packed"), packed.numel(),
+    shape = _shape_ref(N, K, fmt)
+    st = lib().ptqtp_gemm_skinny_static(shape, _dev(packed, torch.uint8, "packed"), packed.numel(),
                                         int(X.shape[0]), _dev(X, torch.float16, "X"), _dev(Y, torch.float16, "Y"),
                                         _stream_ptr(stream))
     _check(st, "ptqtp_gemm_skinny_static")
@@ -333,12 +348,12 @@ def ptqtp_gemm_skinny_static(packed, N, K, X, Y, stream=None, fmt=None):
 
 def ptqtp_gemv_host(packed, N, K, x_host, y_host, x_dev, y_dev, stream=None, fmt=None):
     """Host-buffer call: H2D copy of x, GEMV, D2H copy of y, all on `stream` (no sync)."""
-    shape = make_shape(N, K, fmt=fmt)
+    shape = _shape_ref(N, K, fmt)
     for t, what in ((x_host, "x_host"), (y_host, "y_host")):
         if t.is_cuda or t.dtype != torch.float16 or not t.is_contiguous():
             raise TypeError("%s must be a contiguous fp16 host tensor" % what)
-    st = lib().ptqtp_gemv_host(ctypes.byref(shape), _dev(packed, torch.uint8, "packed"), packed.numel(),
-                               ctypes.c_void_p(x_host.data_ptr()), ctypes.c_void_p(y_host.data_ptr()),
+    st = lib().ptqtp_gemv_host(shape, _dev(packed, torch.uint8, "packed"), packed.numel(),
+                               x_host.data_ptr(), y_host.data_ptr(),
                                _dev(x_dev, torch.float16, "x_dev"), _dev(y_dev, torch.float16, "y_dev"),
                                _stream_ptr(stream))
     _check(st, "ptqtp_gemv_host")
