@@ -127,41 +127,28 @@ __device__ __forceinline__ void mma_f16_first(float (&c)[4], uint32_t a0, uint32
         : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "f"(0.f));
 }
 
-// One launch.  tile0, tiles: the tiles (8 row pairs) of this launch; all_tiles: of the matrix; chunk: superblocks of
-// activations held at a time.
-struct Args7 {
-    const unsigned char* codes;
-    const __half* X;
-    __half* Y;
-    int n, k, m, nrp, tile0, tiles, all_tiles, sbs;
-    int slices, last_active, last_unit;                // format 2
-    int csize, clusters, kw, chunk, early, spin_limit, inject;
-    int* status_word;
-};
-
 // Offsets in dynamic shared memory: the warps' rings, the activations of a chunk in fragment order, the negated group sums of
 // x, the partial sums pushed here [own tile][source][16][stride], sums kept between chunks, barriers (one per ring slot,
 // one for the partial sums).
 struct Smem7 {
-    size_t x, sx, red, keep, bars, total;
+    uint32_t x, sx, red, keep, bars;
+    size_t total;
 };
-__host__ __device__ inline int red_stride7(int npad) { return npad + 2; }      // rows two banks apart
-__host__ __device__ inline Smem7 smem7(int fmt, int npad, int warps, int chunk, int own_tiles, int sources, int kept_tiles) {
-    Smem7 s;
-    s.x = (size_t)(warps / team7(fmt)) * kDepth7 * (fmt == 3 ? kTile3 : kTile2);
-    s.sx = s.x + (size_t)chunk * npad * 1024;
-    s.red = s.sx + (size_t)chunk * 4 * npad * 8;
-    s.keep = s.red + (size_t)own_tiles * sources * 16 * red_stride7(npad) * 4;
-    s.bars = (s.keep + (size_t)kept_tiles * 16 * npad * 4 + 15) / 16 * 16;
-    s.total = s.bars + (size_t)(warps * kDepth7 + 1) * 8 + 8;
+inline int red_stride7(int npad) { return npad + 2; }      // rows two banks apart
+inline Smem7 smem7(int fmt, int npad, int warps, int chunk, int own_tiles, int sources, int kept_tiles) {
+    const size_t x = (size_t)(warps / team7(fmt)) * kDepth7 * (fmt == 3 ? kTile3 : kTile2);
+    const size_t sx = x + (size_t)chunk * npad * 1024, red = sx + (size_t)chunk * 4 * npad * 8;
+    const size_t keep = red + (size_t)own_tiles * sources * 16 * red_stride7(npad) * 4;
+    const size_t bars = (keep + (size_t)kept_tiles * 16 * npad * 4 + 15) / 16 * 16;
+    const Smem7 s = {(uint32_t)x, (uint32_t)sx, (uint32_t)red, (uint32_t)keep, (uint32_t)bars, bars + (size_t)(warps * kDepth7 + 1) * 8 + 8};
     return s;
 }
 
-// int8: eight batch rows (two column tiles) of one group, 32 of its columns per lane (runs t and t + 4 of 16), to 15-bit
+// int8: batch row `row` of column tile nt, 32 columns of one group per lane (runs t and t + 4 of 16), to 15-bit
 // block fixed point: X = round(x 2^s) with the group maximum in [2^13, 2^14), X = 256 hi + lo with both bytes signed, high
 // bytes in the even MMA columns, low bytes in the odd ones.
 template <int FMT, int NT>
-__device__ __forceinline__ void convert7(const uint4 (&r)[2][2], int grp, int pair, int g, int t, unsigned char* xs, int2* records) {
+__device__ __forceinline__ void convert7(const uint4 (&r)[2][2], int grp, int nt, int row, int t, unsigned char* xs, int2* records) {
     uint32_t v[2][8];
     uint32_t m2 = 0u;
 #pragma unroll
@@ -181,7 +168,6 @@ __device__ __forceinline__ void convert7(const uint4 (&r)[2][2], int grp, int pa
         s = 13 - ex;
     }
     const float scale = __uint_as_float((uint32_t)(127 + s) << 23);
-    const int nt = 2 * pair + (g >> 2), row = g & 3;
     uint32_t sum = 0u;
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
@@ -270,9 +256,23 @@ __device__ __forceinline__ void group_int8(const uint32_t (&word)[8], const unsi
     }
 }
 
+// One launch.  The shares are divided on the host (a dozen integer divisions per warp were half a microsecond of a launch): tile0
+// and the tiles (8 row pairs) of a cluster, the superblocks of a rank, C = 1 << lg_csize, kw = 1 << lg_kw; all_tiles: of
+// the matrix; chunk: superblocks of activations held at a time.
+struct Args7 {
+    const unsigned char* codes;
+    const __half* X;
+    __half* Y;
+    int n, k, m, nrp, tile0, t_base, t_rem, all_tiles, sbs, s_base, s_rem;
+    int slices, last_active, last_unit;                // format 2
+    int lg_csize, lg_kw, chunk, early, spin_limit, inject;
+    Smem7 at;
+    int* status_word;
+};
+
 template <int FMT, bool INT8, int NT>
 __global__ void __launch_bounds__(max_warps7(INT8, NT) * 32, 1)
-gemm7_kernel(const Args7 a, const int own_cap, const int rounds_cap) {
+gemm7_kernel(const __grid_constant__ Args7 a) {
     extern __shared__ __align__(128) unsigned char smem[];
     constexpr int ROWS = INT8 ? 4 : 8;                   // batch rows per MMA column tile
     constexpr int NPAD = ROWS * NT, RS = NPAD + 2;
@@ -280,24 +280,21 @@ gemm7_kernel(const Args7 a, const int own_cap, const int rounds_cap) {
     constexpr int kTileBytes = FMT == 3 ? kTile3 : kTile2, TEAM = team7(FMT);
     const int warps = blockDim.x >> 5, warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
     const int g = lane >> 2, t = lane & 3;
-    const int csize = a.csize, crank = (int)blockIdx.x % csize, cl = (int)blockIdx.x / csize;
+    const int csize = 1 << a.lg_csize, crank = (int)blockIdx.x & (csize - 1), cl = (int)blockIdx.x >> a.lg_csize;
     // this cluster's tiles, this rank's superblocks, this warp's share of both
-    const int t_lo = a.tile0 + cl * (a.tiles / a.clusters) + min(cl, a.tiles % a.clusters);
-    const int T = a.tiles / a.clusters + (cl < a.tiles % a.clusters ? 1 : 0);
+    const int t_lo = a.tile0 + cl * a.t_base + min(cl, a.t_rem), T = a.t_base + (cl < a.t_rem ? 1 : 0);
     constexpr int S = FMT == 3 ? 1 : 4;                  // superblocks that stay together
-    const int blocks = (a.sbs + S - 1) / S;
-    const int sb_lo = S * (crank * (blocks / csize) + min(crank, blocks % csize));
-    const int sb_hi = min(a.sbs, sb_lo + S * (blocks / csize + (crank < blocks % csize ? 1 : 0)));
-    const int kw = a.kw, tw = warps / kw, kl = warp % kw, tl = warp / kw;
-    const int chunks = max(1, (sb_hi - sb_lo + a.chunk - 1) / a.chunk);
-    const int sources = csize * kw;
-    const Smem7 so = smem7(FMT, NPAD, warps, a.chunk, own_cap, sources, rounds_cap * warps);
+    const int sb_lo = S * (crank * a.s_base + min(crank, a.s_rem));
+    const int sb_hi = min(a.sbs, sb_lo + S * (a.s_base + (crank < a.s_rem ? 1 : 0)));
+    const int kw = 1 << a.lg_kw, tw = warps >> a.lg_kw, kl = warp & (kw - 1), tl = warp >> a.lg_kw;
+    const int sources = csize << a.lg_kw;
+    const Smem7& so = a.at;
     const uint32_t ring = smem_u32(smem) + (uint32_t)(warp / TEAM * kDepth7 * kTileBytes), xs = smem_u32(smem + so.x), red = smem_u32(smem + so.red);
     unsigned char* ring_p = smem + (size_t)(warp / TEAM) * kDepth7 * kTileBytes;
     float* sx = reinterpret_cast<float*>(smem + so.sx);                   // fp16: minus the sum of x
     int2* records = reinterpret_cast<int2*>(smem + so.sx);                // int8: (2^-s, sum of the integers)
     const uint32_t bars = smem_u32(smem + so.bars) + 8 * (warp / TEAM) * kDepth7, r_full = smem_u32(smem + so.bars) + 8 * warps * kDepth7;
-    const int own_tiles = (T - crank + csize - 1) / csize;               // tiles crank, crank + csize, ... of the cluster
+    const int own_tiles = (T - crank + csize - 1) >> a.lg_csize;               // tiles crank, crank + csize, ... of the cluster
 
     if (a.early) asm volatile("griddepcontrol.launch_dependents;");
     if (lane == 0 && warp % TEAM == 0) {
@@ -355,8 +352,9 @@ gemm7_kernel(const Args7 a, const int own_cap, const int rounds_cap) {
     bool failed = a.inject != 0;
     int cslot = 0;
     uint32_t phase = 0;
-    for (int ch = 0; ch < chunks; ++ch) {
-        const int s0 = sb_lo + ch * a.chunk, s1 = min(sb_hi, s0 + a.chunk), ns = max(0, s1 - s0);
+    for (int s0 = sb_lo, ch = 0;; s0 += a.chunk, ++ch) {
+        const int s1 = min(sb_hi, s0 + a.chunk), ns = max(0, s1 - s0);
+        const bool last = s0 + a.chunk >= sb_hi;
         if (ch > 0) {
             __syncthreads();                             // everybody is done with the activations of the chunk before
             start_chunk(s0, s1);
@@ -368,15 +366,17 @@ gemm7_kernel(const Args7 a, const int own_cap, const int rounds_cap) {
             // the activations: a warp takes eight batch rows of one group, a lane two runs of 16 columns of one row.  CTAs
             // start at different places: all of them read the same lines.
             // (int8: two column tiles of four rows at a time; the last one may be half a pair)
+            // (one column tile: two groups at a time instead)
             constexpr int NP = INT8 ? (NT + 1) / 2 : NT;
-            const int tasks = ns * 4 * NP, rot = tasks ? (cl * 5) % tasks : 0;
+            constexpr bool kPairs = INT8 && NT == 1;
+            const int tasks = kPairs ? 2 * ns : ns * 4 * NP, rot = tasks ? (cl * 5) % tasks : 0;
             constexpr int U = 4;                         // tasks whose loads are in flight
             for (int w0 = warp; w0 < tasks; w0 += U * warps) {
                 uint4 r[U][2][2];
 #pragma unroll
                 for (int q = 0; q < U; ++q) {
                     const int wr = w0 + q * warps + rot, w = wr < tasks ? wr : wr - tasks;
-                    const int mi = 8 * (w % NP) + g, col = kSuper3 * s0 + 128 * (w / NP) + 16 * t;
+                    const int mi = kPairs ? g & 3 : 8 * (w % NP) + g, col = kSuper3 * s0 + 128 * (kPairs ? 2 * w + (g >> 2) : w / NP) + 16 * t;
 #pragma unroll
                     for (int i = 0; i < 2; ++i) {
                         r[q][i][0] = r[q][i][1] = make_uint4(0u, 0u, 0u, 0u);
@@ -392,7 +392,7 @@ gemm7_kernel(const Args7 a, const int own_cap, const int rounds_cap) {
                     if (w0 + q * warps >= tasks) break;
                     const int wr = w0 + q * warps + rot, w = wr < tasks ? wr : wr - tasks;
                     if constexpr (INT8) {
-                        convert7<FMT, NT>(r[q], w / NP, w % NP, g, t, smem + so.x, records);
+                        convert7<FMT, NT>(r[q], kPairs ? 2 * w + (g >> 2) : w / NP, kPairs ? 0 : 2 * (w % NP) + (g >> 2), g & 3, t, smem + so.x, records);
                         continue;
                     }
                     float sum = 0.f;
@@ -521,7 +521,7 @@ gemm7_kernel(const Args7 a, const int own_cap, const int rounds_cap) {
                 issue();
                 if (++cslot == kDepth7) { cslot = 0; phase ^= 1u; }
             }
-            if (ch + 1 < chunks) {
+            if (!last) {
 #pragma unroll
                 for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
@@ -530,9 +530,9 @@ gemm7_kernel(const Args7 a, const int own_cap, const int rounds_cap) {
             }
             // push the partial sums to the rank that owns the tile
             if (!met) { cluster_wait(); met = true; }
-            const int owner = j % csize, src = crank * kw + kl;
+            const int owner = j & (csize - 1), src = crank * kw + kl;
             // first of this lane's sums, in floats
-            const int slot = (((j / csize) * sources + src) * 16 + 2 * g) * RS + (INT8 ? t : 2 * t);
+            const int slot = (((j >> a.lg_csize) * sources + src) * 16 + 2 * g) * RS + (INT8 ? t : 2 * t);
             if (failed) {
 #pragma unroll
                 for (int nt = 0; nt < NT; ++nt)
@@ -565,6 +565,7 @@ gemm7_kernel(const Args7 a, const int own_cap, const int rounds_cap) {
                 }
             }
         }
+        if (last) break;
     }
     if (!met) cluster_wait();
     // all partial sums of this rank's tiles: added in the order of the superblock shares, one rounding
@@ -573,9 +574,11 @@ gemm7_kernel(const Args7 a, const int own_cap, const int rounds_cap) {
     else arrived = wait_bounded<true>(r_full, 0u, a.spin_limit);
     if (!arrived) failed = true;
     const float* mine = reinterpret_cast<const float*>(smem + so.red);
-    for (int idx = threadIdx.x; idx < own_tiles * 16 * a.m; idx += blockDim.x) {
-        const int r = idx & 15, mi = (idx >> 4) % a.m, jj = (idx >> 4) / a.m;
-        const int row = 16 * (t_lo + crank + jj * csize) + r;
+    // a half warp per (tile, batch row), lanes = rows
+    for (int jj = 0, mi = 2 * warp + (lane >> 4);; mi += 2 * warps) {
+        while (mi >= a.m) { mi -= a.m; ++jj; }
+        if (jj >= own_tiles) break;
+        const int r = lane & 15, row = 16 * (t_lo + crank + jj * csize) + r;
         const float* p = mine + (size_t)(jj * sources * 16 + r) * RS + mi;
         float s = 0.f;
         for (int q = 0; q < sources; ++q) s += p[q * 16 * RS];
@@ -588,6 +591,7 @@ gemm7_kernel(const Args7 a, const int own_cap, const int rounds_cap) {
     }
     // a rank that gave up on partial sums must not leave before the others have stopped sending
     if (csize > 1) {
+        __syncwarp();
         cluster_arrive();
         cluster_wait();
     }
@@ -624,7 +628,7 @@ int max_clusters(int csize) {
 
 // The launch shape of a matrix (rows in tiles of 16, superblocks): clusters, CTAs per cluster, warps that split K.
 struct Plan7 {
-    int csize, clusters, kw, per_cluster, share;
+    int csize, clusters, kw, per_cluster, share, blocks;
 };
 template <int FMT, bool INT8>
 Plan7 plan7(int tiles, int sbs) {
@@ -638,6 +642,7 @@ Plan7 plan7(int tiles, int sbs) {
         p.csize = c;
         p.clusters = min(max_clusters<FMT, INT8, 1>(c), tiles);
         p.per_cluster = (tiles + p.clusters - 1) / p.clusters;
+        p.blocks = blocks;
         p.share = S * ((blocks + c - 1) / c);
         p.kw = FMT == 3 ? 1 : 4;                         // format 2: the warps of a team
         double units = 0.0;
@@ -692,15 +697,15 @@ Fit7 fit7(const Plan7& p, int m) {
 }
 
 template <int FMT, bool INT8, int NT>
-ptqtp_status launch_nt7(Args7 a, const Plan7& p, const Fit7& f, size_t smem, int own_cap, cudaStream_t st) {
+ptqtp_status launch_nt7(Args7 a, const Plan7& p, const Fit7& f, int clusters, cudaStream_t st) {
     ptqtp_status s = configure_once<gemm7_kernel<FMT, INT8, NT>>();
     if (s != PTQTP_OK) return s;
     a.chunk = f.chunk;
     a.early = overlap_enabled() && !consume_pack(st) ? 1 : 0;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(a.clusters * p.csize);
+    cfg.gridDim = dim3(clusters * p.csize);
     cfg.blockDim = dim3(f.warps * 32);
-    cfg.dynamicSmemBytes = smem;
+    cfg.dynamicSmemBytes = a.at.total;
     cfg.stream = st;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -710,7 +715,7 @@ ptqtp_status launch_nt7(Args7 a, const Plan7& p, const Fit7& f, size_t smem, int
     attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, gemm7_kernel<FMT, INT8, NT>, a, own_cap, f.rounds);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, gemm7_kernel<FMT, INT8, NT>, a);
     if (e != cudaSuccess) { set_last_cuda_error(e); (void)cudaGetLastError(); return PTQTP_ERR_CUDA; }
     return PTQTP_OK;
 }
@@ -721,8 +726,11 @@ ptqtp_status run7(Args7 a, int m, const uint16_t* X, uint16_t* Y, cudaStream_t s
     if (gemv_status_word(&status_word) != PTQTP_OK) return PTQTP_ERR_CUDA;
     constexpr int ROWS = INT8 ? 4 : 8;
     const Plan7 p = plan7<FMT, INT8>(a.all_tiles, a.sbs);
-    a.csize = p.csize;
-    a.kw = p.kw;
+    auto lg = [](int v) { return v == 1 ? 0 : v == 2 ? 1 : v == 4 ? 2 : 3; };
+    a.lg_csize = lg(p.csize);
+    a.lg_kw = lg(p.kw);
+    a.s_base = p.blocks / p.csize;
+    a.s_rem = p.blocks % p.csize;
     a.spin_limit = wait_poll_limit();
     a.status_word = status_word;
     const Fit7 f = fit7<FMT, INT8>(p, m);
@@ -731,19 +739,20 @@ ptqtp_status run7(Args7 a, int m, const uint16_t* X, uint16_t* Y, cudaStream_t s
     const int launches = (m + ROWS * f.nt - 1) / (ROWS * f.nt);
     for (int tile0 = 0; tile0 < a.all_tiles; tile0 += tiles_per_launch) {
         a.tile0 = tile0;
-        a.tiles = min(tiles_per_launch, a.all_tiles - tile0);
-        a.clusters = min(p.clusters, a.tiles);
+        const int tiles = min(tiles_per_launch, a.all_tiles - tile0), clusters = min(p.clusters, tiles);
+        a.t_base = tiles / clusters;
+        a.t_rem = tiles % clusters;
         for (int i = 0, done = 0; i < launches; ++i) {
             const int rows = (m - done + launches - i - 1) / (launches - i), ntl = (rows + ROWS - 1) / ROWS;
             a.X = reinterpret_cast<const __half*>(X) + (size_t)done * a.k;
             a.Y = reinterpret_cast<__half*>(Y) + (size_t)done * a.n;
             a.m = rows;
             a.inject = take_injected_wait_failure() ? 1 : 0;
-            const size_t smem = total7<FMT, INT8>(p, ntl, f.warps, f.chunk, f.per_cluster, f.rounds);
-            const ptqtp_status s = ntl == 1 ? launch_nt7<FMT, INT8, 1>(a, p, f, smem, own_cap, st)
-                                 : ntl == 2 ? launch_nt7<FMT, INT8, 2>(a, p, f, smem, own_cap, st)
-                                 : ntl == 3 ? launch_nt7<FMT, INT8, 3>(a, p, f, smem, own_cap, st)
-                                            : launch_nt7<FMT, INT8, 4>(a, p, f, smem, own_cap, st);
+            a.at = smem7(FMT, ROWS * ntl, f.warps, f.chunk, own_cap, p.csize * p.kw, f.rounds * f.warps);
+            const ptqtp_status s = ntl == 1 ? launch_nt7<FMT, INT8, 1>(a, p, f, clusters, st)
+                                 : ntl == 2 ? launch_nt7<FMT, INT8, 2>(a, p, f, clusters, st)
+                                 : ntl == 3 ? launch_nt7<FMT, INT8, 3>(a, p, f, clusters, st)
+                                            : launch_nt7<FMT, INT8, 4>(a, p, f, clusters, st);
             if (s != PTQTP_OK) return s;
             done += rows;
         }
