@@ -284,7 +284,7 @@ PTQTP_API ptqtp_status ptqtp_decompose(const float *W, int32_t n, int32_t k, int
  * ideally pinned) to x_dev, runs ptqtp_gemv and delivers y in y_host [N]; everything is enqueued on
  * `stream`, no synchronisation: y_host is valid once the stream has reached this point.  x_dev [K] and
  * y_dev [N] are caller-owned device staging buffers.  When y_host is pinned, 16-byte aligned memory that the
- * device can address (format 2), the kernel stores y there directly and y_dev is left untouched; otherwise
+ * device can address (formats 2 and 3), the kernel stores y there directly and y_dev is left untouched; otherwise
  * y is computed into y_dev and copied to y_host. */
 PTQTP_API ptqtp_status ptqtp_gemv_host(const ptqtp_shape *shape /* host */, const void *packed, size_t packed_bytes,
                              const uint16_t *x_host, uint16_t *y_host, uint16_t *x_dev, uint16_t *y_dev,
@@ -346,15 +346,15 @@ PTQTP_API int ptqtp_set_wait_limit(int polls);
 PTQTP_API void ptqtp_test_fail_next_wait(int launches);
 
 /* Overlap of consecutive GEMV calls on one stream (process-wide level, default 0; returns the old level).
- * Level 0 (default): plain launches; every buffer, `packed` included, follows stream order.  Levels 1 and 2 are
- * an opt-in for callers whose packed blobs are immutable while GEMV calls are in flight (the decode case).
- * Level 1: the GEMV kernels of formats 2 and 3 are launched with programmatic stream
- * serialization: a call may begin reading its `packed` blob while the kernel directly before it on the
+ * Level 0 (default): every buffer, `packed` included, follows stream order as with plain launches: a kernel sets itself
+ * up while the one before it drains, but touches nothing before that one is complete.  Levels 1 and 2 are an opt-in
+ * for callers whose packed blobs are immutable while GEMV calls are in flight (the decode case).
+ * Level 1: a call may begin reading its `packed` blob while the kernel directly before it on the
  * stream is still draining; x is used and y written only after all earlier work on the stream has completed,
  * so stream order holds for them.  Consequence for the caller: the packed blob of a call must be complete
  * before the kernel directly ahead of the call on its stream ends -- it must not be the output buffer of that
- * kernel.  ptqtp_pack is exempt (the first GEMV call after a ptqtp_pack on the same stream is a plain launch),
- * and so are copies (cudaMemcpyAsync and the like are not kernels).  Works inside CUDA graph capture.
+ * kernel.  ptqtp_pack is exempt (the first GEMV call after a ptqtp_pack on the same stream reads nothing before the
+ * pack is complete), and so are copies (cudaMemcpyAsync and the like are not kernels).  Works inside CUDA graph capture.
  * Level 2 adds speculative execution: the kernel reads x at once and computes everything into shared memory
  * while earlier work of the stream may still be running, then waits for that work, reads x again and compares
  * it bit by bit with its first read; y is written only after that, and if a single bit of x differed the whole
