@@ -386,8 +386,8 @@ def ptqtp_test_fail_next_wait(launches):
 
 
 def ptqtp_set_overlap(level):
-    """Overlap level of consecutive GEMV calls: 0 (default) plain launches, 1 programmatic dependent launch, 2 also
-    the speculative read of x.  True/False mean 2/0.  Returns the old level."""
+    """Overlap level of consecutive GEMV calls: 0 (default) stream order for every buffer, 1 the packed blob may be
+    read early, 2 also the speculative read of x.  True/False mean 2/0.  Returns the old level."""
     if level is True:
         level = 2
     return int(lib().ptqtp_set_overlap(int(level)))
