@@ -543,8 +543,9 @@ ptqtp_status launch_gemv4_jobs(Jobs4& J, const uint16_t* x, int warps, int ctas_
         rb_cap += J.rb_base[j] + (J.rb_rem[j] ? 1 : 0);
     }
     const int rows_cap = 16 * rb_cap;
+    const bool auto_warps = warps <= 0;
     const bool alone = warps == -1 || (warps == 0 && !speculation_enabled());   // nothing to gain from sharing an SM with the next launch
-    if (warps <= 0) {
+    if (auto_warps) {
         if (alone) {
             // one CTA has the SM to itself: as many warps as have tiles to stream
             warps = S >= max_warps ? max_warps : S * min(max_warps / S, max(1, rb_cap));
@@ -562,8 +563,13 @@ ptqtp_status launch_gemv4_jobs(Jobs4& J, const uint16_t* x, int warps, int ctas_
     if (auto_depth)
         while (depth > 2 && smem_layout4(J.k, S, rows_cap, warps, depth, units).total > budget) --depth;
     if (depth == 5) depth = 4;
+    // Long rows and many of them (x, partial sums) leave less room for the rings: an automatic choice takes as many warps as
+    // fit, so that whether a matrix is accepted does not depend on the overlap level (16 warps fit up to K = 35200 with one
+    // row block per CTA; 8192 x 32768 and 16384 x 53248 take eight).
+    if (auto_warps)
+        while (warps > 1 && smem_layout4(J.k, S, rows_cap, warps, depth, units).total > budget) warps = warps > 4 ? warps / 2 : warps - 1;
     const size_t smem = smem_layout4(J.k, S, rows_cap, warps, depth, units).total;
-    if (smem > budget) return !auto_depth || !auto_units || ctas_per_sm > 1 || warps > 1 ? PTQTP_ERR_CONFIG : PTQTP_ERR_SHAPE;
+    if (smem > budget) return !auto_depth || !auto_units || ctas_per_sm > 1 || warps > 1 || auto_warps ? PTQTP_ERR_CONFIG : PTQTP_ERR_SHAPE;
 #define PTQTP_LAUNCH_D4(DD)                                                                        \
     case DD:                                                                                       \
         if (J.count > 1)                                                                                  \

@@ -302,6 +302,23 @@ def test_gated_pair_of_two_matrices_in_one_launch(N, K):
     assert np.array_equal(yi.cpu().numpy().astype(np.float64), y)
 
 
+@pytest.mark.parametrize("level", [0, 1, 2])
+@pytest.mark.parametrize("N,K", [(37, 36864), (700, 53248), (37, 81920), (18, 98304)])
+def test_long_rows_are_accepted_at_every_overlap_level(N, K, level):
+    # x alone takes 2 K bytes of shared memory: the rings of 16 warps fit beside it up to K = 35200, of eight, four and two at the
+    # sizes here
+    binding.ptqtp_set_overlap(level)
+    c, c2 = make_case(N, K, seed=800 + N), make_case(N, K, seed=801 + N)
+    x = c["x"]
+    p, p2 = pack_case(c, V3), pack_case(c2, V3)
+    y = binding.ptqtp_gemv(p, N, K, dev(x), fmt=V3)
+    ya, yb = binding.ptqtp_gemv_multi([p, p2], [N, N], K, dev(x))
+    torch.cuda.synchronize()
+    assert_parity(y.cpu().numpy(), oracle_y(c), x, "N=%d K=%d level %d" % (N, K, level))
+    assert_parity(yb.cpu().numpy(), oracle_y(dict(c2, x=x)), x, "second matrix")
+    assert np.array_equal(ya.cpu().numpy().view(np.uint16), y.cpu().numpy().view(np.uint16))
+
+
 def test_several_matrices_argument_checks():
     K = 1024
     cs = [make_case(64, K, seed=1), make_case(32, K, seed=2)]
