@@ -262,7 +262,7 @@ static bool fp16_activations(const Layout3& L3, int m) {
     return us6 < us5;
 }
 // Kernels, in microseconds per call in a chain of its kind (14336 x 4096, 4096 x 14336, 4096 x 4096, 1024 x 4096):
-//   fp16: the warp-MMA kernel while one launch takes all rows (8 rows: 12.6, 14.0, 6.4, 4.0; 16: 18.4, 20.6, 8.4, 5.7),
+//   fp16: the warp-MMA kernel while one launch takes all rows (8 rows: 14.5, 15.7, 6.5, 4.2; 16: 20.3, 21.9, 8.8, 5.3),
 //   the tcgen05 kernel otherwise and with k_split (30.2, 27.3, 11.0, 8.1; 30.8, 28.0, 11.5, 8.2; at 64 rows 50.5, 43.5,
 //   17.2, 11.9 against 79, 79, 38, 13.5 in launches of 16 and 32 rows).
 //   int8: four rows 8.7, 10.5, 5.2, 3.6 on the warp-MMA kernel, 15.0, 27.4, 5.6, 2.6 on the batch-1 tiles kernel at overlap

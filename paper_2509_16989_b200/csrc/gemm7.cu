@@ -5,31 +5,33 @@
 // and multiplies.  Nothing is handed from warp to warp before the end.  The 16 rows of an MMA are 8 row pairs x 2 fields of
 // their code bytes (row of the pair, plane); lanes read the entries of one group pair, not the entries a batch-1 fragment
 // would take, so that an MMA contracts columns of one scale group only.
-//   * fp16 (m16n8k16, fp32 sums; format 3): a 2-bit code at the bits 2f, 2f + 1 of an fp16 pattern is the subnormal
-//     code * 4^f * 2^-24, exactly, so a mask of the even and one of the odd bytes of a word are operand A: 9 half-rate
-//     instructions per 16 codes.  B is the activations as given, a column of B one batch row.
+//   * fp16 (m16n8k16, fp32 sums; format 3): a mask of the even and one of the odd bytes of a code word and an FMA make
+//     two trits of operand A, for 16 codes 9 half-rate instructions and 8 FMAs.  B is the activations as given, a column of B
+//     one batch row: y += alpha d in fp32.
 //   * int8 (m16n8k32, exact int32 sums; formats 3 and 2): three masks per code word; B the activations in 15-bit block
-//     fixed point per 128 columns (as in gemv5.cu and skinny3.cu), two columns, high and low byte, per batch row.
-//   Codes are trit + 1: the sum of x over the group comes off in the epilogue.  An MMA chain holds both planes of a row, which
-//   meet in the same lane: y += alpha (2^s 4^-f d - sum x) in fp32.
+//     fixed point per 128 columns (as in gemv5.cu and skinny3.cu), two columns, high and low byte, per batch row.  Codes are
+//     trit + 1: the sum of x over the group comes off in the epilogue, y += alpha 2^s (4^-f d - sum x).
+//   An MMA chain holds both planes of a row, which meet in the same lane.
 // B is in shared memory, for all of a CTA's columns at once, in fragment order.
 // Grid: clusters of C CTAs split the superblocks of K, clusters split the rows in tiles of 16; in a CTA kw warps split its
 // superblocks.  The partial sums of a tile go to one rank's shared memory (st.async in a cluster), slot by slot, and are added in
 // a fixed order at the end: no atomics, no workspace, reproducible.  C and kw depend on the shape alone.
 //
 // What bounds it, from microbenchmarks on the issue port of an SM quarter: an MMA costs 8 cycles of the tensor pipe and 4 of
-// issue, a mask 2, another instruction 1.  A tile is 64 MMAs per 8 rows and 288 masks and shifts in fp16: about 320 cycles
-// per SM (measured slope 318) against 187 of HBM; int8 with 4 rows 32 MMAs and 96 masks: about 130.  On top of that 3 us
-// per launch: start, activations, last sums.  14336 x 4096, microseconds per call in a chain: 4 rows 8.7 (one-group
-// fragments of gemv5: 16.5), 8 rows 12.6 and 16 rows 18.4 (tcgen05 kernel: 30.3, 31.3).
+// issue, a mask 2, another instruction 1.  A tile is 64 MMAs per 8 rows, 288 masks and shifts and 256 FMAs in fp16: about 270
+// cycles per SM at 8 rows, 340 at 16, against 187 of HBM; int8 with 4 rows 32 MMAs and 96 masks: about 130.  On top of that 3 us
+// per launch: start, activations, last sums.  14336 x 4096, microseconds per call in a chain at level 0: 4 rows 9.7 (one-group
+// fragments of gemv5: 17.4), 8 rows 14.5 and 16 rows 20.3 (tcgen05 kernel: 31.2, 31.9).
 // Clusters of 4 and 8 leave 16 and 28 SMs idle (33 and 15 fit); larger C only where an activation slice does not fit.
 //
 // The same work on tcgen05 with operand A masked straight into tensor memory (64- and 128-row blocks, one or both planes per
 // lane, 14 to 20 specialised warps) took 23 to 26 us on 14336 x 4096 at 16 rows: a poll of an mbarrier takes 110 cycles
 // there whether its phase is complete or not, and codes -> tensor memory -> MMA -> sums is three of them per group.
 //
-// Precision of the fp16 form: 2.0775e-4 off the product in 64 bits (4096 x 4096, 16 rows, normal x), of which 2.0773e-4 is the
-// rounding of y to fp16 (the tcgen05 kernel: 2.0773e-4).
+// Precision of the fp16 form, the rounding of y taken out (512 x 4096, 16 rows; in brackets the tcgen05 kernel with one CTA per
+// row block, with four): 0.82e-7 of the result on normal x (1.44e-7, 0.94e-7), 0.80e-7 on x of mean 4 (1.44e-7, 0.92e-7),
+// 0.82e-7 with a column of 30 to 30000 in every group whose trits are 0 (1.46e-7, 0.93e-7), 2.10e-7 with a column of 1000 in
+// every group and any trits (2.41e-7, 2.15e-7), 1.99e-7 on x over 24 powers of two (2.31e-7, 2.06e-7).
 //
 // The kernel is always launched as a dependent of the kernel before it on the stream: everything that is visible to
 // other work happens after griddepcontrol.wait, and the next kernel may start only then; before it the first tiles are
@@ -127,17 +129,17 @@ __device__ __forceinline__ void mma_f16_first(float (&c)[4], uint32_t a0, uint32
         : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "f"(0.f));
 }
 
-// Offsets in dynamic shared memory: the warps' rings, the activations of a chunk in fragment order, the negated group sums of
-// x, the partial sums pushed here [own tile][source][16][stride], sums kept between chunks, barriers (one per ring slot,
+// Offsets in dynamic shared memory: the warps' rings, the activations of a chunk in fragment order, their group
+// records (int8), the partial sums pushed here [own tile][source][16][stride], sums kept between chunks, barriers (one per ring slot,
 // one for the partial sums).
 struct Smem7 {
     uint32_t x, sx, red, keep, bars;
     size_t total;
 };
 inline int red_stride7(int npad) { return npad + 2; }      // rows two banks apart
-inline Smem7 smem7(int fmt, int npad, int warps, int chunk, int own_tiles, int sources, int kept_tiles) {
+inline Smem7 smem7(int fmt, bool int8, int npad, int warps, int chunk, int own_tiles, int sources, int kept_tiles) {
     const size_t x = (size_t)(warps / team7(fmt)) * kDepth7 * (fmt == 3 ? kTile3 : kTile2);
-    const size_t sx = x + (size_t)chunk * npad * 1024, red = sx + (size_t)chunk * 4 * npad * 8;
+    const size_t sx = x + (size_t)chunk * npad * 1024, red = sx + (int8 ? (size_t)chunk * 4 * npad * 8 : 0);
     const size_t keep = red + (size_t)own_tiles * sources * 16 * red_stride7(npad) * 4;
     const size_t bars = (keep + (size_t)kept_tiles * 16 * npad * 4 + 15) / 16 * 16;
     const Smem7 s = {(uint32_t)x, (uint32_t)sx, (uint32_t)red, (uint32_t)keep, (uint32_t)bars, bars + (size_t)(warps * kDepth7 + 1) * 8 + 8};
@@ -256,6 +258,19 @@ __device__ __forceinline__ void group_int8(const uint32_t (&word)[8], const unsi
     }
 }
 
+// fp16: the trits of field F (two columns) as multiples of 2^-9.  A code under its mask is the subnormal code * 4^F * 2^-24; one
+// FMA makes it code * 2^-9, less the 1 that a code is more than its trit: exact.  (The masked codes themselves as operand A and
+// the sum of x taken off afterwards saved the FMAs, 14336 x 4096 at 8 and 16 rows 13.0 and 18.8 us against 14.5 and 20.3, but a
+// sum then has x where the trit is 0, and the MMA cuts products with a subnormal factor off where it would if that factor
+// were 2^-14: 2.6e-6 of the result on normal x, 0.1 of it next to columns of 30000.)
+template <int F>
+__device__ __forceinline__ uint32_t trits(uint32_t bytes) {
+    const uint32_t code = bytes & (0x00030003u << (2 * F));
+    const __half2 up = __half2half2(__ushort_as_half((unsigned short)((30 - 2 * F) << 10))), one = __half2half2(__ushort_as_half(0x9800u));
+    const __half2 d = __hfma2(*reinterpret_cast<const __half2*>(&code), up, one);        // 2^(15 - 2 F), -2^-9
+    return *reinterpret_cast<const uint32_t*>(&d);
+}
+
 // One launch.  The shares are divided on the host (a dozen integer divisions per warp were half a microsecond of a launch): tile0
 // and the tiles (8 row pairs) of a cluster, the superblocks of a rank, C = 1 << lg_csize, kw = 1 << lg_kw; all_tiles: of
 // the matrix; chunk: superblocks of activations held at a time.
@@ -291,7 +306,6 @@ gemm7_kernel(const __grid_constant__ Args7 a) {
     const Smem7& so = a.at;
     const uint32_t ring = smem_u32(smem) + (uint32_t)(warp / TEAM * kDepth7 * kTileBytes), xs = smem_u32(smem + so.x), red = smem_u32(smem + so.red);
     unsigned char* ring_p = smem + (size_t)(warp / TEAM) * kDepth7 * kTileBytes;
-    float* sx = reinterpret_cast<float*>(smem + so.sx);                   // fp16: minus the sum of x
     int2* records = reinterpret_cast<int2*>(smem + so.sx);                // int8: (2^-s, sum of the integers)
     const uint32_t bars = smem_u32(smem + so.bars) + 8 * (warp / TEAM) * kDepth7, r_full = smem_u32(smem + so.bars) + 8 * warps * kDepth7;
     const int own_tiles = (T - crank + csize - 1) >> a.lg_csize;               // tiles crank, crank + csize, ... of the cluster
@@ -395,16 +409,10 @@ gemm7_kernel(const __grid_constant__ Args7 a) {
                         convert7<FMT, NT>(r[q], kPairs ? 2 * w + (g >> 2) : w / NP, kPairs ? 0 : 2 * (w % NP) + (g >> 2), g & 3, t, smem + so.x, records);
                         continue;
                     }
-                    float sum = 0.f;
 #pragma unroll
                     for (int i = 0; i < 2; ++i) {
                         const uint4 lo = r[q][i][0], hi = r[q][i][1];
                         const uint32_t v[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
-#pragma unroll
-                        for (int e = 0; e < 8; ++e) {
-                            const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&v[e]));
-                            sum += f.x + f.y;
-                        }
                         // four columns (p, q) of a k-step: even ones, then odd ones
                         uint32_t ev[4], od[4];
 #pragma unroll
@@ -422,9 +430,6 @@ gemm7_kernel(const __grid_constant__ Args7 a) {
                             asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(d1), "r"(ev[1]), "r"(od[1]), "r"(ev[3]), "r"(od[3]) : "memory");
                         }
                     }
-                    sum += __shfl_xor_sync(0xffffffffu, sum, 1);
-                    sum += __shfl_xor_sync(0xffffffffu, sum, 2);
-                    if (t == 0) sx[(w / NP) * NPAD + 8 * (w % NP) + g] = -sum;
                 }
             }
         }
@@ -443,7 +448,6 @@ gemm7_kernel(const __grid_constant__ Args7 a) {
                 if (!wait_bounded<false>(bars + 8 * cslot, phase, failed ? 256 : a.spin_limit)) failed = true;
                 const unsigned char* tile = ring_p + cslot * kTileBytes;
                 const unsigned char* xb = smem + so.x + (size_t)(sb - s0) * (NPAD * 1024) + lane * 16;
-                const float* sxb = sx + (sb - s0) * 4 * NPAD + 2 * t;
                 auto group = [&](int G, const uint32_t (&word)[8], const unsigned char* quad) {
                     if constexpr (INT8) {
                         group_int8<NT>(word, xb + G * (NT * 1024), quad, records + ((sb - s0) * 4 + G) * NPAD + t, y);
@@ -457,8 +461,8 @@ gemm7_kernel(const __grid_constant__ Args7 a) {
 #pragma unroll
                         for (int s = 0; s < 2; ++s) {
                             const uint32_t e = word[2 * kk + s], o = e >> 8;
-                            const uint32_t e0 = e & 0x00030003u, e1 = e & 0x000c000cu, e2 = e & 0x00300030u, e3 = e & 0x00c000c0u;
-                            const uint32_t o0 = o & 0x00030003u, o1 = o & 0x000c000cu, o2 = o & 0x00300030u, o3 = o & 0x00c000c0u;
+                            const uint32_t e0 = trits<0>(e), e1 = trits<1>(e), e2 = trits<2>(e), e3 = trits<3>(e);
+                            const uint32_t o0 = trits<0>(o), o1 = trits<1>(o), o2 = trits<2>(o), o3 = trits<3>(o);
 #pragma unroll
                             for (int nt = 0; nt < NT; ++nt) {
                                 if (kk + s == 0) {
@@ -474,13 +478,14 @@ gemm7_kernel(const __grid_constant__ Args7 a) {
                     const uint2 sc = *reinterpret_cast<const uint2*>(quad);
                     const float2 s0v = __half22float2(*reinterpret_cast<const __half2*>(&sc.x));     // row 2 g: alpha1, alpha2
                     const float2 s1v = __half22float2(*reinterpret_cast<const __half2*>(&sc.y));     // row 2 g + 1
+                    // (the scales times 2^9 are exact)
+                    const float k0 = s0v.x * 0x1p9f, k1 = s0v.y * 0x1p9f, k2 = s1v.x * 0x1p9f, k3 = s1v.y * 0x1p9f;
 #pragma unroll
                     for (int nt = 0; nt < NT; ++nt) {
-                        const float2 sv = *reinterpret_cast<const float2*>(sxb + G * NPAD + 8 * nt);
-                        y[nt][0] = fmaf(s0v.y, fmaf(ca[nt][2], 0x1p22f, sv.x), fmaf(s0v.x, fmaf(ca[nt][0], 0x1p24f, sv.x), y[nt][0]));
-                        y[nt][1] = fmaf(s0v.y, fmaf(ca[nt][3], 0x1p22f, sv.y), fmaf(s0v.x, fmaf(ca[nt][1], 0x1p24f, sv.y), y[nt][1]));
-                        y[nt][2] = fmaf(s1v.y, fmaf(cb[nt][2], 0x1p18f, sv.x), fmaf(s1v.x, fmaf(cb[nt][0], 0x1p20f, sv.x), y[nt][2]));
-                        y[nt][3] = fmaf(s1v.y, fmaf(cb[nt][3], 0x1p18f, sv.y), fmaf(s1v.x, fmaf(cb[nt][1], 0x1p20f, sv.y), y[nt][3]));
+                        y[nt][0] = fmaf(k1, ca[nt][2], fmaf(k0, ca[nt][0], y[nt][0]));
+                        y[nt][1] = fmaf(k1, ca[nt][3], fmaf(k0, ca[nt][1], y[nt][1]));
+                        y[nt][2] = fmaf(k3, cb[nt][2], fmaf(k2, cb[nt][0], y[nt][2]));
+                        y[nt][3] = fmaf(k3, cb[nt][3], fmaf(k2, cb[nt][1], y[nt][3]));
                     }
                     }
                 };
@@ -654,7 +659,7 @@ Plan7 plan7(int tiles, int sbs) {
         // tiles of the busiest CTA; a superblock of activations costs about half a tile's time to bring in; a cluster costs
         // the time of a few tiles to start and to meet; two column tiles should fit at once
         double cost = p.per_cluster * (double)p.share + 0.5 * p.share + (c > 1 ? 2.0 : 0.0);
-        if (smem7(FMT, INT8 ? 8 : 16, 8, p.share, (min(p.per_cluster, 32) + c - 1) / c, c * p.kw, 0).total > kSmem7) cost *= 2.0;
+        if (smem7(FMT, INT8, INT8 ? 8 : 16, 8, p.share, (min(p.per_cluster, 32) + c - 1) / c, c * p.kw, 0).total > kSmem7) cost *= 2.0;
         if (best_cost == 0.0 || cost < best_cost) { best_cost = cost; best = p; }
     }
     return best;
@@ -667,7 +672,7 @@ struct Fit7 {
 };
 template <int FMT, bool INT8>
 size_t total7(const Plan7& p, int nt, int warps, int chunk, int tiles, int rounds) {
-    return smem7(FMT, (INT8 ? 4 : 8) * nt, warps, chunk, (tiles + p.csize - 1) / p.csize, p.csize * p.kw, rounds * warps).total;
+    return smem7(FMT, INT8, (INT8 ? 4 : 8) * nt, warps, chunk, (tiles + p.csize - 1) / p.csize, p.csize * p.kw, rounds * warps).total;
 }
 // As many rows of X (up to 32, or 16 for int8) as leave room for all of a rank's activations beside the warps' rings, then as
 // many tiles as leave room for their partial sums: a matrix too tall for one launch takes several, a row too long
@@ -748,7 +753,7 @@ ptqtp_status run7(Args7 a, int m, const uint16_t* X, uint16_t* Y, cudaStream_t s
             a.Y = reinterpret_cast<__half*>(Y) + (size_t)done * a.n;
             a.m = rows;
             a.inject = take_injected_wait_failure() ? 1 : 0;
-            a.at = smem7(FMT, ROWS * ntl, f.warps, f.chunk, own_cap, p.csize * p.kw, f.rounds * f.warps);
+            a.at = smem7(FMT, INT8, ROWS * ntl, f.warps, f.chunk, own_cap, p.csize * p.kw, f.rounds * f.warps);
             const ptqtp_status s = ntl == 1 ? launch_nt7<FMT, INT8, 1>(a, p, f, clusters, st)
                                  : ntl == 2 ? launch_nt7<FMT, INT8, 2>(a, p, f, clusters, st)
                                  : ntl == 3 ? launch_nt7<FMT, INT8, 3>(a, p, f, clusters, st)

@@ -118,6 +118,38 @@ def test_small_and_large_activations():
     assert np.all(np.abs(Y.astype(np.float64) - ref) <= bound)
 
 
+@pytest.mark.parametrize("k_split", [0, 1])
+@pytest.mark.parametrize("N,K,M", [(47, 640, 8), (64, 4096, 5), (330, 10240, 16), (33, 2048, 32)])
+def test_columns_whose_trits_are_zero_add_nothing(N, K, M, k_split):
+    # fp16 operands: one column per scale group holds 20000 and more, with trit 0 in both planes, next to multiples of 2^-10 below
+    # 2^-7.  Every sum without those columns is a multiple of 2^-10 below 2^14, exact in fp32, and every result one below 2,
+    # exact in fp16; 20000 added and taken off again leaves multiples of 2^-8 at best.
+    c = make_case(N, K, seed=19 + M, M=M)
+    rng = np.random.default_rng(9)
+    c["x"] = (rng.integers(-7, 8, (M, K)) * 2.0 ** -10 * (rng.random((M, K)) < 0.2)).astype(np.float16)
+    cols = np.arange(37, K, 128)
+    c["x"][:, cols] = (20000 + 16 * rng.integers(0, 1000, (M, cols.size))).astype(np.float16)
+    c["T1"][:, cols] = c["T2"][:, cols] = 0
+    c["alpha1"] = np.ones_like(c["alpha1"])
+    c["alpha2"] = np.full_like(c["alpha2"], 2.0)
+    exact = c["x"].astype(np.float64) @ (c["T1"].astype(np.float64) + 2 * c["T2"].astype(np.float64)).T
+    assert np.all(np.abs(exact) < 2)
+    Y = binding.ptqtp_gemm_skinny_cfg(pack_for("fp16", c), N, K, dev(c["x"]), path=6, k_split=k_split)
+    assert np.array_equal(Y.cpu().numpy().astype(np.float64), exact)
+
+
+def test_infinite_activations_reach_the_same_rows_on_both_kernels():
+    # an infinity times a trit of 0 is NaN, times other trits an infinity, whichever kernel takes fp16 operands
+    N, K, M = 90, 1024, 6
+    c = make_case(N, K, seed=23, M=M)
+    c["x"][1, 5], c["x"][2, 700], c["x"][4, 1000] = np.inf, -np.inf, np.nan
+    packed = pack_for("fp16", c)
+    want, got = (binding.ptqtp_gemm_skinny_cfg(packed, N, K, dev(c["x"]), path=6, k_split=k).cpu().numpy() for k in (1, 0))
+    assert np.isinf(want[1]).any() and np.isnan(want[1]).any()
+    assert np.array_equal(np.isnan(got), np.isnan(want)) and np.array_equal(got[np.isinf(want)], want[np.isinf(want)])
+    assert np.all(np.isfinite(got[[0, 3, 5]]))
+
+
 @pytest.mark.parametrize("kind", KINDS)
 def test_bounded_wait_gives_up_reports_and_recovers(kind):
     N, K, M = 700, 9216, 12
