@@ -280,6 +280,25 @@ static ptqtp_status skinny_v3(const Layout3& L3, const void* packed, int m, cons
     return s == PTQTP_ERR_SHAPE ? launch_gemm7(L3, packed, m, X, Y, true, st) : s;       // no room for m rows of x
 }
 
+// Small batch on format 2, m >= 2.  A row that passes of up to four (as many as find room) leave alone keeps the batch-1
+// kernel's 16-bit activations per 64 columns; the other rows have 15 bits per 128 columns, on either of two kernels: two rows, and
+// up to four on small matrices, take the register-stationary kernel, whose launches overlap at level 2 (two rows of 4096 x 4096 there:
+// 3.8 us against 6.0); the rest the warp-MMA kernel (four rows of 14336 x 4096, 4096 x 14336, 4096 x 4096: 11.2, 12.4,
+// 6.2 us against 13.7, 18.1, 8.1 at level 0 and 11.7, 16.8, 6.9 at level 2).
+static ptqtp_status skinny_v2(const Layout2& L2, const void* packed, int m, const uint16_t* X, uint16_t* Y, cudaStream_t st) {
+    const int per_pass = gemv3_rows_per_pass(L2, m), alone = per_pass == 1 ? m : m % per_pass == 1 ? 1 : 0;
+    int rows = m - alone;
+    for (int i = rows; i < m; ++i) {
+        const ptqtp_status s = launch_gemv2(L2, packed, X + (size_t)i * L2.k, Y + (size_t)i * L2.n, 0, 0, 0, 0, st);
+        if (s != PTQTP_OK && (i > rows || s == PTQTP_ERR_CUDA)) return s;
+        if (s != PTQTP_OK) { rows = m; break; }          // K too long for it: nothing launched yet
+    }
+    if (rows == 0) return PTQTP_OK;
+    if (rows > 4 || (rows > 1 && L2.k > 8192) || (rows > 2 && L2.total > 2000000)) return launch_gemm7(L2, packed, rows, X, Y, st);
+    const ptqtp_status s = launch_gemv3(L2, packed, rows, X, Y, 0, 0, 0, st);
+    return s == PTQTP_ERR_SHAPE ? launch_gemm7(L2, packed, rows, X, Y, st) : s;
+}
+
 ptqtp_status ptqtp_gemm_skinny(const ptqtp_shape* shape, const void* packed, size_t packed_bytes, int32_t m,
                                const uint16_t* X, uint16_t* Y, void* stream) {
     if (!X || !Y) return PTQTP_ERR_NULL;
@@ -290,16 +309,8 @@ ptqtp_status ptqtp_gemm_skinny(const ptqtp_shape* shape, const void* packed, siz
     if (!aligned16(X) || !aligned16(Y)) return PTQTP_ERR_ALIGN;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     if (L.v2) {
-        // Two rows, and up to four on small matrices, take the register-stationary kernel, whose launches overlap at level
-        // 2 (two rows of 4096 x 4096 there: 3.8 us against 6.0); the rest the warp-MMA kernel (four rows of 14336 x 4096,
-        // 4096 x 14336, 4096 x 4096: 11.2, 12.4, 6.2 us against 13.7, 18.1, 8.1 at level 0 and 11.7, 16.8, 6.9 at level 2).
-        if (m > 4 || (m > 1 && shape->k_in > 8192) || (m > 2 && L.l2.total > 2000000))
-            return launch_gemm7(L.l2, packed, m, X, Y, st);
-        if (m >= 2) {
-            const ptqtp_status sp = launch_gemv3(L.l2, packed, m, X, Y, 0, 0, 0, st);
-            return sp == PTQTP_ERR_SHAPE ? launch_gemm7(L.l2, packed, m, X, Y, st) : sp;
-        }
-        return launch_gemv2(L.l2, packed, X, Y, 0, 0, 0, 0, st);
+        if (m == 1) return launch_gemv2(L.l2, packed, X, Y, 0, 0, 0, 0, st);
+        return skinny_v2(L.l2, packed, m, X, Y, st);
     }
     if (L.v3) return skinny_v3(L.l3, packed, m, X, Y, 0, 0, st);
     // format 1 is a batch-1 layout

@@ -414,7 +414,21 @@ gemv3_kernel(Layout2 L, const unsigned char* __restrict__ packed, const __half* 
     }
 }
 
+// Warps of the library's own choice.
+int auto_warps3(const Layout2& L, int m, int quads_per_cta) {
+    if (m >= 2) return m == 2 && L.slices <= 2 ? 8 : 16;   // converting M rows of x is shared by the CTA's threads
+    return L.slices >= 3 || (long)quads_per_cta * L.slices >= 64 ? 8 : 4;
+}
+
 }  // namespace
+
+int gemv3_rows_per_pass(const Layout2& L, int m) {
+    const int nquads = (L.nrp + 3) / 4, grid = min(sm_count(), nquads), quads = (nquads + grid - 1) / grid;
+    int rows = min(m, kMaxBatch3);
+    while (rows > 1 && smem_layout3(L.k, rows, L.slices, 8 * quads, auto_warps3(L, rows, quads) / kTeamWarps, 2, 0).total > (size_t)227 * 1024)
+        --rows;
+    return rows;
+}
 
 // PTQTP_ERR_SHAPE when the activations of (K, M) leave no room for a two-stage ring in shared memory.
 // warps: 4, 8 or 16 (one, two or four teams; 0 = 4, or 8 for three slices and more or when a CTA streams many units):
@@ -430,10 +444,7 @@ ptqtp_status launch_gemv3(const Layout2& L, const void* packed, int m, const uin
     const int per_sm = ctas_per_sm == 2 ? 2 : 1;
     const int grid = min(per_sm * sm_count(), nquads);
     const int rows_cap = 8 * ((nquads + grid - 1) / grid);
-    if (warps == 0) {
-        warps = L.slices >= 3 || (long)((nquads + grid - 1) / grid) * L.slices >= 64 ? 8 : 4;
-        if (m >= 2) warps = m == 2 && L.slices <= 2 ? 8 : 16;   // converting M rows of x is shared by the CTA's threads
-    }
+    if (warps == 0) warps = auto_warps3(L, m, (nquads + grid - 1) / grid);
     if (warps * per_sm > 16) return PTQTP_ERR_CONFIG;
     const int teams = warps / kTeamWarps;
     const size_t budget = (size_t)(228 / per_sm - 1) * 1024;            // 228 KB per SM, 1 KB of it reserved per CTA

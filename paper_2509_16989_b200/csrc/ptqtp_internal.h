@@ -182,6 +182,8 @@ ptqtp_status gemv_status_word(int** out);      // device address of the word cop
 // 1 <= m <= 4 on the tensor-core path; PTQTP_ERR_SHAPE when (K, m) leaves no room for its ring in shared memory
 ptqtp_status launch_gemv3(const Layout2& L, const void* packed, int m, const uint16_t* X, uint16_t* Y, int warps,
                           int ctas_per_sm, int depth, cudaStream_t st);
+// rows (1 to min(m, 4)) that one such launch of the library's own choice takes; 1: not even two find room
+int gemv3_rows_per_pass(const Layout2& L, int m);
 int sm_count();
 bool speculation_enabled();       // speculative read of x before the dependency wait (ptqtp_set_overlap(2))
 bool overlap_enabled();           // programmatic dependent launch of the GEMV kernels (ptqtp_set_overlap)

@@ -464,6 +464,22 @@ def test_gemm_skinny_ws_two_rounds_per_cta_on_the_70b_shape():
     assert_parity(Y.cpu().numpy()[:, rows], ref, c["x"], "gemm_skinny 70B M=8")
 
 
+@pytest.mark.parametrize("N,K,M,alone", [(64, 1152, 5, 1), (300, 4096, 9, 1), (1000, 2048, 61, 1), (4096, 4096, 5, 1), (37, 36864, 3, 1),
+                                         (20, 65536, 2, 2), (21, 65536, 6, 6)])
+def test_rows_that_passes_of_up_to_four_leave_alone_have_the_batch1_arithmetic(N, K, M, alone):
+    # format 2: the batch-1 kernel holds activations in 16 bits per 64 columns, the batch kernels in 15 bits per 128.  Passes take four
+    # rows, two where K = 36864 leaves room for no more, one where K = 65536 does; a single row is a batch-1 call
+    c = make_case(N, K, seed=400 + N + M, M=M)
+    packed = pack_case(c, binding.FORMAT_V2)
+    X = dev(c["x"])
+    Y = binding.ptqtp_gemm_skinny(packed, N, K, X, fmt=binding.FORMAT_V2)
+    single = [binding.ptqtp_gemv(packed, N, K, X[i].clone(), fmt=binding.FORMAT_V2) for i in range(M - alone, M)]
+    torch.cuda.synchronize()
+    for i, y in zip(range(M - alone, M), single):
+        assert np.array_equal(Y[i].cpu().numpy().view(np.uint16), y.cpu().numpy().view(np.uint16)), i
+    assert_parity(Y.cpu().numpy(), oracle_y(c), c["x"], "N=%d K=%d M=%d" % (N, K, M))
+
+
 @pytest.mark.parametrize("fmt", FORMATS)
 def test_gemv_host_entry_point(fmt):
     c = make_case(300, 2048, seed=9)
