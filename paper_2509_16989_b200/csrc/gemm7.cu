@@ -35,7 +35,7 @@
 //
 // The kernel is always launched as a dependent of the kernel before it on the stream: everything that is visible to
 // other work happens after griddepcontrol.wait, and the next kernel may start only then; before it the first tiles are
-// prefetched into L2.  At overlap levels 1 and 2 they are read, and the next kernel may start at once.  Waits on mbarriers
+// prefetched into L2.  At overlap levels 1 and 2 (where it pays, see launch_nt7) they are read, and the next kernel may start at once.  Waits on mbarriers
 // are bounded: a warp that gives up marks the launch failed (status word) and its rows come out as NaN.
 #include <cuda_fp16.h>
 #include "ptqtp_internal.h"
@@ -706,7 +706,12 @@ ptqtp_status launch_nt7(Args7 a, const Plan7& p, const Fit7& f, int clusters, cu
     ptqtp_status s = configure_once<gemm7_kernel<FMT, INT8, NT>>();
     if (s != PTQTP_OK) return s;
     a.chunk = f.chunk;
-    a.early = overlap_enabled() && !consume_pack(st) ? 1 : 0;
+    // Overlap levels 1 and 2: worth it when the launch fills the device, or leaves room for a whole one beside it.  In between the first
+    // CTAs of the next launch take the idle SMs and wait there while the rest queue for the others: 128 CTAs at level 2, 2048 x 4096
+    // at 3 rows of format 2 6.0 us against 5.1 in stream order, 2048 x 2048 at 8 rows of format 3 5.2 against 4.2; 32 CTAs (512 x
+    // 1024, 2 rows) 3.0 against 3.4, all SMs (14336 x 4096, 4 rows) 9.2 against 9.6.
+    const bool overlap = clusters == max_clusters<FMT, INT8, NT>(p.csize) || 2 * clusters * p.csize <= sm_count();
+    a.early = overlap_enabled() && overlap && !consume_pack(st) ? 1 : 0;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(clusters * p.csize);
     cfg.blockDim = dim3(f.warps * 32);
