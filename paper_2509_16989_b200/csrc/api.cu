@@ -294,7 +294,7 @@ static ptqtp_status skinny_v2(const Layout2& L2, const void* packed, int m, cons
         if (s != PTQTP_OK) { rows = m; break; }          // K too long for it: nothing launched yet
     }
     if (rows == 0) return PTQTP_OK;
-    if (rows > 4 || (rows > 1 && L2.k > 8192) || (rows > 2 && L2.total > 2000000)) return launch_gemm7(L2, packed, rows, X, Y, st);
+    if (rows > 4 || (L2.k > 8192 && (rows > 2 || !gemm7_uneven(L2))) || (rows > 2 && L2.total > 2000000)) return launch_gemm7(L2, packed, rows, X, Y, st);
     const ptqtp_status s = launch_gemv3(L2, packed, rows, X, Y, 0, 0, 0, st);
     return s == PTQTP_ERR_SHAPE ? launch_gemm7(L2, packed, rows, X, Y, st) : s;
 }
@@ -346,7 +346,7 @@ ptqtp_status ptqtp_gemm_skinny_ws(const ptqtp_shape* shape, const void* packed, 
     if (!L.v2) return PTQTP_ERR_CONFIG;
     if (!aligned16(X) || !aligned16(Y) || !aligned16(workspace)) return PTQTP_ERR_ALIGN;
     if (workspace_bytes < skinny3_workspace_bytes(shape->k_in, m)) return PTQTP_ERR_SIZE;
-    if (gemm7_one_launch(L.l2, m)) return launch_gemm7(L.l2, packed, m, X, Y, static_cast<cudaStream_t>(stream));
+    if (gemm7_one_launch(L.l2, m) && !gemm7_uneven(L.l2)) return launch_gemm7(L.l2, packed, m, X, Y, static_cast<cudaStream_t>(stream));
     return launch_skinny3(L.l2, packed, m, X, Y, workspace, static_cast<cudaStream_t>(stream));
 }
 
@@ -360,7 +360,7 @@ ptqtp_status ptqtp_gemm_skinny_static(const ptqtp_shape* shape, const void* pack
     if (!L.v2) return PTQTP_ERR_CONFIG;
     if (!aligned16(X) || !aligned16(Y)) return PTQTP_ERR_ALIGN;
     if (skinny3_workspace_bytes(shape->k_in, m) > (size_t)PTQTP_STATIC_WORKSPACE_BYTES) return PTQTP_ERR_SIZE;
-    if (gemm7_one_launch(L.l2, m)) return launch_gemm7(L.l2, packed, m, X, Y, static_cast<cudaStream_t>(stream));
+    if (gemm7_one_launch(L.l2, m) && !gemm7_uneven(L.l2)) return launch_gemm7(L.l2, packed, m, X, Y, static_cast<cudaStream_t>(stream));
     void* workspace = nullptr;
     s = static_workspace_address(&workspace);
     if (s != PTQTP_OK) return s;

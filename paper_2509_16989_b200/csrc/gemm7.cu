@@ -782,6 +782,14 @@ bool gemm7_one_launch(const Layout3& L, int m, bool int8) { return one_launch7(3
 bool gemm7_one_launch(const Layout2& L, int m) {
     return one_launch7(2, true, (L.nrp + kTileRp3 - 1) / kTileRp3, (L.k + kSuper3 - 1) / kSuper3, m);
 }
+// Clusters of eight CTAs (15 of them find room: 28 SMs idle) whose ranks have unequal shares of the slices: the other kernels on format
+// 2 are faster there (14 slices: 8192 x 28672 at 2 rows 46 us against 40 on the register-stationary kernel, at 8 rows 67 against
+// 62 on the workspace kernel; 16384 x 28672 85 against 78 and 129 against 103; 16 slices: 8192 x 32768 46 against 51, 65
+// against 68).
+bool gemm7_uneven(const Layout2& L) {
+    const Plan7 p = plan7<2, true>((L.nrp + kTileRp3 - 1) / kTileRp3, (L.k + kSuper3 - 1) / kSuper3);
+    return p.csize == 8 && p.blocks % 8 != 0;
+}
 
 // 1 <= m <= 64 rows of X (16-byte aligned).
 ptqtp_status launch_gemm7(const Layout3& L, const void* packed, int m, const uint16_t* X, uint16_t* Y, bool int8, cudaStream_t st) {

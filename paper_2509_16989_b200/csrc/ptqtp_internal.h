@@ -168,6 +168,7 @@ ptqtp_status launch_gemm7(const Layout3& L, const void* packed, int m, const uin
 ptqtp_status launch_gemm7(const Layout2& L, const void* packed, int m, const uint16_t* X, uint16_t* Y, cudaStream_t st);
 bool gemm7_one_launch(const Layout3& L, int m, bool int8);
 bool gemm7_one_launch(const Layout2& L, int m);
+bool gemm7_uneven(const Layout2& L);          // its clusters of eight CTAs have unequal shares of K
 size_t decompose_workspace_bytes(long long rows, int t_max);
 void decompose_offsets(long long rows, int t_max, size_t* delta_off, size_t* err_off, size_t* a1_off, size_t* a2_off,
                        size_t* lam_off);

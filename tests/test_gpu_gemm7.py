@@ -90,6 +90,24 @@ def test_matrix_taller_than_a_launch(kind):
     assert_parity(Y, (X.double() @ W.T).cpu().numpy(), X.cpu().numpy(), kind)
 
 
+@pytest.mark.parametrize("N,K,M,writes", [(8192, 28672, 8, True), (8192, 32768, 8, False), (4096, 28672, 8, False), (8192, 28672, 3, True)])
+def test_workspace_call_leaves_uneven_clusters_to_the_workspace_kernel(N, K, M, writes):
+    # 14 slices over clusters of eight: the kernel that converts X into the workspace is faster; 16 slices, or clusters of four: not
+    g = torch.Generator(device="cuda")
+    g.manual_seed(6)
+    trits = lambda: torch.randint(-1, 2, (N, K), generator=g, device="cuda", dtype=torch.int8)  # noqa: E731
+    scale = lambda: (torch.randn((N, K // 128), generator=g, device="cuda") * 0.02).abs().half()  # noqa: E731
+    T1, T2, a1, a2 = trits(), trits(), scale(), scale()
+    X = torch.randn((M, K), generator=g, device="cuda").half()
+    packed, _ = binding.ptqtp_pack(T1, T2, a1, a2, fmt=V2)
+    ws = torch.full((binding.gemm_skinny_workspace_size(N, K, M, fmt=V2),), 0xA5, dtype=torch.uint8, device="cuda")
+    Y = binding.ptqtp_gemm_skinny_ws(packed, N, K, X, workspace=ws, fmt=V2)
+    assert bool((ws != 0xA5).any()) == writes
+    rows = torch.cat([torch.arange(64, device="cuda"), torch.arange(N - 64, N, device="cuda")])
+    W = a1[rows].double().repeat_interleave(128, 1) * T1[rows].double() + a2[rows].double().repeat_interleave(128, 1) * T2[rows].double()
+    assert_parity(Y[:, rows].cpu().numpy(), (X.double() @ W.T).cpu().numpy(), X.cpu().numpy(), "%d x %d" % (N, K))
+
+
 @pytest.mark.parametrize("kind", KINDS)
 def test_exact_on_integers(kind):
     N, K, M = 200, 10240, 7
