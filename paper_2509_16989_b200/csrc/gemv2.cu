@@ -458,7 +458,7 @@ ptqtp_status copy_gemv2_status(int32_t* status_host, cudaStream_t st) {
     return PTQTP_OK;
 }
 
-// gated: y[i] = silu(row 2i) * row 2i+1 instead of the rows themselves (N even).
+// gated: y[i] = silu(row 2i) * row 2i+1 instead of the rows themselves (N even).  in_order: as at overlap level 0.
 // warps: per CTA, 0 = the default below, -1 = as many as fit (for a call that is known to run alone).
 // ctas_per_sm: CTAs of this launch per SM (0 = one).  units: slice units per bulk copy (1, 2 or 4; 0 = 2).
 // The defaults keep a CTA small (4 to 8 warps, two ring slots of two units per warp) so that the CTAs of several
@@ -466,9 +466,9 @@ ptqtp_status copy_gemv2_status(int32_t* status_host, cudaStream_t st) {
 // execution the head of one launch (fetching x) and the tail of another (verifying x, reducing) then overlap the
 // streaming of a third.  Measured on the LLaMA-3-8B shapes, 4 warps beat 8 and 16.
 ptqtp_status launch_gemv2(const Layout2& L, const void* packed, const uint16_t* x, uint16_t* y, int warps,
-                          int ctas_per_sm, int depth, int units, cudaStream_t st, bool gated) {
+                          int ctas_per_sm, int depth, int units, cudaStream_t st, bool gated, bool in_order) {
     const int S = L.slices;
-    const int speculate = speculation_enabled() ? 1 : 0;
+    const int speculate = speculation_enabled() && !in_order ? 1 : 0;
     if (ctas_per_sm < 0 || ctas_per_sm > 4) return PTQTP_ERR_CONFIG;
     if (warps < -1 || warps > kMaxWarps2) return PTQTP_ERR_CONFIG;
     if (units != 0 && units != 1 && units != 2 && units != 4) return PTQTP_ERR_CONFIG;
@@ -476,7 +476,7 @@ ptqtp_status launch_gemv2(const Layout2& L, const void* packed, const uint16_t* 
     const int max_warps = kMaxWarps2 / per_sm;
     const size_t budget = (size_t)(228 / per_sm - 1) * 1024;          // 228 KB per SM, 1 KB of it reserved per CTA
     const int grid = min(per_sm * sm_count(), L.nrp);
-    if (warps == 0 && !overlap_enabled()) warps = -1;   // plain launches never share an SM
+    if (warps == 0 && (!overlap_enabled() || in_order)) warps = -1;   // nothing to gain from sharing an SM with the next launch
     if (warps == -1) {
         // the caller knows that the call runs alone (copies on both sides of it): one CTA takes the whole SM
         warps = S >= max_warps ? max_warps : S * (max_warps / S);
