@@ -101,18 +101,47 @@ def _special(kind, rng):
         W = torch.from_numpy(W).bfloat16().float().numpy()
     elif kind == "one plane":           # W = c * sign: the second scale is nothing but rounding
         W = (np.where(rng.random(W.shape) < 0.5, 1.0, -1.0) * 0.3).astype(np.float32)
+    elif kind == "planes":              # what two planes represent: the error falls to the rounding of its own sums
+        t = rng.integers(-1, 2, (2,) + W.shape)
+        W = (0.02 * t[0] + 0.0075 * t[1]).astype(np.float32)
     elif kind == "extremes":
         W[:20] *= np.float32(1e-41)     # subnormal
         W[20:40] *= np.float32(1e36)
     return W
 
 
-@pytest.mark.parametrize("kind", ["inexact sums", "few values", "short mantissas", "one plane", "extremes"])
+@pytest.mark.parametrize("kind", ["inexact sums", "few values", "short mantissas", "one plane", "planes", "extremes"])
 @pytest.mark.parametrize("G,kw,okw", [(128, {}, {}), (20, {}, {}), (160, {"eps": 1e-2}, {"eps": 1e-2}),
                                       (5, {"t_max": 2}, {"T_max": 2}), (64, {"eps": 0.0, "t_max": 30}, {"eps": 0.0, "T_max": 30})])
 def test_sorted_sweeps_match_the_oracle(kind, G, kw, okw):
     W = _special(kind, np.random.default_rng(70 + G))
     assert_same(run(W, group=G, **kw), decompose_c(W, G=G, **okw), "%s G=%d" % (kind, G))
+
+
+@pytest.mark.parametrize("G", [128, 20, 7])
+def test_non_finite_weights_stay_in_their_group_rows(G):
+    # a NaN or an infinity makes the scales of its group-row NaN in the first sweep and its planes 0 (no candidate is nearer than
+    # another); the rule is then never met, and the other group-rows are those of t_max sweeps
+    W = (np.random.default_rng(90 + G).standard_normal((40, 8 * G)) * 0.02).astype(np.float32)
+    hurt = np.zeros((40, 8), bool)
+    for row, col, v in ((0, 3, np.nan), (5, 2 * G, np.inf), (5, 7 * G + 1, -np.inf), (39, 8 * G - 1, np.nan), (17, G, np.inf),
+                        (17, G + 2, -np.inf)):
+        W[row, col] = v
+        hurt[row, col // G] = True
+    ref = decompose_c(np.where(np.isfinite(W), W, np.float32(0.01)), G=G, T_max=9, eps=0.0)
+    for canonicalize in (True, False):
+        got = run(W, group=G, t_max=9, canonicalize=canonicalize)
+        if not canonicalize:
+            ref = decompose_c(np.where(np.isfinite(W), W, np.float32(0.01)), G=G, T_max=9, eps=0.0, canonicalize=False)
+        assert got["sweeps"] == 9
+        cols = np.repeat(hurt, G, axis=1)
+        for k in ("T1", "T2"):
+            assert np.array_equal(got[k][~cols], ref[k][~cols]) and not got[k][cols].any()
+        for k in ("alpha1", "alpha2"):
+            assert np.all(np.abs(got[k][~hurt] - ref[k][~hurt]) <= 1e-12) and np.isnan(got[k][hurt]).all()
+            assert np.array_equal(got[k + "_fp16"][~hurt].view(np.uint16), ref[k + "_fp16"][~hurt].view(np.uint16))
+            assert np.isnan(got[k + "_fp16"][hurt]).all()
+        assert np.isnan(got["delta_history"]).all() and np.isnan(got["err_history"]).all()
 
 
 def test_decompose_pack_gemv_pipeline_on_the_gpu():
