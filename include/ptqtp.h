@@ -204,7 +204,7 @@ PTQTP_API ptqtp_status ptqtp_gemm_skinny(const ptqtp_shape *shape /* host */, co
 /* ptqtp_gemm_skinny on format 3 with the kernel chosen by the caller (tuning and tests; PTQTP_ERR_CONFIG for the
  * other formats).  path: 0 = library choice, 5 = int8 MMAs on block-fixed-point activations, 6 = fp16 activations as
  * given.  k_split (path 6): with 1, 2, 4 or 8 the tcgen05 kernel, that many CTAs of a cluster sharing the columns of a block
- * of 128 rows; 0 = library choice of kernel and split.  Same result definition as ptqtp_gemm_skinny. */
+ * of 128 rows; -1 = the tcgen05 kernel with a split of its own choice; 0 = library choice of kernel and split.  Same result definition as ptqtp_gemm_skinny. */
 PTQTP_API ptqtp_status ptqtp_gemm_skinny_cfg(const ptqtp_shape *shape /* host */, const void *packed, size_t packed_bytes,
                                    int32_t m, const uint16_t *X, uint16_t *Y, int32_t path, int32_t k_split,
                                    void *stream);

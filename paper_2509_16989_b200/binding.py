@@ -298,7 +298,7 @@ def ptqtp_gemm_skinny(packed, N, K, X, Y=None, stream=None, fmt=None):
 
 
 def ptqtp_gemm_skinny_cfg(packed, N, K, X, Y=None, path=0, k_split=0, stream=None):
-    """ptqtp_gemm_skinny on format 3 with the kernel chosen by the caller (path 0 / 5 / 6, k_split 0 / 1 / 2 / 4 / 8)."""
+    """ptqtp_gemm_skinny on format 3 with the kernel chosen by the caller (path 0 / 5 / 6, k_split -1 / 0 / 1 / 2 / 4 / 8)."""
     shape = _shape_ref(N, K, FORMAT_V3)
     M = X.shape[0]
     if Y is None:

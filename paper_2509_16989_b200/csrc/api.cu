@@ -263,7 +263,7 @@ static bool fp16_activations(const Layout3& L3, int m) {
 }
 // Kernels, in microseconds per call in a chain of its kind (14336 x 4096, 4096 x 14336, 4096 x 4096, 1024 x 4096):
 //   fp16: the warp-MMA kernel while one launch takes all rows (8 rows: 14.5, 15.7, 6.5, 4.2; 16: 20.3, 21.9, 8.8, 5.3),
-//   the tcgen05 kernel otherwise and with k_split (30.2, 27.3, 11.0, 8.1; 30.8, 28.0, 11.5, 8.2; at 64 rows 50.5, 43.5,
+//   the tcgen05 kernel otherwise and with k_split (-1: a split of its own choice) (30.2, 27.3, 11.0, 8.1; 30.8, 28.0, 11.5, 8.2; at 64 rows 50.5, 43.5,
 //   17.2, 11.9 against 79, 79, 38, 13.5 in launches of 16 and 32 rows).
 //   int8: four rows 8.7, 10.5, 5.2, 3.6 on the warp-MMA kernel, 15.0, 27.4, 5.6, 2.6 on the batch-1 tiles kernel at overlap
 //   level 2, where its launches overlap (16.5, 27.5, 8.6, 6.5 at level 0): small matrices of up to four rows stay there,
@@ -272,7 +272,7 @@ static ptqtp_status skinny_v3(const Layout3& L3, const void* packed, int m, cons
                               int k_split, cudaStream_t st) {
     if (path == 6 || (path == 0 && fp16_activations(L3, m))) {
         if (k_split == 0 && gemm7_one_launch(L3, m, false)) return launch_gemm7(L3, packed, m, X, Y, false, st);
-        return launch_gemm6(L3, packed, m, X, Y, k_split, st);
+        return launch_gemm6(L3, packed, m, X, Y, k_split == -1 ? 0 : k_split, st);
     }
     if (m > 4 || (m > 1 && L3.k > 8192) || (m > 2 && L3.total > 8500000)) return launch_gemm7(L3, packed, m, X, Y, true, st);
     if (m == 1) return launch_gemv4(L3, packed, X, Y, 0, 0, 0, 0, st);

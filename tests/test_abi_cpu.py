@@ -128,6 +128,7 @@ def test_host_side_validation_codes(L):
     assert L.ptqtp_gemm_skinny_cfg(sp, ok_ptr, size, 8, ok_ptr, ok_ptr, 6, 0, None) == binding.ERR_CONFIG
     assert L.ptqtp_gemm_skinny_cfg(ctypes.byref(s3), ok_ptr, z3, 8, ok_ptr, ok_ptr, 4, 0, None) == binding.ERR_CONFIG
     assert L.ptqtp_gemm_skinny_cfg(ctypes.byref(s3), ok_ptr, z3, 8, ok_ptr, ok_ptr, 6, 3, None) == binding.ERR_CONFIG
+    assert L.ptqtp_gemm_skinny_cfg(ctypes.byref(s3), ok_ptr, z3, 8, ok_ptr, ok_ptr, 6, -2, None) == binding.ERR_CONFIG
     assert L.ptqtp_gemm_skinny_cfg(ctypes.byref(s3), ok_ptr, z3, 0, ok_ptr, ok_ptr, 6, 0, None) == binding.ERR_SHAPE
     assert L.ptqtp_gemm_skinny_cfg(ctypes.byref(s3), ok_ptr, z3, 8, odd_ptr, ok_ptr, 6, 0, None) == binding.ERR_ALIGN
     assert L.ptqtp_gemm_skinny_cfg(ctypes.byref(s3), ok_ptr, z3, 8, None, ok_ptr, 6, 0, None) == binding.ERR_NULL

@@ -22,9 +22,10 @@ def _run(c, packed, N, K, **kw):
 @pytest.mark.parametrize("N,K,M", [(1, 128, 2), (5, 256, 5), (7, 1152, 16), (33, 2048, 17), (130, 3200, 31),
                                    (257, 5120, 32), (64, 14336, 33), (1000, 6144, 48), (37, 36864, 49),
                                    (192, 3072, 64), (2400, 4096, 9), (129, 640, 2), (255, 512, 64), (256, 384, 20)])
-def test_ragged_shapes_and_batch_sizes(N, K, M):
+@pytest.mark.parametrize("k_split", [0, -1])             # 0: up to 32 rows the warp-MMA kernel, as the library would
+def test_ragged_shapes_and_batch_sizes(N, K, M, k_split):
     c = make_case(N, K, seed=900 + N + M, M=M)
-    Y = _run(c, pack_case(c, V3), N, K)
+    Y = _run(c, pack_case(c, V3), N, K, k_split=k_split)
     assert_parity(Y, np.atleast_2d(oracle_y(c)), np.atleast_2d(c["x"]), "N=%d K=%d M=%d" % (N, K, M))
     assert binding.ptqtp_kernel_status() == 0
 
@@ -41,9 +42,10 @@ def test_every_k_split(N, K, M, k_split):
 
 @pytest.mark.parametrize("N,K,M", [(14336, 4096, 64), (4096, 14336, 16), (1024, 4096, 37), (4096, 4096, 8),
                                    (28672, 4096, 33)])
-def test_full_size_shapes(N, K, M):
+@pytest.mark.parametrize("k_split", [0, -1])
+def test_full_size_shapes(N, K, M, k_split):
     c = make_case(N, K, seed=5 + M, M=M)
-    Y = _run(c, pack_case(c, V3), N, K)
+    Y = _run(c, pack_case(c, V3), N, K, k_split=k_split)
     assert_parity(Y, oracle_y(c), c["x"], "N=%d K=%d M=%d" % (N, K, M))
     assert binding.ptqtp_kernel_status() == 0
 
@@ -65,6 +67,17 @@ def test_exact_on_integers():
             cm = dict(c, x=c["x"][:m].copy())
             Y = _run(cm, packed, N, K, k_split=k_split)
             assert np.array_equal(Y.astype(np.int64), exact[:m]), (m, k_split)
+
+
+@pytest.mark.parametrize("N,K,M", [(300, 4096, 40), (14336, 4096, 16), (4096, 4096, 64)])
+def test_the_tcgen05_kernel_can_be_asked_for_with_a_split_of_its_own(N, K, M):
+    # k_split = -1 is one of the explicit splits, bit for bit; 0 is the library's choice of kernel, which for up to 32 rows is another one
+    # (sums that differ in the last bits of fp32: some of 229376 results round to another fp16 number)
+    c = make_case(N, K, seed=88, M=M)
+    packed = pack_case(c, V3)
+    own, chosen = (_run(c, packed, N, K, k_split=k).view(np.uint16) for k in (-1, 0))
+    assert any(np.array_equal(own, _run(c, packed, N, K, k_split=k).view(np.uint16)) for k in (1, 2, 4, 8))
+    assert np.array_equal(own, chosen) == (M > 32)
 
 
 def test_rows_do_not_depend_on_their_neighbours():
@@ -102,7 +115,7 @@ def test_argument_checks():
     c = make_case(N, K, seed=1, M=8)
     x = dev(c["x"])
     p3 = pack_case(c, V3)
-    for kw in (dict(path=4), dict(path=6, k_split=3), dict(path=6, k_split=16)):
+    for kw in (dict(path=4), dict(path=6, k_split=3), dict(path=6, k_split=16), dict(path=6, k_split=-2)):
         with pytest.raises(binding.PtqtpError) as e:
             binding.ptqtp_gemm_skinny_cfg(p3, N, K, x, **kw)
         assert e.value.status == binding.ERR_CONFIG
@@ -141,7 +154,7 @@ def test_many_launches_on_two_streams_give_the_same_bits():
     xs = [dev(c["x"]) for c in cs]
     want = []
     for c, p, x in zip(cs, packed, xs):
-        want.append(binding.ptqtp_gemm_skinny_cfg(p, N, K, x, path=6).cpu().numpy().view(np.uint16))
+        want.append(binding.ptqtp_gemm_skinny_cfg(p, N, K, x, path=6, k_split=-1).cpu().numpy().view(np.uint16))
     streams = [torch.cuda.Stream(), torch.cuda.Stream()]
     outs = [[torch.empty((x.shape[0], N), dtype=torch.float16, device="cuda") for x in xs] for _ in range(2)]
     torch.cuda.synchronize()
@@ -160,5 +173,5 @@ def test_many_launches_on_two_streams_give_the_same_bits():
             got = outs[si][j].cpu().numpy()
             assert_parity(got, oracle_y(cs[j]), cs[j]["x"], "stream %d case %d" % (si, j))
     for j in range(4):
-        a = binding.ptqtp_gemm_skinny_cfg(packed[j], N, K, xs[j], path=6).cpu().numpy().view(np.uint16)
+        a = binding.ptqtp_gemm_skinny_cfg(packed[j], N, K, xs[j], path=6, k_split=-1).cpu().numpy().view(np.uint16)
         assert np.array_equal(a, want[j])
