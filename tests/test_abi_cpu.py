@@ -154,7 +154,7 @@ def test_decompose_host_side_checks(L):
 
 
 def test_process_wide_settings_defaults_and_setters(L):
-    # plain launches are the default: every buffer, the packed blob included, follows stream order
+    # the default is level 0: every buffer, the packed blob included, follows stream order
     assert L.ptqtp_set_overlap(1) == 0
     assert L.ptqtp_set_overlap(7) == 1
     assert L.ptqtp_set_overlap(-3) == 2

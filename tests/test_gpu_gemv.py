@@ -441,18 +441,21 @@ def test_gemm_skinny_config2_shape_every_batch_size_both_entry_points(M):
     assert_parity(Yw.cpu().numpy()[:, rows], ref, c["x"], "gemm_skinny_ws M=%d" % M)
 
 
-def test_gemm_skinny_ws_two_rounds_per_cta_on_the_70b_shape():
+@pytest.mark.parametrize("M,converts", [(8, False), (9, True), (16, True)])
+def test_gemm_skinny_ws_two_rounds_per_cta_on_the_70b_shape(M, converts):
     # N > 17760: a CTA of the workspace kernel owns more quads than it has compute warps and takes a second round
-    # (accumulators reset, code steps crossing the round boundary); the static entry point shares that path
+    # (accumulators reset, code steps crossing the round boundary); the static entry point shares that path.  Up to eight rows take
+    # the warp-MMA kernel, which leaves the workspace alone.
     N, K = LLAMA3_70B["gate_up"]
-    M = 8
     c = make_case(N, K, seed=3, M=M, p_zero=0.5)
     packed = pack_case(c, binding.FORMAT_V2)
     rows = _edge_and_sampled_rows(N, 6)
     ref = oracle_y(c, rows)
     X = dev(c["x"])
-    Yw = binding.ptqtp_gemm_skinny_ws(packed, N, K, X, fmt=binding.FORMAT_V2)
+    ws = torch.full((binding.gemm_skinny_workspace_size(N, K, M, fmt=binding.FORMAT_V2),), 0xA5, dtype=torch.uint8, device="cuda")
+    Yw = binding.ptqtp_gemm_skinny_ws(packed, N, K, X, workspace=ws, fmt=binding.FORMAT_V2)
     torch.cuda.synchronize()
+    assert bool((ws != 0xA5).any()) == converts
     assert_parity(Yw.cpu().numpy()[:, rows], ref, c["x"], "gemm_skinny_ws two rounds")
     assert binding.gemm_skinny_workspace_size(N, K, M) <= binding.STATIC_WORKSPACE_BYTES
     Ys = torch.empty((M, N), dtype=torch.float16, device="cuda")
@@ -461,7 +464,7 @@ def test_gemm_skinny_ws_two_rounds_per_cta_on_the_70b_shape():
     assert np.array_equal(Ys.cpu().numpy().view(np.uint16), Yw.cpu().numpy().view(np.uint16))
     Y = binding.ptqtp_gemm_skinny(packed, N, K, X, fmt=binding.FORMAT_V2)
     torch.cuda.synchronize()
-    assert_parity(Y.cpu().numpy()[:, rows], ref, c["x"], "gemm_skinny 70B M=8")
+    assert_parity(Y.cpu().numpy()[:, rows], ref, c["x"], "gemm_skinny 70B M=%d" % M)
 
 
 @pytest.mark.parametrize("N,K,M,alone", [(64, 1152, 5, 1), (300, 4096, 9, 1), (1000, 2048, 61, 1), (4096, 4096, 5, 1), (37, 36864, 3, 1),
@@ -580,7 +583,7 @@ def test_overlapped_chain_keeps_stream_order(graph, level):
 
 @pytest.mark.parametrize("level", [0, 1])
 def test_other_overlap_levels_on_ragged_and_long_shapes(level):
-    # level 0: plain launches with whole-SM CTAs; level 1: dependent launch without speculative execution
+    # level 0: stream order for every buffer; level 1: the packed blob may be read early; no speculative execution at either
     old = binding.ptqtp_set_overlap(level)
     try:
         for N, K in ((5, 1152), (1000, 14336), (37, 36864), (4097, 6144), (2, 128)):

@@ -1,0 +1,184 @@
+"""Stream order of the small-batch kernels, which are launched as dependents of one another at every overlap level: chains in
+which every call reads what the call before it wrote, blobs written directly ahead of a call, the workspace and the output
+shared by consecutive calls.  All results are compared bit for bit with synchronised calls."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2509_16989_b200 import binding
+from paper_2509_16989_b200.inputs import make_case
+from gpu_util import assert_parity, dev, oracle_y, pack_case
+
+pytestmark = pytest.mark.gpu
+V2, V3 = binding.FORMAT_V2, binding.FORMAT_V3
+N = K = 2048
+
+# name -> (format, call); what it runs on 2048 x 2048 by the number of rows:
+#   gemv5/gemm7  two rows: batch-1 tiles kernel; more: warp MMAs on int8 activations
+#   gemm7 fp16   warp MMAs on fp16 activations
+#   gemm6        tcgen05 kernel, two CTAs per row block
+#   gemv3/gemm7  format 2, up to three rows: register-stationary kernel; more: warp MMAs (and a batch-1 launch for a row left alone)
+#   workspace    format 2: warp MMAs, from 17 rows on conversion kernel and workspace kernel
+FORMS = {
+    "gemv5/gemm7": (V3, lambda p, X, Y, ws, n=N, k=K: binding.ptqtp_gemm_skinny_cfg(p, n, k, X, Y=Y, path=5)),
+    "gemm7 fp16": (V3, lambda p, X, Y, ws, n=N, k=K: binding.ptqtp_gemm_skinny_cfg(p, n, k, X, Y=Y, path=6)),
+    "gemm6": (V3, lambda p, X, Y, ws, n=N, k=K: binding.ptqtp_gemm_skinny_cfg(p, n, k, X, Y=Y, path=6, k_split=2)),
+    "gemv3/gemm7": (V2, lambda p, X, Y, ws, n=N, k=K: binding.ptqtp_gemm_skinny(p, n, k, X, Y=Y, fmt=V2)),
+    "workspace": (V2, lambda p, X, Y, ws, n=N, k=K: binding.ptqtp_gemm_skinny_ws(p, n, k, X, Y=Y, workspace=ws, fmt=V2)),
+}
+
+
+@pytest.fixture(scope="module")
+def layers():
+    # two layers with a gain of about one, so that long chains stay in the range of fp16
+    out = []
+    for seed in (50, 51):
+        c = make_case(N, K, seed=seed)
+        for a in ("alpha1", "alpha2"):
+            c[a] = (c[a].astype(np.float32) * 1.28).astype(np.float16)
+        out.append({V2: pack_case(c, V2), V3: pack_case(c, V3)})
+    return out
+
+
+@pytest.fixture(autouse=True)
+def default_level():
+    old = binding.ptqtp_set_overlap(0)
+    yield
+    binding.ptqtp_set_overlap(old)
+
+
+def bits(t):
+    return t.cpu().numpy().view(np.uint16)
+
+
+def every_pair():
+    """Names in an order in which every one follows every one, itself included."""
+    names, out = list(FORMS), []
+    for i, a in enumerate(names):
+        out.append(a)
+        for b in names[i + 1:]:
+            out += [a, b]
+        out.append(a)
+    return out + [names[0]] + names[::-1]
+
+
+@pytest.mark.parametrize("graph", [False, True])
+@pytest.mark.parametrize("level", [0, 1, 2])
+@pytest.mark.parametrize("M", [2, 5, 6, 24])
+def test_chain_of_every_kernel_behind_every_kernel(layers, M, level, graph):
+    order = every_pair()
+    assert len({(a, b) for a, b in zip(order, order[1:])}) == len(FORMS) ** 2
+    X = dev(make_case(N, K, seed=52, M=M)["x"])
+    ws = torch.empty(binding.gemm_skinny_workspace_size(N, K, M, fmt=V2), dtype=torch.uint8, device="cuda")
+    Y = [torch.empty((M, N), dtype=torch.float16, device="cuda") for _ in order]
+    Z = [torch.empty((M, N), dtype=torch.float16, device="cuda") for _ in range(2)]
+
+    def chain(ys, sync=False):
+        for i, name in enumerate(order):
+            fmt, call = FORMS[name]
+            call(layers[i % 2][fmt], X if i == 0 else ys[(i - 1) % len(ys)], ys[i % len(ys)], ws)
+            if sync:
+                torch.cuda.synchronize()
+
+    chain(Y, sync=True)
+    want = [bits(y) for y in Y]
+    assert np.isfinite(want[-1].view(np.float16)).all() and np.abs(want[-1].view(np.float16).astype(np.float64)).max() > 1e-2
+    binding.ptqtp_set_overlap(level)
+    stream = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(stream):
+        for ys in (Y, Z):                                # every result kept, then two buffers that take turns
+            for y in ys:
+                y.fill_(float("nan"))
+            if graph:
+                g = torch.cuda.CUDAGraph()
+                with torch.cuda.graph(g, stream=stream):
+                    chain(ys)
+                for _ in range(3):
+                    g.replay()
+            else:
+                chain(ys)
+                chain(ys)
+            stream.synchronize()
+    for i, y in enumerate(Y):
+        assert np.array_equal(bits(y), want[i]), (i, order[i])
+    assert np.array_equal(bits(Z[(len(order) - 1) % 2]), want[-1])
+    assert binding.ptqtp_kernel_status() == 0
+
+
+@pytest.mark.parametrize("M", [2, 6, 24])
+def test_blob_written_by_a_kernel_directly_ahead_at_level_0(layers, M):
+    # the blob of every call is rewritten by an elementwise kernel, and the call before that is one that releases its dependents early
+    X = dev(make_case(N, K, seed=53, M=M)["x"])
+    ws = torch.empty(binding.gemm_skinny_workspace_size(N, K, M, fmt=V2), dtype=torch.uint8, device="cuda")
+    for name, (fmt, call) in FORMS.items():
+        want = []
+        for lay in layers:
+            y = torch.empty((M, N), dtype=torch.float16, device="cuda")
+            call(lay[fmt], X, y, ws)
+            want.append(bits(y))
+        blob = torch.empty_like(layers[0][fmt])
+        ys = [torch.empty((M, N), dtype=torch.float16, device="cuda") for _ in range(6)]
+        torch.cuda.synchronize()
+        for i, y in enumerate(ys):
+            torch.add(layers[i % 2][fmt], 0, out=blob)
+            call(blob, X, y, ws)
+        torch.cuda.synchronize()
+        for i, y in enumerate(ys):
+            assert np.array_equal(bits(y), want[i % 2]), (name, i)
+
+
+@pytest.mark.parametrize("level", [0, 1, 2])
+@pytest.mark.parametrize("M", [2, 6, 24])
+def test_pack_directly_before_a_call(M, level):
+    # the same blob is packed anew and used by the next call without any synchronisation
+    cs = [make_case(N, K, seed=54 + i, M=M) for i in range(2)]
+    X = dev(cs[0]["x"])
+    planes = [tuple(dev(c[k]) for k in ("T1", "T2", "alpha1", "alpha2")) for c in cs]
+    ws = torch.empty(binding.gemm_skinny_workspace_size(N, K, M, fmt=V2), dtype=torch.uint8, device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    refs = [oracle_y(dict(c, x=cs[0]["x"])) for c in cs]
+    binding.ptqtp_set_overlap(level)
+    for name, (fmt, call) in FORMS.items():
+        blob = torch.empty(binding.packed_size(N, K, fmt=fmt), dtype=torch.uint8, device="cuda")
+        ys = [torch.empty((M, N), dtype=torch.float16, device="cuda") for _ in range(6)]
+        torch.cuda.synchronize()
+        for i, y in enumerate(ys):
+            binding.ptqtp_pack(*planes[i % 2], packed=blob, dev_status=status, fmt=fmt)
+            call(blob, X, y, ws)
+        torch.cuda.synchronize()
+        for i, y in enumerate(ys):
+            assert_parity(y.cpu().numpy(), refs[i % 2], cs[0]["x"], "%s call %d" % (name, i))
+            assert np.array_equal(bits(y), bits(ys[i % 2])), (name, i)
+    assert int(status.item()) == 0
+
+
+@pytest.mark.parametrize("level", [0, 1, 2])
+def test_small_batch_behind_batch_1_and_back(layers, level):
+    # activations of a batch written row by row by batch-1 calls, and a row of a small-batch result read by a batch-1 call
+    M = 6
+    x = dev(make_case(N, K, seed=56, M=M)["x"])
+    ws = torch.empty(binding.gemm_skinny_workspace_size(N, K, M, fmt=V2), dtype=torch.uint8, device="cuda")
+
+    def run(sync):
+        out = []
+        for name, (fmt, call) in FORMS.items():
+            X = torch.full((M, K), float("nan"), dtype=torch.float16, device="cuda")
+            Y, z = torch.empty((M, N), dtype=torch.float16, device="cuda"), torch.empty(N, dtype=torch.float16, device="cuda")
+            torch.cuda.synchronize()
+            for m in range(M):
+                binding.ptqtp_gemv(layers[0][fmt], N, K, x[m], y=X[m], fmt=fmt)
+                if sync:
+                    torch.cuda.synchronize()
+            call(layers[1][fmt], X, Y, ws)
+            if sync:
+                torch.cuda.synchronize()
+            binding.ptqtp_gemv(layers[0][fmt], N, K, Y[M - 1], y=z, fmt=fmt)
+            torch.cuda.synchronize()
+            out.append((name, bits(Y), bits(z)))
+        return out
+
+    want = run(True)
+    binding.ptqtp_set_overlap(level)
+    for (name, Y, z), (_, Yw, zw) in zip(run(False), want):
+        assert np.array_equal(Y, Yw) and np.array_equal(z, zw), name

@@ -29,9 +29,11 @@ def close_to(y_new, y_old, x):
         assert np.max(np.abs(a[m] - b[m])) <= MAX_ABS_COEF * np.max(np.abs(x[m].astype(np.float64))) * np.sqrt(x.shape[1])
 
 
-def test_static_workspace_entry_point_matches_workspace_entry_point_twice():
+@pytest.mark.parametrize("M,converts", [(6, False), (24, True)])
+def test_static_workspace_entry_point_matches_workspace_entry_point_twice(M, converts):
+    # six rows take a kernel that leaves the workspace alone, 24 the one that converts X into it
     L = binding.lib()
-    N, K, M = 1000, 4096, 6
+    N, K = 1000, 4096
     c = make_case(N, K, seed=70, M=M)
     packed, st = binding.ptqtp_pack(dev(c["T1"]), dev(c["T2"]), dev(c["alpha1"]), dev(c["alpha2"]))
     torch.cuda.synchronize()
@@ -40,7 +42,7 @@ def test_static_workspace_entry_point_matches_workspace_entry_point_twice():
     stream = ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
     need = binding.gemm_skinny_workspace_size(N, K, M)
     assert 0 < need <= binding.STATIC_WORKSPACE_BYTES
-    ws = torch.empty(need, dtype=torch.uint8, device="cuda")
+    ws = torch.full((need,), 0xA5, dtype=torch.uint8, device="cuda")
     for call, seed in enumerate((71, 72)):                       # two calls in a row, different activations
         x = make_case(N, K, seed=seed, M=M)["x"]
         X = dev(x)
@@ -49,6 +51,8 @@ def test_static_workspace_entry_point_matches_workspace_entry_point_twice():
         rc = L.ptqtp_gemm_skinny_ws(ctypes.byref(shape), packed.data_ptr(), packed.numel(), M, X.data_ptr(),
                                     Y_old.data_ptr(), ws.data_ptr(), ws.numel(), stream)
         assert rc == binding.OK
+        torch.cuda.synchronize()
+        assert bool((ws != 0xA5).any()) == converts
         rc = L.ptqtp_gemm_skinny_static(ctypes.byref(shape), packed.data_ptr(), packed.numel(), M, X.data_ptr(),
                                         Y_new.data_ptr(), stream)
         assert rc == binding.OK, binding.status_string(rc)
