@@ -9,7 +9,7 @@ namespace ptqtp {
 
 static thread_local int g_last_cuda_error = 0;
 // Process-wide settings, read by every launch and written by their setters from any thread.
-static std::atomic<int> g_overlap{0};                  // ptqtp_set_overlap: plain launches unless the caller opts in
+static std::atomic<int> g_overlap{0};                  // ptqtp_set_overlap: stream order for every buffer unless the caller opts in
 static std::atomic<int> g_wait_limit{1 << 22};         // ptqtp_set_wait_limit
 static std::atomic<int> g_fail_waits{0};               // ptqtp_test_fail_next_wait
 
@@ -22,8 +22,8 @@ bool take_injected_wait_failure() {
     return false;
 }
 
-// Streams on which ptqtp_pack was the library's last call: the next GEMV launch there is a plain launch, so that
-// it reads the packed planes only after the pack kernel has completed (a dependent launch reads them earlier).
+// Streams on which ptqtp_pack was the library's last call: the next launch there that would read packed planes before earlier
+// work of the stream is complete (overlap levels 1 and 2) is a plain one, or waits first.
 static std::mutex g_pack_mutex;
 static std::vector<cudaStream_t> g_pack_streams;
 static bool g_pack_overflow = false;
@@ -261,20 +261,23 @@ static bool fp16_activations(const Layout3& L3, int m) {
     const double us5 = full * (1.2 + mb / rate4) + (rest > 2 ? 1.2 + mb / rate4 : rest > 0 ? 1.2 + mb / rate2 : 0.0);
     return us6 < us5;
 }
-// Kernels, in microseconds per call in a chain of its kind (14336 x 4096, 4096 x 14336, 4096 x 4096, 1024 x 4096):
-//   fp16: the warp-MMA kernel while one launch takes all rows (8 rows: 14.5, 15.7, 6.5, 4.2; 16: 20.3, 21.9, 8.8, 5.3),
-//   the tcgen05 kernel otherwise and with k_split (-1: a split of its own choice) (30.2, 27.3, 11.0, 8.1; 30.8, 28.0, 11.5, 8.2; at 64 rows 50.5, 43.5,
-//   17.2, 11.9 against 79, 79, 38, 13.5 in launches of 16 and 32 rows).
-//   int8: four rows 8.7, 10.5, 5.2, 3.6 on the warp-MMA kernel, 15.0, 27.4, 5.6, 2.6 on the batch-1 tiles kernel at overlap
-//   level 2, where its launches overlap (16.5, 27.5, 8.6, 6.5 at level 0): small matrices of up to four rows stay there,
-//   and so do two rows (6.9, 13.2, 3.2, 2.0 at level 2 against 8.4, 9.8, 5.2, 3.5) unless K is long.
+// Kernels, in microseconds per call in a chain of its kind at overlap level 0 (14336 x 4096, 4096 x 14336, 4096 x 4096, 1024 x 4096):
+//   fp16: the warp-MMA kernel while one launch takes all rows (8 rows: 14.7, 15.7, 6.5, 4.2; 16: 20.3, 21.7, 8.8, 5.2),
+//   the tcgen05 kernel otherwise and with k_split (-1: a split of its own choice) (30.2, 27.3, 11.0, 8.1; 30.8, 28.0, 11.5, 8.2; at 64 rows 50.3, 43.7,
+//   17.4, 11.6 against 79, 79, 38, 13.5 in launches of 16 and 32 rows).
+//   int8: four rows 9.5, 10.4, 5.4, 3.6 on the warp-MMA kernel, 17.4, 28.3, 7.6, 5.7 on the batch-1 tiles kernel, whose launches
+//   overlap at level 2 (9.2, 10.6, 5.3, 3.6 and 15.6, 28.3, 6.3, 3.3 there).  At level 2 the line is between 2.2 MB (1024 x 4096,
+//   2048 x 2048: 3.3, 2.9 against 3.6, 3.4) and 4.5 MB (2048 x 4096: 5.0 against 4.2) for three and four rows, and for two rows
+//   at K = 8192 (7.7, 14.0, 3.8, 2.4 against 9.2, 10.4, 5.3, 3.6).  At levels 0 and 1 the warp-MMA kernel is the faster one below
+//   it too (2048 x 2048, three rows: 3.4 against 6.2); the choice goes by the size alone, so that the bits of a result do not
+//   depend on the level.
 static ptqtp_status skinny_v3(const Layout3& L3, const void* packed, int m, const uint16_t* X, uint16_t* Y, int path,
                               int k_split, cudaStream_t st) {
     if (path == 6 || (path == 0 && fp16_activations(L3, m))) {
         if (k_split == 0 && gemm7_one_launch(L3, m, false)) return launch_gemm7(L3, packed, m, X, Y, false, st);
         return launch_gemm6(L3, packed, m, X, Y, k_split == -1 ? 0 : k_split, st);
     }
-    if (m > 4 || (m > 1 && L3.k > 8192) || (m > 2 && L3.total > 8500000)) return launch_gemm7(L3, packed, m, X, Y, true, st);
+    if (m > 4 || (m > 1 && L3.k > 8192) || (m > 2 && L3.total > 4000000)) return launch_gemm7(L3, packed, m, X, Y, true, st);
     if (m == 1) return launch_gemv4(L3, packed, X, Y, 0, 0, 0, 0, st);
     const ptqtp_status s = launch_gemv5(L3, packed, m, X, Y, 0, 0, st);
     return s == PTQTP_ERR_SHAPE ? launch_gemm7(L3, packed, m, X, Y, true, st) : s;       // no room for m rows of x
@@ -282,9 +285,10 @@ static ptqtp_status skinny_v3(const Layout3& L3, const void* packed, int m, cons
 
 // Small batch on format 2, m >= 2.  A row that passes of up to four (as many as find room) leave alone keeps the batch-1
 // kernel's 16-bit activations per 64 columns; the other rows have 15 bits per 128 columns, on either of two kernels: two rows, and
-// up to four on small matrices, take the register-stationary kernel, whose launches overlap at level 2 (two rows of 4096 x 4096 there:
-// 3.8 us against 6.0); the rest the warp-MMA kernel (four rows of 14336 x 4096, 4096 x 14336, 4096 x 4096: 11.2, 12.4,
-// 6.2 us against 13.7, 18.1, 8.1 at level 0 and 11.7, 16.8, 6.9 at level 2).
+// up to four on small matrices, take the register-stationary kernel, whose launches overlap at level 2 (two rows of 4096 x 4096
+// there 4.4 us against 5.6; at level 0 6.6 against 6.0); the rest the warp-MMA kernel.  For three and four rows the line is
+// near 1.1 MB at every level (1024 x 2048: 3.4 and 3.6 us against 3.4 and 3.4 at level 0, 3.6 and 3.9 against 3.5 and 3.4 at level
+// 2; 1024 x 1024 3.1 against 3.3 and 3.1; 1536 x 2048 4.0 and 4.2 against 3.6 and 3.5 at level 2).
 static ptqtp_status skinny_v2(const Layout2& L2, const void* packed, int m, const uint16_t* X, uint16_t* Y, cudaStream_t st) {
     const int per_pass = gemv3_rows_per_pass(L2, m), alone = per_pass == 1 ? m : m % per_pass == 1 ? 1 : 0;
     int rows = m - alone;
@@ -297,7 +301,7 @@ static ptqtp_status skinny_v2(const Layout2& L2, const void* packed, int m, cons
         if (s != PTQTP_OK) { rows = m; break; }          // K too long for it: nothing launched yet
     }
     if (rows == 0) return PTQTP_OK;
-    if (rows > 4 || (L2.k > 8192 && (rows > 2 || !gemm7_uneven(L2))) || (rows > 2 && L2.total > 2000000)) return launch_gemm7(L2, packed, rows, X, Y, st);
+    if (rows > 4 || (L2.k > 8192 && (rows > 2 || !gemm7_uneven(L2))) || (rows > 2 && L2.total > 1400000)) return launch_gemm7(L2, packed, rows, X, Y, st);
     const ptqtp_status s = launch_gemv3(L2, packed, rows, X, Y, 0, 0, 0, st);
     return s == PTQTP_ERR_SHAPE ? launch_gemm7(L2, packed, rows, X, Y, st) : s;
 }
