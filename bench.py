@@ -6,7 +6,7 @@ already resident in HBM.  Steps rotate over `--sets` distinct copies of the laye
 928 MB) so that every packed byte comes from HBM, not from L2.  The timed steps are one CUDA graph
 (up to 512 steps per graph), so a run of 20 steps has no graph boundary inside it.
 
-The library's default is plain launches; this program opts in to overlap level 2 (programmatic
+The library's default is level 0, stream order for every buffer; this program opts in to overlap level 2 (programmatic
 dependent launch with speculative execution) as a decoder would whose packed blobs never change while
 GEMV calls are in flight, and says so in `config.overlap`.
 
@@ -612,7 +612,7 @@ def run_gpu(args):
                 plain = chain.capture(steps_fn(R))
                 detail["step_without_overlap"] = {
                     "us_per_layer": 1e3 * chain.time_ms([plain] * 20) / (20 * R),
-                    "what": "ptqtp_set_overlap(0), the library default: plain launches, every call waits for the one before it"}
+                    "what": "ptqtp_set_overlap(0), the library default: every call reads its buffers after the one before it is complete"}
                 del plain
             finally:
                 binding.ptqtp_set_overlap(old_level)
@@ -666,7 +666,7 @@ def run_gpu(args):
                    "parallelism": "replicas only" if world > 1 else "1 gpu", "bytes_per_step": STEP_BYTES,
                    "packed_format": fmt,
                    "overlap": "opt-in ptqtp_set_overlap(2): programmatic dependent launch with speculative execution "
-                              "(packed blobs are immutable during the run); the library default is plain launches, see "
+                              "(packed blobs are immutable during the run); the library default is level 0 (stream order for every buffer), see "
                               "shapes.step_without_overlap"},
         "us_per_layer": 1e3 * ms_per_step,
         "weight_gbs": STEP_WEIGHT_BYTES / (ms_per_step * 1e-3) / 1e9,

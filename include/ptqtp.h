@@ -347,10 +347,11 @@ PTQTP_API void ptqtp_test_fail_next_wait(int launches);
 
 /* Overlap of consecutive GEMV calls on one stream (process-wide level, default 0; returns the old level).
  * Level 0 (default): every buffer, `packed` included, follows stream order as with plain launches: a kernel sets itself
- * up while the one before it drains, but touches nothing before that one is complete.  Levels 1 and 2 are an opt-in
+ * up while the one before it drains, but reads and writes no buffer before that one is complete (small-batch calls on format 3
+ * prefetch from `packed` into L2, where a later write updates what was prefetched).  Levels 1 and 2 are an opt-in
  * for callers whose packed blobs are immutable while GEMV calls are in flight (the decode case).
  * Level 1: a call may begin reading its `packed` blob while the kernel directly before it on the
- * stream is still draining; x is used and y written only after all earlier work on the stream has completed,
+ * stream is still draining (the small-batch calls do; the batch-1 calls behave as at level 0); x is used and y written only after all earlier work on the stream has completed,
  * so stream order holds for them.  Consequence for the caller: the packed blob of a call must be complete
  * before the kernel directly ahead of the call on its stream ends -- it must not be the output buffer of that
  * kernel.  ptqtp_pack is exempt (the first GEMV call after a ptqtp_pack on the same stream reads nothing before the

@@ -20,8 +20,8 @@
 // What bounds it, from microbenchmarks on the issue port of an SM quarter: an MMA costs 8 cycles of the tensor pipe and 4 of
 // issue, a mask 2, another instruction 1.  A tile is 64 MMAs per 8 rows, 288 masks and shifts and 256 FMAs in fp16: about 270
 // cycles per SM at 8 rows, 340 at 16, against 187 of HBM; int8 with 4 rows 32 MMAs and 96 masks: about 130.  On top of that 3 us
-// per launch: start, activations, last sums.  14336 x 4096, microseconds per call in a chain at level 0: 4 rows 9.7 (one-group
-// fragments of gemv5: 17.4), 8 rows 14.5 and 16 rows 20.3 (tcgen05 kernel: 31.2, 31.9).
+// per launch: start, activations, last sums.  14336 x 4096, microseconds per call in a chain at level 0: 4 rows 9.5 (one-group
+// fragments of gemv5: 17.4), 8 rows 14.7 and 16 rows 20.3 (tcgen05 kernel: 31.2, 31.9).
 // Clusters of 4 and 8 leave 16 and 28 SMs idle (33 and 15 fit); larger C only where an activation slice does not fit.
 //
 // The same work on tcgen05 with operand A masked straight into tensor memory (64- and 128-row blocks, one or both planes per
@@ -260,7 +260,7 @@ __device__ __forceinline__ void group_int8(const uint32_t (&word)[8], const unsi
 
 // fp16: the trits of field F (two columns) as multiples of 2^-9.  A code under its mask is the subnormal code * 4^F * 2^-24; one
 // FMA makes it code * 2^-9, less the 1 that a code is more than its trit: exact.  (The masked codes themselves as operand A and
-// the sum of x taken off afterwards saved the FMAs, 14336 x 4096 at 8 and 16 rows 13.0 and 18.8 us against 14.5 and 20.3, but a
+// the sum of x taken off afterwards saved the FMAs, 14336 x 4096 at 8 and 16 rows 13.0 and 18.8 us against 14.7 and 20.3, but a
 // sum then has x where the trit is 0, and the MMA cuts products with a subnormal factor off where it would if that factor
 // were 2^-14: 2.6e-6 of the result on normal x, 0.1 of it next to columns of 30000.)
 template <int F>
@@ -787,8 +787,8 @@ bool gemm7_one_launch(const Layout2& L, int m) {
 // 62 on the workspace kernel; 16384 x 28672 85 against 78 and 129 against 103; 16 slices: 8192 x 32768 46 against 51, 65
 // against 68).
 bool gemm7_uneven(const Layout2& L) {
-    const Plan7 p = plan7<2, true>((L.nrp + kTileRp3 - 1) / kTileRp3, (L.k + kSuper3 - 1) / kSuper3);
-    return p.csize == 8 && p.blocks % 8 != 0;
+    if (L.slices <= 8 || L.slices % 8 == 0) return false;
+    return plan7<2, true>((L.nrp + kTileRp3 - 1) / kTileRp3, (L.k + kSuper3 - 1) / kSuper3).csize == 8;
 }
 
 // 1 <= m <= 64 rows of X (16-byte aligned).
