@@ -262,7 +262,7 @@ static bool fp16_activations(const Layout3& L3, int m) {
     return us6 < us5;
 }
 // Kernels, in microseconds per call in a chain of its kind at overlap level 0 (14336 x 4096, 4096 x 14336, 4096 x 4096, 1024 x 4096):
-//   fp16: the warp-MMA kernel while one launch takes all rows (8 rows: 14.7, 15.7, 6.5, 4.2; 16: 20.3, 21.7, 8.8, 5.2),
+//   fp16: the warp-MMA kernel while one launch takes all rows (8 rows: 14.3, 15.3, 6.4, 4.3; 16: 19.9, 21.3, 8.6, 5.3),
 //   the tcgen05 kernel otherwise and with k_split (-1: a split of its own choice) (30.2, 27.3, 11.0, 8.1; 30.8, 28.0, 11.5, 8.2; at 64 rows 50.3, 43.7,
 //   17.4, 11.6 against 79, 79, 38, 13.5 in launches of 16 and 32 rows).
 //   int8: four rows 9.5, 10.4, 5.4, 3.6 on the warp-MMA kernel, 17.4, 28.3, 7.6, 5.7 on the batch-1 tiles kernel, whose launches

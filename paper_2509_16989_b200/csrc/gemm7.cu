@@ -5,9 +5,8 @@
 // and multiplies.  Nothing is handed from warp to warp before the end.  The 16 rows of an MMA are 8 row pairs x 2 fields of
 // their code bytes (row of the pair, plane); lanes read the entries of one group pair, not the entries a batch-1 fragment
 // would take, so that an MMA contracts columns of one scale group only.
-//   * fp16 (m16n8k16, fp32 sums; format 3): a mask of the even and one of the odd bytes of a code word and an FMA make
-//     two trits of operand A, for 16 codes 9 half-rate instructions and 8 FMAs.  B is the activations as given, a column of B
-//     one batch row: y += alpha d in fp32.
+//   * fp16 (m16n8k16, fp32 sums; format 3): a shift and a mask of a code word make two trits of operand A, 15 instructions per 16
+//     trits.  B is the activations as given, a column of B one batch row: y += alpha d in fp32.
 //   * int8 (m16n8k32, exact int32 sums; formats 3 and 2): three masks per code word; B the activations in 15-bit block
 //     fixed point per 128 columns (as in gemv5.cu and skinny3.cu), two columns, high and low byte, per batch row.  Codes are
 //     trit + 1: the sum of x over the group comes off in the epilogue, y += alpha 2^s (4^-f d - sum x).
@@ -17,11 +16,11 @@
 // superblocks.  The partial sums of a tile go to one rank's shared memory (st.async in a cluster), slot by slot, and are added in
 // a fixed order at the end: no atomics, no workspace, reproducible.  C and kw depend on the shape alone.
 //
-// What bounds it, from microbenchmarks on the issue port of an SM quarter: an MMA costs 8 cycles of the tensor pipe and 4 of
-// issue, a mask 2, another instruction 1.  A tile is 64 MMAs per 8 rows, 288 masks and shifts and 256 FMAs in fp16: about 270
-// cycles per SM at 8 rows, 340 at 16, against 187 of HBM; int8 with 4 rows 32 MMAs and 96 masks: about 130.  On top of that 3 us
-// per launch: start, activations, last sums.  14336 x 4096, microseconds per call in a chain at level 0: 4 rows 9.5 (one-group
-// fragments of gemv5: 17.4), 8 rows 14.7 and 16 rows 20.3 (tcgen05 kernel: 31.2, 31.9).
+// What bounds it, from microbenchmarks on an SM quarter: an MMA takes 8 cycles, a mask or shift 2 on another pipe beside it, a
+// single-precision instruction 1 that the MMAs wait for.  A tile is 64 MMAs per 8 rows and 480 masks and shifts in fp16: 240 cycles
+// per SM at 8 rows, 256 at 16, and the sums, against 187 of HBM; int8 with 4 rows 32 MMAs and 96 masks: 64.  On top of that 3 us per
+// launch: start, activations, last sums.  14336 x 4096, microseconds per call in a chain at level 0: 4 rows 9.5 (one-group fragments of
+// gemv5: 17.4), 8 rows 14.3 and 16 rows 19.9 (tcgen05 kernel: 31.2, 31.9).
 // Clusters of 4 and 8 leave 16 and 28 SMs idle (33 and 15 fit); larger C only where an activation slice does not fit.
 //
 // The same work on tcgen05 with operand A masked straight into tensor memory (64- and 128-row blocks, one or both planes per
@@ -258,17 +257,16 @@ __device__ __forceinline__ void group_int8(const uint32_t (&word)[8], const unsi
     }
 }
 
-// fp16: the trits of field F (two columns) as multiples of 2^-9.  A code under its mask is the subnormal code * 4^F * 2^-24; one
-// FMA makes it code * 2^-9, less the 1 that a code is more than its trit: exact.  (The masked codes themselves as operand A and
-// the sum of x taken off afterwards saved the FMAs, 14336 x 4096 at 8 and 16 rows 13.0 and 18.8 us against 14.7 and 20.3, but a
-// sum then has x where the trit is 0, and the MMA cuts products with a subnormal factor off where it would if that factor
-// were 2^-14: 2.6e-6 of the result on normal x, 0.1 of it next to columns of 30000.)
-template <int F>
-__device__ __forceinline__ uint32_t trits(uint32_t bytes) {
-    const uint32_t code = bytes & (0x00030003u << (2 * F));
-    const __half2 up = __half2half2(__ushort_as_half((unsigned short)((30 - 2 * F) << 10))), one = __half2half2(__ushort_as_half(0x9800u));
-    const __half2 d = __hfma2(*reinterpret_cast<const __half2*>(&code), up, one);        // 2^(15 - 2 F), -2^-9
-    return *reinterpret_cast<const uint32_t*>(&d);
+// fp16: the trits of field F of the even or odd bytes of a code word (two columns), times 2: a code at the top of a half, inverted, is
+// the sign and the top bit of the exponent (00 -> -2, 01 -> -0, 10 -> 2).  Exact and normal, and all of it on a pipe that
+// runs beside the MMAs (FMAs do not: 8 cycles + 2; made with one FMA per two trits 14336 x 4096 took 14.7 and 20.4 us at 8 and 16
+// rows, against 14.3 and 19.9).  The codes themselves, masked subnormals, as operand A and the sum of x taken off
+// afterwards took 13.0 and 18.8, but a sum then has x where the trit is 0, and the MMA cuts products with a
+// subnormal factor off where it would if that factor were 2^-14: 2.6e-6 of the result on normal x, 0.1 of it next to columns
+// of 30000.
+template <int F, bool ODD>
+__device__ __forceinline__ uint32_t trits(uint32_t word) {
+    return ~(word << ((ODD ? 6 : 14) - 2 * F)) & 0xc000c000u;
 }
 
 // One launch.  The shares are divided on the host (a dozen integer divisions per warp were half a microsecond of a launch): tile0
@@ -460,9 +458,9 @@ gemm7_kernel(const __grid_constant__ Args7 a) {
                         for (int nt = 0; nt < NT; ++nt) b[nt] = *reinterpret_cast<const uint4*>(xb + ((G * NT + nt) * 4 + kk) * 512);
 #pragma unroll
                         for (int s = 0; s < 2; ++s) {
-                            const uint32_t e = word[2 * kk + s], o = e >> 8;
-                            const uint32_t e0 = trits<0>(e), e1 = trits<1>(e), e2 = trits<2>(e), e3 = trits<3>(e);
-                            const uint32_t o0 = trits<0>(o), o1 = trits<1>(o), o2 = trits<2>(o), o3 = trits<3>(o);
+                            const uint32_t w = word[2 * kk + s];
+                            const uint32_t e0 = trits<0, false>(w), e1 = trits<1, false>(w), e2 = trits<2, false>(w), e3 = trits<3, false>(w);
+                            const uint32_t o0 = trits<0, true>(w), o1 = trits<1, true>(w), o2 = trits<2, true>(w), o3 = trits<3, true>(w);
 #pragma unroll
                             for (int nt = 0; nt < NT; ++nt) {
                                 if (kk + s == 0) {
@@ -478,8 +476,7 @@ gemm7_kernel(const __grid_constant__ Args7 a) {
                     const uint2 sc = *reinterpret_cast<const uint2*>(quad);
                     const float2 s0v = __half22float2(*reinterpret_cast<const __half2*>(&sc.x));     // row 2 g: alpha1, alpha2
                     const float2 s1v = __half22float2(*reinterpret_cast<const __half2*>(&sc.y));     // row 2 g + 1
-                    // (the scales times 2^9 are exact)
-                    const float k0 = s0v.x * 0x1p9f, k1 = s0v.y * 0x1p9f, k2 = s1v.x * 0x1p9f, k3 = s1v.y * 0x1p9f;
+                    const float k0 = 0.5f * s0v.x, k1 = 0.5f * s0v.y, k2 = 0.5f * s1v.x, k3 = 0.5f * s1v.y;
 #pragma unroll
                     for (int nt = 0; nt < NT; ++nt) {
                         y[nt][0] = fmaf(k1, ca[nt][2], fmaf(k0, ca[nt][0], y[nt][0]));
