@@ -106,7 +106,7 @@ def test_chain_of_every_kernel_behind_every_kernel(layers, M, level, graph):
     assert binding.ptqtp_kernel_status() == 0
 
 
-@pytest.mark.parametrize("M", [2, 6, 24])
+@pytest.mark.parametrize("M", [2, 5, 6, 24])
 def test_blob_written_by_a_kernel_directly_ahead_at_level_0(layers, M):
     # the blob of every call is rewritten by an elementwise kernel, and the call before that is one that releases its dependents early
     X = dev(make_case(N, K, seed=53, M=M)["x"])
@@ -129,7 +129,7 @@ def test_blob_written_by_a_kernel_directly_ahead_at_level_0(layers, M):
 
 
 @pytest.mark.parametrize("level", [0, 1, 2])
-@pytest.mark.parametrize("M", [2, 6, 24])
+@pytest.mark.parametrize("M", [2, 5, 6, 24])
 def test_pack_directly_before_a_call(M, level):
     # the same blob is packed anew and used by the next call without any synchronisation
     cs = [make_case(N, K, seed=54 + i, M=M) for i in range(2)]
