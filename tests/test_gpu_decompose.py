@@ -118,6 +118,19 @@ def test_sorted_sweeps_match_the_oracle(kind, G, kw, okw):
     assert_same(run(W, group=G, **kw), decompose_c(W, G=G, **okw), "%s G=%d" % (kind, G))
 
 
+@pytest.mark.parametrize("G", [1, 3, 16, 31, 32, 33, 63, 64, 65, 128, 129, 132, 255, 256])
+def test_every_sort_width_and_ragged_batches_of_group_rows(G):
+    # sorts of 32, 64, 128 and 256 values with and without padding, vector loads and single ones, the last batch of 32 group-rows and
+    # of eight cut short; magnitudes repeated with both signs, zeros of both signs among them
+    rng = np.random.default_rng(400 + G)
+    for rows in (1, 7, 9, 33):
+        W = (rng.standard_normal((rows, G)) * 0.02).astype(np.float32)
+        W[:, ::3] = np.copysign(W[:, :1], W[:, ::3])
+        W[::2, 1::5] = np.copysign(np.float32(0.0), W[::2, 1::5])
+        for canonicalize in (True, False):
+            assert_same(run(W, group=G, canonicalize=canonicalize), decompose_c(W, G=G, canonicalize=canonicalize), "%d x %d" % (rows, G))
+
+
 @pytest.mark.parametrize("G", [128, 20, 7])
 def test_non_finite_weights_stay_in_their_group_rows(G):
     # a NaN or an infinity makes the scales of its group-row NaN in the first sweep and its planes 0 (no candidate is nearer than
