@@ -261,10 +261,19 @@ static bool fp16_activations(const Layout3& L3, int m) {
     const double us5 = full * (1.2 + mb / rate4) + (rest > 2 ? 1.2 + mb / rate4 : rest > 0 ? 1.2 + mb / rate2 : 0.0);
     return us6 < us5;
 }
+// fp16: the warp-MMA kernel or the tcgen05 kernel (also with an explicit k_split), in microseconds per call in a chain at overlap level 0:
+//   8 rows: always warp MMAs (14336 x 4096 13.9 and 15.5, 4096 x 14336 14.8 and 15.2, 4096 x 4096 6.0 and 7.5).
+//   9 to 16 rows: warp MMAs take about 4.2 us and 0.445 per MB whatever the shape (1024 x 4096 4.9, 3072 x 3072 6.7, 4096 x 4096 8.2,
+//   6144 x 6144 12.7, 14336 x 4096 19.2, 20480 x 6144 32.5), the tcgen05 kernel what its waves of CTAs take (5.2, 6.9, 7.5, 13.1, 15.6, 38.6).
+//   17 to 32 rows: tcgen05 but for small matrices, where its start and end are most of the call (1024 x 2048 at 24 and 32 rows 5.0 and
+//   5.0 against 5.3 and 5.4, 1024 x 4096 5.4 and 6.4 against 5.7 and 5.8, 2048 x 2048 5.9 and 7.0 against 5.4 and 5.4; 14336 x 4096
+//   33.2 against 17.3).  More rows: always tcgen05.
+static bool warp_mmas_for_fp16(const Layout3& L3, int m) {
+    if (m <= 8) return true;
+    if (m <= 16) return gemm8_us(L3, m) > 4.2 + 0.445 * 1e-6 * (double)L3.total;
+    return m <= 24 ? L3.total < 2300000 && L3.n < 2048 : m <= 32 && L3.total < 1300000;
+}
 // Kernels, in microseconds per call in a chain of its kind at overlap level 0 (14336 x 4096, 4096 x 14336, 4096 x 4096, 1024 x 4096):
-//   fp16: the warp-MMA kernel while one launch takes all rows (8 rows: 14.3, 15.3, 6.4, 4.3; 16: 19.9, 21.3, 8.6, 5.3),
-//   the tcgen05 kernel otherwise and with k_split (-1: a split of its own choice) (30.2, 27.3, 11.0, 8.1; 30.8, 28.0, 11.5, 8.2; at 64 rows 50.3, 43.7,
-//   17.4, 11.6 against 79, 79, 38, 13.5 in launches of 16 and 32 rows).
 //   int8: four rows 9.5, 10.4, 5.4, 3.6 on the warp-MMA kernel, 17.4, 28.3, 7.6, 5.7 on the batch-1 tiles kernel, whose launches
 //   overlap at level 2 (9.2, 10.6, 5.3, 3.6 and 15.6, 28.3, 6.3, 3.3 there).  At level 2 the line is between 2.2 MB (1024 x 4096,
 //   2048 x 2048: 3.3, 2.9 against 3.6, 3.4) and 4.5 MB (2048 x 4096: 5.0 against 4.2) for three and four rows, and for two rows
@@ -274,8 +283,9 @@ static bool fp16_activations(const Layout3& L3, int m) {
 static ptqtp_status skinny_v3(const Layout3& L3, const void* packed, int m, const uint16_t* X, uint16_t* Y, int path,
                               int k_split, cudaStream_t st) {
     if (path == 6 || (path == 0 && fp16_activations(L3, m))) {
-        if (k_split == 0 && gemm7_one_launch(L3, m, false)) return launch_gemm7(L3, packed, m, X, Y, false, st);
-        return launch_gemm6(L3, packed, m, X, Y, k_split == -1 ? 0 : k_split, st);
+        if (k_split == 0 && warp_mmas_for_fp16(L3, m) && gemm7_one_launch(L3, m, false))
+            return launch_gemm7(L3, packed, m, X, Y, false, st);
+        return launch_gemm8(L3, packed, m, X, Y, k_split, st);
     }
     if (m > 4 || (m > 1 && L3.k > 8192) || (m > 2 && L3.total > 4000000)) return launch_gemm7(L3, packed, m, X, Y, true, st);
     if (m == 1) return launch_gemv4(L3, packed, X, Y, 0, 0, 0, 0, st);

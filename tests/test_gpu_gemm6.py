@@ -30,6 +30,20 @@ def test_ragged_shapes_and_batch_sizes(N, K, M, k_split):
     assert binding.ptqtp_kernel_status() == 0
 
 
+@pytest.mark.parametrize("K", [128, 384, 512, 640, 2176, 4608])
+def test_every_number_of_tiles_and_groups_left_over(K):
+    # blocks of one to eight tiles (quarters of a block empty or half full), rows that no 16-byte store takes, superblocks of one to four
+    # groups at the end, more and fewer superblocks than stages, both sides of every class of batch sizes
+    for i, N in enumerate((1, 15, 17, 40, 63, 79, 96, 113, 128, 136, 241)):
+        for M in ((16, 33), (17, 48), (32, 64), (9, 49))[i % 4]:
+            c = make_case(N, K, seed=600 + N + M, M=M)
+            packed = pack_case(c, V3)
+            for k_split in (-1, 1, 0):
+                Y = _run(c, packed, N, K, k_split=k_split)
+                assert_parity(Y, np.atleast_2d(oracle_y(c)), np.atleast_2d(c["x"]), "N=%d K=%d M=%d split %d" % (N, K, M, k_split))
+    assert binding.ptqtp_kernel_status() == 0
+
+
 @pytest.mark.parametrize("k_split", [1, 2, 4, 8])
 @pytest.mark.parametrize("N,K,M", [(300, 4096, 24), (130, 1536, 64), (2050, 512, 7), (48, 7168, 40)])
 def test_every_k_split(N, K, M, k_split):
