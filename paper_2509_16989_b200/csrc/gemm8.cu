@@ -327,7 +327,6 @@ gemm8_kernel(const __grid_constant__ Args8 a) {
                 tc_fence_after();
 #pragma unroll
                 for (int tl = 0; tl < 2; ++tl) {
-                    const bool live = 2 * q + tl < tiles;
                     const uint32_t dst = tlane + 64 * stage + ((uint32_t)(16 * tl) << 16);
                     uint32_t w[4], p[16];
 #pragma unroll
@@ -336,13 +335,13 @@ gemm8_kernel(const __grid_constant__ Args8 a) {
                         p[4 * i] = trits<0, false>(w[i]); p[4 * i + 1] = trits<0, true>(w[i]);
                         p[4 * i + 2] = trits<2, false>(w[i]); p[4 * i + 3] = trits<2, true>(w[i]);
                     }
-                    if (live) tmem_st_16x256b_x4(dst, p);
+                    tmem_st_16x256b_x4(dst, p);          // (a tile past the block's: lanes that nobody reads)
 #pragma unroll
                     for (int i = 0; i < 4; ++i) {
                         p[4 * i] = trits<1, false>(w[i]); p[4 * i + 1] = trits<1, true>(w[i]);
                         p[4 * i + 2] = trits<3, false>(w[i]); p[4 * i + 3] = trits<3, true>(w[i]);
                     }
-                    if (live) tmem_st_16x256b_x4(dst + 32, p);
+                    tmem_st_16x256b_x4(dst + 32, p);
                 }
                 asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
                 tc_fence_before();
@@ -359,7 +358,7 @@ gemm8_kernel(const __grid_constant__ Args8 a) {
         uint64_t y[C::kSums / 2], part[LEVELS == 2 ? C::kSums / 2 : 1];
 #pragma unroll
         for (int i = 0; i < C::kSums / 2; ++i) y[i] = 0ull;
-        int cs = 0, gi = 0, ds = 0;
+        int cs = 0, gi = 0;
         uint32_t cph = 0;
         bool ok = true;
 #pragma unroll 1
@@ -378,6 +377,7 @@ gemm8_kernel(const __grid_constant__ Args8 a) {
 #pragma unroll
             for (int G = 0; G < 4; ++G, ++gi) {
                 if (gi >= ng) break;
+                const int ds = G % C::kDSets;        // (superblocks start with an even group)
                 ok = group_done(gi);
                 if (!ok) break;
                 tc_fence_after();
@@ -400,7 +400,6 @@ gemm8_kernel(const __grid_constant__ Args8 a) {
                         else y[(c0 + i) / 2] = add2(y[(c0 + i) / 2], fma2(a1, e1, fma2(a2, e2, 0ull)));       // (one rounding at the size of the sum)
                     }
                 }
-                if (++ds == C::kDSets) ds = 0;
             }
             if constexpr (LEVELS == 2) {
 #pragma unroll
