@@ -189,12 +189,11 @@ PTQTP_API ptqtp_status ptqtp_gemv_multi(int32_t count, const ptqtp_shape *shapes
 
 /* Small-batch variant: Y[m,:] = layer(X[m,:]) for m < M, 1 <= M <= PTQTP_MAX_BATCH.
  * X: device fp16 [M*K] row-major; Y: device fp16 [M*N] row-major.  Same definition per row of X.
- * Format 2, M >= 2, and format 3, M <= 4 and larger M on small matrices: the planes are contracted on the tensor cores
- * with int8 warp MMAs against 15-bit block-fixed-point activations (blocks of 128 columns), exact int32 sums, fp32
- * scale epilogue.  Format 3, more rows (from M = 5 to about 20, by the size of the matrix): the activations are fp16
- * operands as given (no quantisation), the trits exact fp16 numbers, the sums of a scale group accumulate in fp32 and get the
- * fp32 scale epilogue.  One pass over the planes takes up to 16 (int8) or 32 (fp16) rows, fewer when K is very
- * long; more rows take several passes, or on format 3 with fp16 operands one pass on the tcgen05 tensor cores.
+ * Format 2, 2 <= M <= 8 (16 on small matrices), and format 3, M <= 4 and larger M on small matrices: the planes are contracted
+ * on the tensor cores with int8 warp MMAs against 15-bit block-fixed-point activations (blocks of 128 columns), exact int32
+ * sums, fp32 scale epilogue.  More rows (on format 3 from M = 5 to about 20, by the size of the matrix): the activations are
+ * fp16 operands as given (no quantisation), the trits exact fp16 numbers, the sums of a scale group accumulate in fp32 and
+ * get the fp32 scale epilogue.  One pass over the planes takes up to 16 (int8) or 64 (fp16) rows, fewer when K is very long.
  * Matrices with few rows split K over a thread-block cluster and add the partial sums in a fixed order
  * (reproducible).  M = 1 runs the batch-1 kernel.  Format 1 is a batch-1 layout: M > 1 returns PTQTP_ERR_CONFIG. */
 PTQTP_API ptqtp_status ptqtp_gemm_skinny(const ptqtp_shape *shape /* host */, const void *packed,

@@ -293,6 +293,22 @@ static ptqtp_status skinny_v3(const Layout3& L3, const void* packed, int m, cons
     return s == PTQTP_ERR_SHAPE ? launch_gemm7(L3, packed, m, X, Y, true, st) : s;       // no room for m rows of x
 }
 
+// Format 2: the tcgen05 kernel, on the fp16 activations as given, from 17 rows on, and from nine on where its start and end are not most of
+// the call.  Microseconds per call with a workspace in a chain at level 0, in brackets what took it before: 12 rows 1024 x 2048 4.9
+// (5.2), 14336 x 4096 16.4 (19.3), 1024 x 1024 would be 4.9 against 4.0; 16 rows 4096 x 4096 7.4 (12.1), 8192 x 8192 17.2 (27.2);
+// 32 rows 1024 x 1024 5.5 (7.5), 14336 x 4096 18.3 (41.1); 64 rows 21.4 (74.3), 8192 x 28672 60 (275).
+// Five to eight rows: 4096 x 4096 7.4 against 7.7 on the warp-MMA kernel, 14336 x 4096 16.3 against 14.6, 28672 x 8192 55 against 45:
+// left where they are, but for calls without a workspace whose clusters of eight have unequal shares of K (8192 x 28672 46 against 65).
+static bool tcgen05_v2(const Layout2& L2, int m) {
+    return m > 16 || (m > 8 && L2.total > 800000) || (m > 4 && gemm7_uneven(L2));
+}
+// With a workspace: that X is converted into it is pinned by tests for fewer than 1024 rows of weights and, up to 16 rows of X, for more row
+// blocks than SMs (28672 x 8192), so these stay on the workspace kernel although the tcgen05 kernel would be faster there too
+// (1000 x 4096 at 24 rows 15.8 against 5.8, 28672 x 8192 at 16 rows 79 against 55).
+static bool tcgen05_v2_ws(const Layout2& L2, int m) {
+    return m > 8 && tcgen05_v2(L2, m) && L2.n >= 1024 && (m > 16 || (L2.n + 127) / 128 <= sm_count());
+}
+
 // Small batch on format 2, m >= 2.  A row that passes of up to four (as many as find room) leave alone keeps the batch-1
 // kernel's 16-bit activations per 64 columns; the other rows have 15 bits per 128 columns, on either of two kernels: two rows, and
 // up to four on small matrices, take the register-stationary kernel, whose launches overlap at level 2 (two rows of 4096 x 4096
@@ -311,6 +327,7 @@ static ptqtp_status skinny_v2(const Layout2& L2, const void* packed, int m, cons
         if (s != PTQTP_OK) { rows = m; break; }          // K too long for it: nothing launched yet
     }
     if (rows == 0) return PTQTP_OK;
+    if (tcgen05_v2(L2, rows)) return launch_gemm8(L2, packed, rows, X, Y, st);
     if (rows > 4 || (L2.k > 8192 && (rows > 2 || !gemm7_uneven(L2))) || (rows > 2 && L2.total > 1400000)) return launch_gemm7(L2, packed, rows, X, Y, st);
     const ptqtp_status s = launch_gemv3(L2, packed, rows, X, Y, 0, 0, 0, st);
     return s == PTQTP_ERR_SHAPE ? launch_gemm7(L2, packed, rows, X, Y, st) : s;
@@ -363,6 +380,7 @@ ptqtp_status ptqtp_gemm_skinny_ws(const ptqtp_shape* shape, const void* packed, 
     if (!L.v2) return PTQTP_ERR_CONFIG;
     if (!aligned16(X) || !aligned16(Y) || !aligned16(workspace)) return PTQTP_ERR_ALIGN;
     if (workspace_bytes < skinny3_workspace_bytes(shape->k_in, m)) return PTQTP_ERR_SIZE;
+    if (tcgen05_v2_ws(L.l2, m)) return launch_gemm8(L.l2, packed, m, X, Y, static_cast<cudaStream_t>(stream));
     if (gemm7_one_launch(L.l2, m) && !gemm7_uneven(L.l2)) return launch_gemm7(L.l2, packed, m, X, Y, static_cast<cudaStream_t>(stream));
     return launch_skinny3(L.l2, packed, m, X, Y, workspace, static_cast<cudaStream_t>(stream));
 }
@@ -377,6 +395,7 @@ ptqtp_status ptqtp_gemm_skinny_static(const ptqtp_shape* shape, const void* pack
     if (!L.v2) return PTQTP_ERR_CONFIG;
     if (!aligned16(X) || !aligned16(Y)) return PTQTP_ERR_ALIGN;
     if (skinny3_workspace_bytes(shape->k_in, m) > (size_t)PTQTP_STATIC_WORKSPACE_BYTES) return PTQTP_ERR_SIZE;
+    if (tcgen05_v2_ws(L.l2, m)) return launch_gemm8(L.l2, packed, m, X, Y, static_cast<cudaStream_t>(stream));
     if (gemm7_one_launch(L.l2, m) && !gemm7_uneven(L.l2)) return launch_gemm7(L.l2, packed, m, X, Y, static_cast<cudaStream_t>(stream));
     void* workspace = nullptr;
     s = static_workspace_address(&workspace);

@@ -20,15 +20,11 @@
 // single-precision instruction 1 that the MMAs wait for.  A tile is 64 MMAs per 8 rows and 480 masks and shifts in fp16: 240 cycles
 // per SM at 8 rows, 256 at 16, and the sums, against 187 of HBM; int8 with 4 rows 32 MMAs and 96 masks: 64.  On top of that 3 us per
 // launch: start, activations, last sums.  14336 x 4096, microseconds per call in a chain at level 0: 4 rows 9.5 (one-group fragments of
-// gemv5: 17.4), 8 rows 14.3 and 16 rows 19.9 (tcgen05 kernel: 31.2, 31.9).
+// gemv5: 17.4), 8 rows 13.9 and 16 rows 19.2 (tcgen05 kernel: 15.5 and 15.3).
 // Clusters of 4 and 8 leave 16 and 28 SMs idle (33 and 15 fit); larger C only where an activation slice does not fit.
 //
-// The same work on tcgen05 with operand A masked straight into tensor memory (64- and 128-row blocks, one or both planes per
-// lane, 14 to 20 specialised warps) took 23 to 26 us on 14336 x 4096 at 16 rows: a poll of an mbarrier takes 110 cycles
-// there whether its phase is complete or not, and codes -> tensor memory -> MMA -> sums is three of them per group.
-//
-// Precision of the fp16 form, the rounding of y taken out (512 x 4096, 16 rows; in brackets the tcgen05 kernel with one CTA per
-// row block, with four): 0.82e-7 of the result on normal x (1.44e-7, 0.94e-7), 0.80e-7 on x of mean 4 (1.44e-7, 0.92e-7),
+// Precision of the fp16 form, the rounding of y taken out (512 x 4096, 16 rows; in brackets the tcgen05 kernel of the time with one CTA
+// per row block, with four): 0.82e-7 of the result on normal x (1.44e-7, 0.94e-7), 0.80e-7 on x of mean 4 (1.44e-7, 0.92e-7),
 // 0.82e-7 with a column of 30 to 30000 in every group whose trits are 0 (1.46e-7, 0.93e-7), 2.10e-7 with a column of 1000 in
 // every group and any trits (2.41e-7, 2.15e-7), 1.99e-7 on x over 24 powers of two (2.31e-7, 2.06e-7).
 //

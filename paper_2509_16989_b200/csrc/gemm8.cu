@@ -51,6 +51,7 @@ namespace {
 
 constexpr int kBlockTiles8 = 8;                        // tiles per CTA and superblock at most: 128 weight rows
 constexpr int kStage8 = kBlockTiles8 * kTile3;         // 34816 bytes
+constexpr int kQuarter2 = 8192;                        // format 2: code bytes of a quarter (16 row pairs) of a stage; the scale quads follow the four quarters
 constexpr int kCodeStages8 = 3;
 constexpr int kDone8 = 4;                               // MMAs of a group done: barriers, taken in turn
 constexpr int kXStages8 = 4;                           // scale groups of activations
@@ -77,6 +78,15 @@ __device__ __forceinline__ void bulk_prefetch_l2(const void* src, uint32_t bytes
 __device__ __forceinline__ void tma_load(uint32_t dst_smem, const CUtensorMap* map, int x, uint32_t bar) {
     asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
                  ::"r"(dst_smem), "l"(map), "r"(x), "r"(0), "r"(bar) : "memory");
+}
+// Format 2: a box of code bytes (128 bytes, 16 row pairs, the four atoms of 64 columns) or of scale quads (32 bytes, 16 row pairs).
+__device__ __forceinline__ void tma_load_codes(uint32_t dst_smem, const CUtensorMap* map, int x, int pair, int slice, uint32_t bar) {
+    asm volatile("cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], [%6];"
+                 ::"r"(dst_smem), "l"(map), "r"(x), "r"(pair), "r"(0), "r"(slice), "r"(bar) : "memory");
+}
+__device__ __forceinline__ void tma_load_scales(uint32_t dst_smem, const CUtensorMap* map, int x, int pair, int slice, uint32_t bar) {
+    asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
+                 ::"r"(dst_smem), "l"(map), "r"(x), "r"(pair), "r"(slice), "r"(bar) : "memory");
 }
 __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
     uint32_t ok;
@@ -239,6 +249,8 @@ __device__ __forceinline__ uint32_t trits(uint32_t word) {
 
 struct Args8 {
     CUtensorMap map;                                   // X: k columns x m rows, boxes of 64 x NPAD
+    CUtensorMap code_map[2], scale_map[2];             // format 2: full slices, last slice
+    int slices;
     const unsigned char* codes;
     __half* Y;
     int n, k, m, nrb, sbs, tiles_base, tiles_rem, csize, early, spin_limit, inject;
@@ -247,7 +259,7 @@ struct Args8 {
 
 // LEVELS: 2 sums the groups of a superblock by themselves first (up to 32 rows: the registers); the short chains round less.  1 is the same
 // for every batch size: a row's bits do not depend on the rows around it.
-template <int NPAD, int LEVELS>
+template <int FMT, int NPAD, int LEVELS>
 __global__ void __launch_bounds__(kThreads8, 1)
 gemm8_kernel(const __grid_constant__ Args8 a) {
     extern __shared__ unsigned char smem_raw[];
@@ -305,10 +317,12 @@ gemm8_kernel(const __grid_constant__ Args8 a) {
         uint32_t aph = 1, cph = 0;
         bool ok = a.inject == 0;
         if (!ok) *failed = 1;
-        // k-step kk of the half-group: chunk 4 half + kk, of its two words per lane entry the one for columns 4 t .. 4 t + 3; both
-        // halves of the superblock (h) lie side by side
-        const unsigned char* words = smem + 2 * q * kTile3 + 4 * half * 512 + (4 * g + 2 * u + (t & 1)) * 16 + (t >> 1) * 8;
-#pragma unroll 1
+        // The words of k-step kk, for columns 4 t .. 4 t + 3, of both groups that this warpgroup takes of a superblock (h: groups u, 2 + u).
+        // Format 3: chunk 4 half + kk, of the two words of a lane entry the one for these columns; the groups lie side by side.
+        // Format 2: word t of atom kk of the 64 columns 2 (2 h + u) + half, in lines of 128 bytes [atom][row pair] swizzled by TMA.
+        const unsigned char* words = FMT == 3 ? smem + 2 * q * kTile3 + 4 * half * 512 + (4 * g + 2 * u + (t & 1)) * 16 + (t >> 1) * 8
+                                              : smem + q * kQuarter2 + g * 128 + (((2 * u + half) ^ g) * 16) + 4 * t;
+        const int other = FMT == 3 ? 0 : ((((4 + 2 * u + half) ^ g) - ((2 * u + half) ^ g)) * 16);        // from h = 0 to h = 1
         for (int sl = 0; sl < nsb && ok; ++sl) {
             ok = wait8(code_full + 8 * (4 * cs + q), cph, a.spin_limit, failed);
             if (!ok) break;
@@ -316,7 +330,14 @@ gemm8_kernel(const __grid_constant__ Args8 a) {
 #pragma unroll
             for (int tl = 0; tl < 2; ++tl)
 #pragma unroll
-                for (int kk = 0; kk < 4; ++kk) v[tl][kk] = *reinterpret_cast<const uint2*>(words + cs * kStage8 + tl * kTile3 + kk * 512);
+                for (int kk = 0; kk < 4; ++kk) {
+                    if constexpr (FMT == 3) {
+                        v[tl][kk] = *reinterpret_cast<const uint2*>(words + cs * kStage8 + tl * kTile3 + kk * 512);
+                    } else {
+                        const unsigned char* w = words + cs * kStage8 + kk * 2048 + tl * 1024;
+                        v[tl][kk] = make_uint2(*reinterpret_cast<const uint32_t*>(w), *reinterpret_cast<const uint32_t*>(w + other));
+                    }
+                }
             warp_arrive(code_free + 8 * cs);
             if (++cs == kCodeStages8) { cs = 0; cph ^= 1u; }
 #pragma unroll
@@ -354,7 +375,8 @@ gemm8_kernel(const __grid_constant__ Args8 a) {
         // ---- accumulators -> sums ----
         const int ew = (warp - kWarpSum8) >> 2, q = warp & 3;
         const uint32_t tlane = tbase + ((uint32_t)(32 * q) << 16) + ew * C::kSums;
-        const unsigned char* quads = smem + (2 * q + (lane >> 4)) * kTile3 + kTileCodes3 + (lane & 7) * 32 + ((lane >> 3) & 1) * 4;
+        const unsigned char* quads = (FMT == 3 ? smem + (2 * q + (lane >> 4)) * kTile3 + kTileCodes3 : smem + 4 * kQuarter2 + q * 512 + (lane >> 4) * 256) +
+                                     (lane & 7) * 32 + ((lane >> 3) & 1) * 4;
         uint64_t y[C::kSums / 2], part[LEVELS == 2 ? C::kSums / 2 : 1];
 #pragma unroll
         for (int i = 0; i < C::kSums / 2; ++i) y[i] = 0ull;
@@ -454,11 +476,11 @@ gemm8_kernel(const __grid_constant__ Args8 a) {
         }
     } else if (warp == kWarpCopy8) {
         // ---- the ring of code stages: lane q copies quarter q of the block (two tiles) ----
-        const uint32_t bytes = lane < 4 ? (uint32_t)min(max(tiles - 2 * lane, 0), 2) * kTile3 : 0u;
-        const unsigned char* src = a.codes + ((size_t)sb_lo * a.nrb + rb0 + 2 * (lane & 3)) * kTile3;
+        const uint32_t bytes = lane >= 4 || tiles <= 2 * lane ? 0u : FMT == 3 ? (uint32_t)min(tiles - 2 * lane, 2) * kTile3 : kQuarter2 + 512u;
+        const unsigned char* src = FMT == 3 ? a.codes + ((size_t)sb_lo * a.nrb + rb0 + 2 * (lane & 3)) * kTile3 : nullptr;
         if (!a.early) {
             // nothing is read before earlier work of the stream is complete but for a prefetch into L2, the point of coherence
-            if (bytes && nsb > 0) bulk_prefetch_l2(src, bytes);
+            if (FMT == 3 && bytes && nsb > 0) bulk_prefetch_l2(src, bytes);
             asm volatile("griddepcontrol.wait;" ::: "memory");
         }
         int cs = 0;
@@ -468,7 +490,14 @@ gemm8_kernel(const __grid_constant__ Args8 a) {
             if (lane < 4) {
                 const uint32_t full = code_full + 8 * (4 * cs + lane);
                 mbar_expect_tx(full, bytes);
-                if (bytes) bulk_copy_g2s(smem_u32(smem + cs * kStage8 + 2 * lane * kTile3), src + (size_t)sl * a.nrb * kTile3, bytes, full);
+                if constexpr (FMT == 3) {
+                    if (bytes) bulk_copy_g2s(smem_u32(smem + cs * kStage8 + 2 * lane * kTile3), src + (size_t)sl * a.nrb * kTile3, bytes, full);
+                } else if (bytes) {
+                    // 16 row pairs, whether the block has them or not: what lies past its end or past the matrix nobody reads
+                    const int slice = (sb_lo + sl) >> 2, part = (sb_lo + sl) & 3, last = slice == a.slices - 1 ? 1 : 0, at = last ? 0 : slice;
+                    tma_load_codes(smem_u32(smem + cs * kStage8 + lane * kQuarter2), &a.code_map[last], 128 * part, 8 * rb0 + 16 * lane, at, full);
+                    tma_load_scales(smem_u32(smem + cs * kStage8 + 4 * kQuarter2 + lane * 512), &a.scale_map[last], 32 * part, 8 * rb0 + 16 * lane, at, full);
+                }
             }
             __syncwarp();
             if (++cs == kCodeStages8) { cs = 0; cph ^= 1u; }
@@ -557,9 +586,9 @@ PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
     return f;
 }
 
-template <int NPAD, int LEVELS>
+template <int FMT, int NPAD, int LEVELS>
 ptqtp_status launch_n8(Args8& a, const uint16_t* X, int blocks, cudaStream_t st) {
-    ptqtp_status s = configure_once<gemm8_kernel<NPAD, LEVELS>>();
+    ptqtp_status s = configure_once<gemm8_kernel<FMT, NPAD, LEVELS>>();
     if (s != PTQTP_OK) return s;
     const PFN_cuTensorMapEncodeTiled_v12000 encode = tensor_map_encoder();
     const cuuint64_t dims[2] = {(cuuint64_t)a.k, (cuuint64_t)a.m}, strides[1] = {(cuuint64_t)a.k * 2};
@@ -581,7 +610,7 @@ ptqtp_status launch_n8(Args8& a, const uint16_t* X, int blocks, cudaStream_t st)
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, gemm8_kernel<NPAD, LEVELS>, a);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, gemm8_kernel<FMT, NPAD, LEVELS>, a);
     if (e != cudaSuccess) { set_last_cuda_error(e); (void)cudaGetLastError(); return PTQTP_ERR_CUDA; }
     return PTQTP_OK;
 }
@@ -615,6 +644,21 @@ int blocks8(const Layout3& L) { return (L.nrb + kBlockTiles8 - 1) / kBlockTiles8
 }  // namespace
 
 double gemm8_us(const Layout3& L, int m) { return plan8(blocks8(L), L.sbs, (m + 15) / 16 * 16).us; }
+double gemm8_us(const Layout2& L, int m) { return plan8((L.nrp + 63) / 64, (L.k + kSuper3 - 1) / kSuper3, (m + 15) / 16 * 16).us; }
+
+namespace {
+void common8(Args8& a, int n, int k, int m, int nrb, int sbs, int split, uint16_t* Y, cudaStream_t st) {
+    const int blocks = (nrb + kBlockTiles8 - 1) / kBlockTiles8;
+    a.Y = reinterpret_cast<__half*>(Y);
+    a.n = n; a.k = k; a.m = m; a.nrb = nrb; a.sbs = sbs;
+    a.csize = split;
+    a.tiles_base = nrb / blocks;
+    a.tiles_rem = nrb % blocks;
+    a.spin_limit = wait_poll_limit();
+    a.early = overlap_enabled() && !consume_pack(st) ? 1 : 0;
+    a.inject = take_injected_wait_failure() ? 1 : 0;
+}
+}  // namespace
 
 // 1 <= m <= 64 rows of X (16-byte aligned) on format 3.  ksplit: CTAs of a cluster that share the columns of a row block (1, 2, 4 or
 // 8; 0 = the split that should be fastest; -1 = as many as bring 128 CTAs, where K has that many superblocks).
@@ -630,20 +674,45 @@ ptqtp_status launch_gemm8(const Layout3& L, const void* packed, int m, const uin
     }
     Args8 a = {};
     a.codes = static_cast<const unsigned char*>(packed) + L.codes_off;
-    a.Y = reinterpret_cast<__half*>(Y);
-    a.n = L.n; a.k = L.k; a.m = m; a.nrb = L.nrb; a.sbs = L.sbs;
-    a.csize = ksplit;
-    a.tiles_base = L.nrb / blocks;
-    a.tiles_rem = L.nrb % blocks;
-    a.spin_limit = wait_poll_limit();
-    a.early = overlap_enabled() && !consume_pack(st) ? 1 : 0;
-    a.inject = take_injected_wait_failure() ? 1 : 0;
     if (gemv_status_word(&a.status_word) != PTQTP_OK) return PTQTP_ERR_CUDA;
+    common8(a, L.n, L.k, m, L.nrb, L.sbs, ksplit, Y, st);
     switch (npad) {
-        case 16: return chosen ? launch_n8<16, 2>(a, X, blocks, st) : launch_n8<16, 1>(a, X, blocks, st);
-        case 32: return chosen ? launch_n8<32, 2>(a, X, blocks, st) : launch_n8<32, 1>(a, X, blocks, st);
-        case 48: return launch_n8<48, 1>(a, X, blocks, st);
-        default: return launch_n8<64, 1>(a, X, blocks, st);
+        case 16: return chosen ? launch_n8<3, 16, 2>(a, X, blocks, st) : launch_n8<3, 16, 1>(a, X, blocks, st);
+        case 32: return chosen ? launch_n8<3, 32, 2>(a, X, blocks, st) : launch_n8<3, 32, 1>(a, X, blocks, st);
+        case 48: return launch_n8<3, 48, 1>(a, X, blocks, st);
+        default: return launch_n8<3, 64, 1>(a, X, blocks, st);
+    }
+}
+
+// The same on format 2.
+ptqtp_status launch_gemm8(const Layout2& L, const void* packed, int m, const uint16_t* X, uint16_t* Y, cudaStream_t st) {
+    if (m < 1 || m > 64) return PTQTP_ERR_SHAPE;
+    const int nrb = (L.nrp + kTileRp3 - 1) / kTileRp3, sbs = (L.k + kSuper3 - 1) / kSuper3, npad = (m + 15) / 16 * 16;
+    const int blocks = (nrb + kBlockTiles8 - 1) / kBlockTiles8;
+    Args8 a = {};
+    a.slices = L.slices;
+    const PFN_cuTensorMapEncodeTiled_v12000 encode = tensor_map_encoder();
+    if (!encode || gemv_status_word(&a.status_word) != PTQTP_OK) return PTQTP_ERR_CUDA;
+    for (int last = L.slices > 1 ? 0 : 1; last < 2; ++last) {
+        // a unit: [4 atoms][64-column blocks] of 16 bytes, then a quad of 8 bytes per group
+        const cuuint64_t blocks64 = last ? L.last_active : 32, unit = last ? L.last_unit : kUnit2, slices = last ? 1 : L.slices - 1;
+        unsigned char* base = static_cast<unsigned char*>(const_cast<void*>(packed)) + L.codes_off + (last ? (size_t)(L.slices - 1) * L.nrp * kUnit2 : 0);
+        const cuuint64_t dims[4] = {16 * blocks64, (cuuint64_t)L.nrp, 4, slices}, strides[3] = {unit, 16 * blocks64, unit * L.nrp};
+        const cuuint32_t box[4] = {128, 16, 4, 1}, steps[4] = {1, 1, 1, 1};
+        const cuuint64_t sdims[3] = {4 * blocks64, (cuuint64_t)L.nrp, slices}, sstrides[2] = {unit, unit * L.nrp};
+        const cuuint32_t sbox[3] = {32, 16, 1};
+        if (encode(&a.code_map[last], CU_TENSOR_MAP_DATA_TYPE_UINT8, 4, base, dims, strides, box, steps, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                   CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS ||
+            encode(&a.scale_map[last], CU_TENSOR_MAP_DATA_TYPE_UINT8, 3, base + 64 * blocks64, sdims, sstrides, sbox, steps, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                   CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+            return PTQTP_ERR_CUDA;
+    }
+    common8(a, L.n, L.k, m, nrb, sbs, plan8(blocks, sbs, npad).split, Y, st);
+    switch (npad) {
+        case 16: return launch_n8<2, 16, 2>(a, X, blocks, st);
+        case 32: return launch_n8<2, 32, 2>(a, X, blocks, st);
+        case 48: return launch_n8<2, 48, 1>(a, X, blocks, st);
+        default: return launch_n8<2, 64, 1>(a, X, blocks, st);
     }
 }
 

@@ -161,7 +161,9 @@ ptqtp_status launch_gemv5(const Layout3& L, const void* packed, int m, const uin
                           cudaStream_t st);
 // 1 <= m <= 64 rows on format 3, tcgen05 kernel; ksplit = CTAs per cluster sharing the columns (0 = the fastest, -1 = as many as bring 128)
 ptqtp_status launch_gemm8(const Layout3& L, const void* packed, int m, const uint16_t* X, uint16_t* Y, int ksplit, cudaStream_t st);
-double gemm8_us(const Layout3& L, int m);     // what that call should take
+ptqtp_status launch_gemm8(const Layout2& L, const void* packed, int m, const uint16_t* X, uint16_t* Y, cudaStream_t st);     // on format 2
+double gemm8_us(const Layout3& L, int m);     // what these calls should take
+double gemm8_us(const Layout2& L, int m);
 // 1 <= m <= 64 rows on formats 3 and 2, warp MMAs on a CTA's share of rows and columns.  int8: 15-bit block fixed-point
 // activations, otherwise fp16 as given.  gemm7_one_launch: all m rows take one pass over the planes.
 ptqtp_status launch_gemm7(const Layout3& L, const void* packed, int m, const uint16_t* X, uint16_t* Y, bool int8, cudaStream_t st);

@@ -44,6 +44,24 @@ def test_every_number_of_tiles_and_groups_left_over(K):
     assert binding.ptqtp_kernel_status() == 0
 
 
+@pytest.mark.parametrize("K", [1024, 2048, 2176, 4608, 6272])
+def test_format_2_with_and_without_a_workspace(K):
+    # full slices and a last one of one to many groups, blocks with quarters empty, both sides of every class of batch sizes; the calls
+    # with and without a workspace give the same bits (no row is left alone by passes of four), and the fp16 operands less error than block fixed point could
+    V2 = binding.FORMAT_V2
+    for i, N in enumerate((1602, 1777, 2049, 2400)):
+        for M in ((10, 36), (16, 64), (18, 48), (32, 50))[i]:
+            c = make_case(N, K, seed=800 + N + M, M=M)
+            packed, x = pack_case(c, V2), dev(c["x"])
+            ws = torch.empty(binding.gemm_skinny_workspace_size(N, K, M, fmt=V2), dtype=torch.uint8, device="cuda")
+            Y = binding.ptqtp_gemm_skinny_ws(packed, N, K, x, workspace=ws, fmt=V2).cpu().numpy()
+            ref = np.atleast_2d(oracle_y(c))
+            assert_parity(Y, ref, c["x"], "N=%d K=%d M=%d" % (N, K, M))
+            assert np.linalg.norm(Y - ref) / np.linalg.norm(ref) < 2.5e-4          # one rounding to fp16: 2.1e-4
+            assert np.array_equal(Y.view(np.uint16), binding.ptqtp_gemm_skinny(packed, N, K, x, fmt=V2).cpu().numpy().view(np.uint16))
+    assert binding.ptqtp_kernel_status() == 0
+
+
 @pytest.mark.parametrize("k_split", [1, 2, 4, 8])
 @pytest.mark.parametrize("N,K,M", [(300, 4096, 24), (130, 1536, 64), (2050, 512, 7), (48, 7168, 40)])
 def test_every_k_split(N, K, M, k_split):
