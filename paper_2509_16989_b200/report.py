@@ -145,7 +145,7 @@ def config2(T):
              us_per_batch_row=round(us / M, 3), gbs=round(nb / us / 1e3, 1), bytes=nb)
     del bufs
     torch.cuda.empty_cache()
-    # the same sweep on format 3 (M = 2..7: warp-MMA passes of four rows; M >= 8: the tcgen05 kernel), every 8B shape
+    # the same sweep on format 3 (warp MMAs up to 8 to 32 rows by the size, then the tcgen05 kernel), every 8B shape
     for name in ("gate", "down", "q", "k"):
         N, K = LLAMA3_8B[name]
         c = make_case(N, K, seed=2, M=64)
