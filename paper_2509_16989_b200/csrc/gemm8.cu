@@ -1,5 +1,5 @@
-// Dual-trit-plane layer for up to 64 activation rows per launch on packed format 3 (the batch-1 layout), on the fifth-generation
-// tensor cores (tcgen05.mma, operand A and accumulators in tensor memory):
+// Dual-trit-plane layer for up to 64 activation rows per launch on packed formats 3 and 2, on the fifth-generation tensor cores
+// (tcgen05.mma, operand A and accumulators in tensor memory):
 //     Y[m] = alpha1 (.) (T1 X[m]) + alpha2 (.) (T2 X[m]),   m < M <= 64.
 //
 // A CTA owns up to 128 weight rows (8 tiles per superblock, contiguous in the blob); a row is a lane of every MMA.  Per scale group
@@ -14,6 +14,9 @@
 //     columns each.
 //   * one warp copies the codes (bulk copies, a superblock at a time, four barriers so that the first quarter can start alone), one the
 //     activations (TMA, 128-byte swizzle, rows past M as zeros), fp16 as given.
+// Format 2 differs in the copies and in where a word lies: two tensor maps for the code bytes and two for the scale quads (full slices, the last
+// slice) bring the same 512 columns of 128 rows by TMA, as lines of 128 bytes [atom][row pair] whose swizzle spreads the eight row
+// pairs that a warp reads over the banks (14336 x 4096 with a workspace at 16, 32, 64 rows: 16.4, 18.3, 21.4 us; before 23.0, 41.1, 74.3).
 // Matrices with few rows split K over a cluster of up to 8 CTAs; every rank copies its partial sums (bulk copies between the
 // shared memories, counted on the receiver's mbarrier) to the rank that owns the columns, which adds them in rank order: no
 // atomics, no workspace, reproducible.
