@@ -309,8 +309,10 @@ gemm8_kernel(const __grid_constant__ Args8 a) {
     auto group_done = [&](int g) { return wait8(done + 8 * (g % kDone8), (uint32_t)(g / kDone8) & 1u, a.spin_limit, failed); };
     if (a.csize > 1) cluster_arrive();                   // awaited before the first store into another rank
     const int rows = min(16 * tiles, a.n - 16 * rb0);
+    // One warp of a CTA releases the next launch for all of it.  The copying warp, which has not waited yet, does so only where launches
+    // may overlap; otherwise the next kernel starts when everything before this one is complete, as after a plain launch.
     if (warp != kWarpCopy8) asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;");
+    if (warp != kWarpCopy8 || a.early) asm volatile("griddepcontrol.launch_dependents;");
 
     if (warp < kDecoders8) {
         // ---- codes -> trits in tensor memory ----

@@ -1,11 +1,15 @@
 """Stream order of the small-batch kernels, which are launched as dependents of one another at every overlap level: chains in
 which every call reads what the call before it wrote, blobs written directly ahead of a call, the workspace and the output
 shared by consecutive calls.  All results are compared bit for bit with synchronised calls."""
+import ctypes
+import os
+import subprocess
+
 import numpy as np
 import pytest
 import torch
 
-from paper_2509_16989_b200 import binding
+from paper_2509_16989_b200 import binding, build
 from paper_2509_16989_b200.inputs import make_case
 from gpu_util import assert_parity, dev, oracle_y, pack_case
 
@@ -38,6 +42,19 @@ def layers():
             c[a] = (c[a].astype(np.float32) * 1.28).astype(np.float16)
         out.append({V2: pack_case(c, V2), V3: pack_case(c, V3)})
     return out
+
+
+@pytest.fixture(scope="module")
+def neighbours(tmp_path_factory):
+    """The kernels of dependent_launch.cu."""
+    src = os.path.join(os.path.dirname(os.path.abspath(__file__)), "dependent_launch.cu")
+    out = str(tmp_path_factory.mktemp("native") / "dependent_launch.so")
+    subprocess.run([build._nvcc()] + build.NVCC_FLAGS + [src, "-o", out], check=True)
+    lib = ctypes.CDLL(out)
+    vp = ctypes.c_void_p
+    lib.run_late_writer.argtypes = [vp, ctypes.c_int, ctypes.c_longlong, vp]
+    lib.run_early_reader.argtypes = [vp, vp, vp]
+    return lib
 
 
 @pytest.fixture(autouse=True)
@@ -182,3 +199,67 @@ def test_small_batch_behind_batch_1_and_back(layers, level):
     binding.ptqtp_set_overlap(level)
     for (name, Y, z), (_, Yw, zw) in zip(run(False), want):
         assert np.array_equal(Y, Yw) and np.array_equal(z, zw), name
+
+
+@pytest.mark.parametrize("level", [0, 1, 2])
+@pytest.mark.parametrize("M", [2, 5, 6, 24])
+def test_a_call_in_stream_order_releases_the_next_kernel_after_all_that_came_before(layers, neighbours, M, level):
+    # level 0, and the call after a pack at levels 1 and 2: a kernel behind the call that reads without waiting sees what a kernel ahead
+    # of the call writes late, although that one released its dependents at once
+    X = dev(make_case(N, K, seed=58, M=M)["x"])
+    Y = torch.empty((M, N), dtype=torch.float16, device="cuda")
+    ws = torch.empty(binding.gemm_skinny_workspace_size(N, K, M, fmt=V2), dtype=torch.uint8, device="cuda")
+    c = make_case(16, 128, seed=59)
+    planes = tuple(dev(c[k]) for k in ("T1", "T2", "alpha1", "alpha2"))
+    small = torch.empty(binding.packed_size(16, 128, fmt=V3), dtype=torch.uint8, device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    word, seen = (torch.zeros(64, dtype=torch.int32, device="cuda") for _ in range(2))
+    stream = torch.cuda.Stream()
+    for name, (fmt, call) in FORMS.items():
+        with torch.cuda.stream(stream):
+            call(layers[0][fmt], X, Y, ws)               # loads the kernels
+            binding.ptqtp_set_overlap(level)
+            for i in range(4):
+                stream.synchronize()
+                if level:
+                    binding.ptqtp_pack(*planes, packed=small, dev_status=status, fmt=V3)
+                assert neighbours.run_late_writer(word.data_ptr(), i + 1, 200_000, stream.cuda_stream) == 0
+                call(layers[0][fmt], X, Y, ws)
+                assert neighbours.run_early_reader(word.data_ptr(), seen.data_ptr() + 4 * i, stream.cuda_stream) == 0
+            stream.synchronize()
+            binding.ptqtp_set_overlap(0)
+        assert seen[:4].tolist() == [1, 2, 3, 4], name
+    assert binding.ptqtp_kernel_status() == 0
+
+
+@pytest.mark.parametrize("level", [0, 1, 2])
+@pytest.mark.parametrize("M", [5, 24])
+def test_two_blobs_packed_directly_before_two_calls(M, level):
+    # the second call reads a blob whose pack is two kernels ahead of it
+    cs = [make_case(N, K, seed=60 + i, M=M) for i in range(2)]
+    X = dev(cs[0]["x"])
+    planes = [tuple(dev(c[k]) for k in ("T1", "T2", "alpha1", "alpha2")) for c in cs]
+    ws = torch.empty(binding.gemm_skinny_workspace_size(N, K, M, fmt=V2), dtype=torch.uint8, device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    want = {}
+    for name, (fmt, call) in FORMS.items():
+        for i in range(2):
+            y = torch.empty((M, N), dtype=torch.float16, device="cuda")
+            call(binding.ptqtp_pack(*planes[i], fmt=fmt)[0], X, y, ws)
+            want[name, i] = bits(y)
+    binding.ptqtp_set_overlap(level)
+    for a, (fmt_a, call_a) in FORMS.items():
+        for b, (fmt_b, call_b) in FORMS.items():
+            blobs = [torch.empty(binding.packed_size(N, K, fmt=f), dtype=torch.uint8, device="cuda") for f in (fmt_a, fmt_b)]
+            ys = [torch.empty((M, N), dtype=torch.float16, device="cuda") for _ in range(8)]
+            torch.cuda.synchronize()
+            for i in range(4):
+                binding.ptqtp_pack(*planes[i % 2], packed=blobs[0], dev_status=status, fmt=fmt_a)
+                binding.ptqtp_pack(*planes[(i + 1) % 2], packed=blobs[1], dev_status=status, fmt=fmt_b)
+                call_a(blobs[0], X, ys[2 * i], ws)
+                call_b(blobs[1], X, ys[2 * i + 1], ws)
+            torch.cuda.synchronize()
+            for i in range(4):
+                assert np.array_equal(bits(ys[2 * i]), want[a, i % 2]), (a, b, i)
+                assert np.array_equal(bits(ys[2 * i + 1]), want[b, (i + 1) % 2]), (a, b, i)
+    assert int(status.item()) == 0
