@@ -438,7 +438,10 @@ gemm8_kernel(const __grid_constant__ Args8 a) {
 #pragma unroll
             for (int i = 0; i < C::kSums / 2; ++i) y[i] = 0x7fc000007fc00000ull;
         }
-        // [column][row] over the code stages: every group is summed, so all of them have been read
+        // [column][row] over the first code stage.  The last group's MMAs follow from every decoder's words, so these have been read, but of the
+        // scales only those of superblocks whose first group is two groups back (two sets of accumulators): a last superblock of one or
+        // two groups may be entered by the other summing warps only now.  Nobody stores before all of them are through.
+        asm volatile("bar.sync 1, %0;" ::"n"(32 * kSummers8) : "memory");
         float* dst = reinterpret_cast<float*>(smem) + ew * C::kSums * 128 + 32 * q + 16 * (lane >> 4) + 2 * (lane & 7) + ((lane >> 3) & 1);
 #pragma unroll
         for (int i = 0; i < C::kSums; i += 2) {

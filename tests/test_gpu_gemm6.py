@@ -44,6 +44,22 @@ def test_every_number_of_tiles_and_groups_left_over(K):
     assert binding.ptqtp_kernel_status() == 0
 
 
+@pytest.mark.parametrize("K,k_split", [(128, 1), (256, 1), (640, 2), (1664, 1), (1792, -1), (3200, 1), (3840, 2), (6272, 1), (7808, 4)])
+def test_partial_sums_over_a_last_superblock_of_one_or_two_groups(K, k_split):
+    # the partial sums are written where the codes and scales of superblocks 0, 3, 6, ... of a CTA were: a CTA whose last superblock is one
+    # of these and has one or two groups; many row blocks, the same bits every time, rows and scales so different that one taken for
+    # another shows
+    N = 4100
+    for M in (5, 16, 33, 64):
+        c = make_case(N, K, seed=700 + K + M, M=M)
+        c["alpha1"] = (c["alpha1"].astype(np.float32) * np.exp2(np.arange(N) % 5)[:, None]).astype(np.float16)
+        packed, x = pack_case(c, V3), dev(c["x"])
+        Y = [binding.ptqtp_gemm_skinny_cfg(packed, N, K, x, path=6, k_split=k_split) for _ in range(40)]
+        assert all(torch.equal(Y[0].view(torch.int16), y.view(torch.int16)) for y in Y[1:])
+        assert_parity(Y[0].cpu().numpy(), oracle_y(c), c["x"], "K=%d M=%d split %d" % (K, M, k_split))
+    assert binding.ptqtp_kernel_status() == 0
+
+
 @pytest.mark.parametrize("K", [1024, 2048, 2176, 4608, 6272])
 def test_format_2_with_and_without_a_workspace(K):
     # full slices and a last one of one to many groups, blocks with quarters empty, both sides of every class of batch sizes; the calls
