@@ -494,6 +494,8 @@ gemm8_kernel(const __grid_constant__ Args8 a) {
         int cs = 0;
         uint32_t cph = 1;
         for (int sl = 0; sl < nsb; ++sl) {
+            // past the first round of the ring a stage is freed by warps that wait for the kernel ahead: its time is not for the polls to count
+            if (a.early && sl == kCodeStages8) asm volatile("griddepcontrol.wait;" ::: "memory");
             if (!wait8(code_free + 8 * cs, cph, a.spin_limit, failed)) break;
             if (lane < 4) {
                 const uint32_t full = code_full + 8 * (4 * cs + lane);
@@ -510,7 +512,7 @@ gemm8_kernel(const __grid_constant__ Args8 a) {
             __syncwarp();
             if (++cs == kCodeStages8) { cs = 0; cph ^= 1u; }
         }
-        if (a.early) asm volatile("griddepcontrol.wait;" ::: "memory");
+        if (a.early && nsb <= kCodeStages8) asm volatile("griddepcontrol.wait;" ::: "memory");
     } else {
         // ---- activations, a scale group of all rows at a time ----
         int xs = 0;

@@ -263,3 +263,43 @@ def test_two_blobs_packed_directly_before_two_calls(M, level):
                 assert np.array_equal(bits(ys[2 * i]), want[a, i % 2]), (a, b, i)
                 assert np.array_equal(bits(ys[2 * i + 1]), want[b, (i + 1) % 2]), (a, b, i)
     assert int(status.item()) == 0
+
+
+@pytest.mark.parametrize("level", [0, 1, 2])
+@pytest.mark.parametrize("form", ["format 3", "format 2"])
+def test_polls_of_the_tcgen05_kernel_do_not_count_the_time_of_the_kernel_ahead(neighbours, form, level):
+    # a kernel ahead that releases its dependents at once and works for longer than the polls of a wait last (a launch alone is healthy
+    # with 16; 256 run out within these 30 ms); more superblocks per CTA than the ring of codes has stages
+    n, k, M = (300, 8192, 24) if form == "format 3" else (2048, 16384, 24)
+    c = make_case(n, k, seed=61, M=M)
+    packed, X = pack_case(c, V3 if form == "format 3" else V2), dev(c["x"])
+    Y = torch.empty((M, n), dtype=torch.float16, device="cuda")
+    word = torch.zeros(1, dtype=torch.int32, device="cuda")
+    stream = torch.cuda.Stream()
+
+    def call():
+        if form == "format 3":
+            binding.ptqtp_gemm_skinny_cfg(packed, n, k, X, Y=Y, path=6, k_split=1)
+        else:
+            binding.ptqtp_gemm_skinny(packed, n, k, X, Y=Y, fmt=V2)
+
+    binding.ptqtp_kernel_status_clear()
+    with torch.cuda.stream(stream):
+        call()
+        stream.synchronize()
+        want = bits(Y)
+        Y.zero_()
+        binding.ptqtp_set_overlap(level)
+        old = binding.ptqtp_set_wait_limit(256)
+        try:
+            stream.synchronize()
+            assert neighbours.run_late_writer(word.data_ptr(), 1, 30_000_000, stream.cuda_stream) == 0
+            call()
+            stream.synchronize()
+        finally:
+            binding.ptqtp_set_wait_limit(old)
+    assert word.item() == 1
+    status = binding.ptqtp_kernel_status()
+    binding.ptqtp_kernel_status_clear()
+    assert status == 0 and np.array_equal(bits(Y), want)
+    assert_parity(Y.cpu().numpy(), oracle_y(c), c["x"], form)
