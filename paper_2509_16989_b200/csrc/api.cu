@@ -265,13 +265,17 @@ static bool fp16_activations(const Layout3& L3, int m) {
 //   8 rows: always warp MMAs (14336 x 4096 13.9 and 15.5, 4096 x 14336 14.8 and 15.2, 4096 x 4096 6.0 and 7.5).
 //   9 to 16 rows: warp MMAs take about 4.2 us and 0.445 per MB whatever the shape (1024 x 4096 4.9, 3072 x 3072 6.7, 4096 x 4096 8.2,
 //   6144 x 6144 12.7, 14336 x 4096 19.2, 20480 x 6144 32.5), the tcgen05 kernel what its waves of CTAs take (5.2, 6.9, 7.5, 13.1, 15.6, 38.6).
-//   17 to 32 rows: tcgen05 but for small matrices, where its start and end are most of the call (1024 x 2048 at 24 and 32 rows 5.0 and
-//   5.0 against 5.3 and 5.4, 1024 x 4096 5.4 and 6.4 against 5.7 and 5.8, 2048 x 2048 5.9 and 7.0 against 5.4 and 5.4; 14336 x 4096
-//   33.2 against 17.3).  More rows: always tcgen05.
+//   17 to 32 rows: the one that takes less time.  Small matrices, where the tcgen05 kernel's start and end are most of the call, stay with
+//   the warp MMAs (1024 x 2048 at 24 and 32 rows 5.0 and 5.0 against 5.3 and 5.4, 1024 x 4096 5.4 and 6.4 against 5.7 and 5.8), and
+//   so do matrices whose superblocks find no even split or whose last wave is nearly empty (18 rows: 2048 x 1536 5.0 against 6.8, 4096 x
+//   1024 4.6 against 5.5, 5003 x 512 4.1 against 5.2, 20480 x 512 8.6 against 10.0); 14336 x 4096 33.2 against 17.3.  Over 603
+//   calls beside the first line the slower kernel is taken 20 times where it costs more than 3 % (11 % at most; with that line alone
+//   66 times, 36 %).  More rows: always tcgen05.
 static bool warp_mmas_for_fp16(const Layout3& L3, int m) {
     if (m <= 8) return true;
-    if (m <= 16) return gemm8_us(L3, m) > 4.2 + 0.445 * 1e-6 * (double)L3.total;
-    return m <= 24 ? L3.total < 2300000 && L3.n < 2048 : m <= 32 && L3.total < 1300000;
+    if (m <= 16) return gemm8_plan_us(L3, m) > 4.2 + 0.445 * 1e-6 * (double)L3.total;
+    if (m > 32) return false;
+    return (m <= 24 ? L3.total < 2300000 && L3.n < 2048 : L3.total < 1300000) || gemm7_us(L3, m) < gemm8_us(L3, m);
 }
 // Kernels, in microseconds per call in a chain of its kind at overlap level 0 (14336 x 4096, 4096 x 14336, 4096 x 4096, 1024 x 4096):
 //   int8: four rows 9.5, 10.4, 5.4, 3.6 on the warp-MMA kernel, 17.4, 28.3, 7.6, 5.7 on the batch-1 tiles kernel, whose launches
@@ -293,14 +297,18 @@ static ptqtp_status skinny_v3(const Layout3& L3, const void* packed, int m, cons
     return s == PTQTP_ERR_SHAPE ? launch_gemm7(L3, packed, m, X, Y, true, st) : s;       // no room for m rows of x
 }
 
-// Format 2: the tcgen05 kernel, on the fp16 activations as given, from 17 rows on, and from nine on where its start and end are not most of
-// the call.  Microseconds per call with a workspace in a chain at level 0, in brackets what took it before: 12 rows 1024 x 2048 4.9
-// (5.2), 14336 x 4096 16.4 (19.3), 1024 x 1024 would be 4.9 against 4.0; 16 rows 4096 x 4096 7.4 (12.1), 8192 x 8192 17.2 (27.2);
-// 32 rows 1024 x 1024 5.5 (7.5), 14336 x 4096 18.3 (41.1); 64 rows 21.4 (74.3), 8192 x 28672 60 (275).
+// Format 2: the tcgen05 kernel, on the fp16 activations as given, from 17 rows on, and from nine on where it takes less time than the warp
+// MMAs and more than its start and end.  Microseconds per call with a workspace in a chain at level 0, in brackets what takes it
+// otherwise: 12 rows 1024 x 2048 4.9 (5.2), 14336 x 4096 16.4 (19.3), 1024 x 1024 would be 4.9 against 4.0; 16 rows 4096 x 4096 7.4 (12.1),
+// 8192 x 8192 17.2 (27.2); 32 rows 1024 x 1024 5.5 (7.5), 14336 x 4096 18.3 (41.1); 64 rows 21.4 (74.3), 8192 x 28672 60 (275).
+// Three superblocks over two CTAs, a second wave of a few blocks and few rows of many columns stay with the warp MMAs (10 rows: 1024 x
+// 1536 4.5 against 6.2, 20480 x 2048 14.5 against 20.1, 128 x 28672 9.1 against 13.5).  Over 961 calls of 9 to 16 rows the slower kernel
+// is taken 16 times where it costs more than 3 % (12 % at most; by the bytes alone 125 times, 47 %).
 // Five to eight rows: 4096 x 4096 7.4 against 7.7 on the warp-MMA kernel, 14336 x 4096 16.3 against 14.6, 28672 x 8192 55 against 45:
 // left where they are, but for calls without a workspace whose clusters of eight have unequal shares of K (8192 x 28672 46 against 65).
 static bool tcgen05_v2(const Layout2& L2, int m) {
-    return m > 16 || (m > 8 && L2.total > 800000) || (m > 4 && gemm7_uneven(L2));
+    if (m > 16) return true;
+    return ((m > 8 && L2.total > 800000) || (m > 4 && gemm7_uneven(L2))) && gemm8_us(L2, m) < gemm7_us(L2, m);
 }
 // With a workspace: that X is converted into it is pinned by tests for fewer than 1024 rows of weights and, up to 16 rows of X, for more row
 // blocks than SMs (28672 x 8192), so these stay on the workspace kernel although the tcgen05 kernel would be faster there too

@@ -162,7 +162,8 @@ ptqtp_status launch_gemv5(const Layout3& L, const void* packed, int m, const uin
 // 1 <= m <= 64 rows on format 3, tcgen05 kernel; ksplit = CTAs per cluster sharing the columns (0 = the fastest, -1 = as many as bring 128)
 ptqtp_status launch_gemm8(const Layout3& L, const void* packed, int m, const uint16_t* X, uint16_t* Y, int ksplit, cudaStream_t st);
 ptqtp_status launch_gemm8(const Layout2& L, const void* packed, int m, const uint16_t* X, uint16_t* Y, cudaStream_t st);     // on format 2
-double gemm8_us(const Layout3& L, int m);     // what these calls should take
+double gemm8_plan_us(const Layout3& L, int m);     // what its plan reckons with
+double gemm8_us(const Layout3& L, int m);     // what these calls take, up to 32 rows
 double gemm8_us(const Layout2& L, int m);
 // 1 <= m <= 64 rows on formats 3 and 2, warp MMAs on a CTA's share of rows and columns.  int8: 15-bit block fixed-point
 // activations, otherwise fp16 as given.  gemm7_one_launch: all m rows take one pass over the planes.
@@ -170,6 +171,8 @@ ptqtp_status launch_gemm7(const Layout3& L, const void* packed, int m, const uin
 ptqtp_status launch_gemm7(const Layout2& L, const void* packed, int m, const uint16_t* X, uint16_t* Y, cudaStream_t st);
 bool gemm7_one_launch(const Layout3& L, int m, bool int8);
 bool gemm7_one_launch(const Layout2& L, int m);
+double gemm7_us(const Layout3& L, int m);     // what these calls take: fp16, 17 to 32 rows in one launch
+double gemm7_us(const Layout2& L, int m);     // 9 to 16 rows
 bool gemm7_uneven(const Layout2& L);          // its clusters of eight CTAs have unequal shares of K
 size_t decompose_workspace_bytes(long long rows, int t_max);
 void decompose_offsets(long long rows, int t_max, size_t* delta_off, size_t* err_off, size_t* a1_off, size_t* a2_off,

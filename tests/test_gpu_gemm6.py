@@ -1,4 +1,4 @@
-"""GPU parity of the tcgen05 small-batch kernel on format 3 (fp16 trits from tensor memory against fp16
+"""GPU parity of the tcgen05 small-batch kernel on formats 3 and 2 (fp16 trits from tensor memory against fp16
 activations, fp32 accumulators in tensor memory) against the fp64 oracle: ragged shapes, every batch size class,
 every K split of a cluster, exact integer cases, the library's dispatch and the give-up path of its bounded waits."""
 import numpy as np
@@ -22,7 +22,7 @@ def _run(c, packed, N, K, **kw):
 @pytest.mark.parametrize("N,K,M", [(1, 128, 2), (5, 256, 5), (7, 1152, 16), (33, 2048, 17), (130, 3200, 31),
                                    (257, 5120, 32), (64, 14336, 33), (1000, 6144, 48), (37, 36864, 49),
                                    (192, 3072, 64), (2400, 4096, 9), (129, 640, 2), (255, 512, 64), (256, 384, 20)])
-@pytest.mark.parametrize("k_split", [0, -1])             # 0: up to 32 rows the warp-MMA kernel, as the library would
+@pytest.mark.parametrize("k_split", [0, -1])             # 0: the warp-MMA kernel where the library takes it, up to 32 rows
 def test_ragged_shapes_and_batch_sizes(N, K, M, k_split):
     c = make_case(N, K, seed=900 + N + M, M=M)
     Y = _run(c, pack_case(c, V3), N, K, k_split=k_split)
@@ -63,7 +63,7 @@ def test_partial_sums_over_a_last_superblock_of_one_or_two_groups(K, k_split):
 @pytest.mark.parametrize("K", [1024, 2048, 2176, 4608, 6272])
 def test_format_2_with_and_without_a_workspace(K):
     # full slices and a last one of one to many groups, blocks with quarters empty, both sides of every class of batch sizes; the calls
-    # with and without a workspace give the same bits (no row is left alone by passes of four), and the fp16 operands less error than block fixed point could
+    # with and without a workspace give the same bits (no row is left alone by passes of four; up to 16 rows of K = 1024 both run the warp MMAs)
     V2 = binding.FORMAT_V2
     for i, N in enumerate((1602, 1777, 2049, 2400)):
         for M in ((10, 36), (16, 64), (18, 48), (32, 50))[i]:
@@ -73,8 +73,35 @@ def test_format_2_with_and_without_a_workspace(K):
             Y = binding.ptqtp_gemm_skinny_ws(packed, N, K, x, workspace=ws, fmt=V2).cpu().numpy()
             ref = np.atleast_2d(oracle_y(c))
             assert_parity(Y, ref, c["x"], "N=%d K=%d M=%d" % (N, K, M))
-            assert np.linalg.norm(Y - ref) / np.linalg.norm(ref) < 2.5e-4          # one rounding to fp16: 2.1e-4
+            assert np.linalg.norm(Y - ref) / np.linalg.norm(ref) < 2.5e-4          # one rounding to fp16: 2.1e-4 (and block fixed point: 2.3e-4)
             assert np.array_equal(Y.view(np.uint16), binding.ptqtp_gemm_skinny(packed, N, K, x, fmt=V2).cpu().numpy().view(np.uint16))
+    assert binding.ptqtp_kernel_status() == 0
+
+
+@pytest.mark.parametrize("fmt,N,K,M,fp16", [(2, 1024, 1536, 10, False), (2, 2048, 1536, 12, False), (2, 1536, 1024, 16, False), (2, 20480, 2048, 10, False),
+                                            (2, 128, 28672, 10, False), (2, 128, 28672, 6, False), (2, 1280, 2048, 12, True), (2, 4096, 1024, 16, True),
+                                            (2, 2048, 3072, 10, True), (2, 1024, 1536, 18, True), (3, 2048, 1536, 18, True), (3, 4096, 1024, 20, True),
+                                            (3, 5003, 512, 32, True), (3, 20480, 512, 24, True), (3, 2560, 1536, 25, True)])
+def test_either_side_of_the_lines_between_the_kernels(fmt, N, K, M, fp16):
+    # one column of 20000 per scale group, with trit 0 in both planes, next to others below 2^-7: with fp16 operands it adds nothing, block
+    # fixed point (the warp MMAs on format 2) has no bits left for the others
+    g = torch.Generator(device="cuda")
+    g.manual_seed(N + M)
+    trits = lambda: torch.randint(-1, 2, (N, K), generator=g, device="cuda", dtype=torch.int8)  # noqa: E731
+    scale = lambda: (torch.randn((N, K // 128), generator=g, device="cuda") * 0.02).abs().half()  # noqa: E731
+    T1, T2, a1, a2 = trits(), trits(), scale(), scale()
+    T1[:, 37::128] = T2[:, 37::128] = 0
+    X = (torch.randn((M, K), generator=g, device="cuda") * 2.0 ** -9).half()
+    X[:, 37::128] = 20000.0
+    W = a1.double().repeat_interleave(128, 1) * T1.double() + a2.double().repeat_interleave(128, 1) * T2.double()
+    ref = X.double() @ W.T
+    packed, _ = binding.ptqtp_pack(T1, T2, a1, a2, fmt=fmt)
+    Y = binding.ptqtp_gemm_skinny(packed, N, K, X, fmt=fmt).double()
+    error = float((Y - ref).norm() / ref.norm())
+    assert error < 1e-3 if fp16 else error > 0.1, error
+    X = torch.randn((M, K), generator=g, device="cuda").half()
+    Y = binding.ptqtp_gemm_skinny(packed, N, K, X, fmt=fmt).cpu().numpy()
+    assert_parity(Y, (X.double() @ W.T).cpu().numpy(), X.cpu().numpy(), "%d x %d, %d rows" % (N, K, M))
     assert binding.ptqtp_kernel_status() == 0
 
 
@@ -119,8 +146,8 @@ def test_exact_on_integers():
 
 @pytest.mark.parametrize("N,K,M", [(300, 4096, 40), (14336, 4096, 16), (4096, 4096, 64)])
 def test_the_tcgen05_kernel_can_be_asked_for_with_a_split_of_its_own(N, K, M):
-    # k_split = -1 is one of the explicit splits, bit for bit; 0 is the library's choice of kernel, which for up to 32 rows is another one
-    # (sums that differ in the last bits of fp32: some of 229376 results round to another fp16 number)
+    # k_split = -1 is one of the explicit splits, bit for bit; 0 is the library's choice, which for up to 32 rows is another kernel or the
+    # one that sums the groups of a superblock by themselves first (the last bits of fp32: some of 229376 results round to another fp16 number)
     c = make_case(N, K, seed=88, M=M)
     packed = pack_case(c, V3)
     own, chosen = (_run(c, packed, N, K, k_split=k).view(np.uint16) for k in (-1, 0))
