@@ -15,33 +15,41 @@ from gpu_util import assert_parity, dev, oracle_y, pack_case
 
 pytestmark = pytest.mark.gpu
 V2, V3 = binding.FORMAT_V2, binding.FORMAT_V3
-N = K = 2048
+N = 2048
+SMALL = 896                                              # columns and rows of a matrix whose batches the workspace kernel takes
+SIZES = [(N, 2), (N, 5), (N, 6), (N, 24), (SMALL, 24)]
 
-# name -> (format, call); what it runs on 2048 x 2048 by the number of rows:
+# name -> (format, call); what it runs on 2048 x 2048 by the number of rows, and on 896 x 896 at 24:
 #   gemv5/gemm7  two rows: batch-1 tiles kernel; more: warp MMAs on int8 activations
-#   gemm7 fp16   warp MMAs on fp16 activations
-#   gemm6        tcgen05 kernel, two CTAs per row block
-#   gemv3/gemm7  format 2, up to three rows: register-stationary kernel; more: warp MMAs (and a batch-1 launch for a row left alone)
-#   workspace    format 2: warp MMAs, from 17 rows on conversion kernel and workspace kernel
+#   gemm7 fp16   warp MMAs on fp16 activations; 24 rows of 2048 x 2048: tcgen05 kernel
+#   gemm8        tcgen05 kernel, two CTAs per row block
+#   format 2     up to three rows: register-stationary kernel; five and six: warp MMAs (and a batch-1 launch for a row left alone); 24:
+#                tcgen05 kernel
+#   workspace    format 2: up to six rows warp MMAs, 24 tcgen05 kernel; 24 rows of 896 x 896: conversion kernel and workspace kernel
 FORMS = {
-    "gemv5/gemm7": (V3, lambda p, X, Y, ws, n=N, k=K: binding.ptqtp_gemm_skinny_cfg(p, n, k, X, Y=Y, path=5)),
-    "gemm7 fp16": (V3, lambda p, X, Y, ws, n=N, k=K: binding.ptqtp_gemm_skinny_cfg(p, n, k, X, Y=Y, path=6)),
-    "gemm6": (V3, lambda p, X, Y, ws, n=N, k=K: binding.ptqtp_gemm_skinny_cfg(p, n, k, X, Y=Y, path=6, k_split=2)),
-    "gemv3/gemm7": (V2, lambda p, X, Y, ws, n=N, k=K: binding.ptqtp_gemm_skinny(p, n, k, X, Y=Y, fmt=V2)),
-    "workspace": (V2, lambda p, X, Y, ws, n=N, k=K: binding.ptqtp_gemm_skinny_ws(p, n, k, X, Y=Y, workspace=ws, fmt=V2)),
+    "gemv5/gemm7": (V3, lambda p, X, Y, ws, n: binding.ptqtp_gemm_skinny_cfg(p, n, n, X, Y=Y, path=5)),
+    "gemm7 fp16": (V3, lambda p, X, Y, ws, n: binding.ptqtp_gemm_skinny_cfg(p, n, n, X, Y=Y, path=6)),
+    "gemm8": (V3, lambda p, X, Y, ws, n: binding.ptqtp_gemm_skinny_cfg(p, n, n, X, Y=Y, path=6, k_split=2)),
+    "format 2": (V2, lambda p, X, Y, ws, n: binding.ptqtp_gemm_skinny(p, n, n, X, Y=Y, fmt=V2)),
+    "workspace": (V2, lambda p, X, Y, ws, n: binding.ptqtp_gemm_skinny_ws(p, n, n, X, Y=Y, workspace=ws, fmt=V2)),
 }
 
 
 @pytest.fixture(scope="module")
 def layers():
-    # two layers with a gain of about one, so that long chains stay in the range of fp16
-    out = []
-    for seed in (50, 51):
-        c = make_case(N, K, seed=seed)
-        for a in ("alpha1", "alpha2"):
-            c[a] = (c[a].astype(np.float32) * 1.28).astype(np.float16)
-        out.append({V2: pack_case(c, V2), V3: pack_case(c, V3)})
+    # two layers of either size with a gain of about one, so that long chains stay in the range of fp16
+    out = {}
+    for n in (N, SMALL):
+        for seed in (50, 51):
+            c = make_case(n, n, seed=seed)
+            for a in ("alpha1", "alpha2"):
+                c[a] = (c[a].astype(np.float32) * 1.28 * (2048 / n) ** 0.5).astype(np.float16)
+            out.setdefault(n, []).append({V2: pack_case(c, V2), V3: pack_case(c, V3)})
     return out
+
+
+def workspace(n, M):
+    return torch.empty(binding.gemm_skinny_workspace_size(n, n, M, fmt=V2), dtype=torch.uint8, device="cuda")
 
 
 @pytest.fixture(scope="module")
@@ -79,21 +87,30 @@ def every_pair():
     return out + [names[0]] + names[::-1]
 
 
+@pytest.mark.parametrize("n,M", SIZES)
+def test_the_workspace_kernel_is_reached(layers, n, M):
+    # it alone writes the workspace
+    ws = workspace(n, M).fill_(0xA5)
+    fmt, call = FORMS["workspace"]
+    call(layers[n][0][fmt], dev(make_case(n, n, seed=57, M=M)["x"]), torch.empty((M, n), dtype=torch.float16, device="cuda"), ws, n)
+    assert bool((ws != 0xA5).any()) == (n == SMALL)
+
+
 @pytest.mark.parametrize("graph", [False, True])
 @pytest.mark.parametrize("level", [0, 1, 2])
-@pytest.mark.parametrize("M", [2, 5, 6, 24])
-def test_chain_of_every_kernel_behind_every_kernel(layers, M, level, graph):
+@pytest.mark.parametrize("n,M", SIZES)
+def test_chain_of_every_kernel_behind_every_kernel(layers, n, M, level, graph):
     order = every_pair()
     assert len({(a, b) for a, b in zip(order, order[1:])}) == len(FORMS) ** 2
-    X = dev(make_case(N, K, seed=52, M=M)["x"])
-    ws = torch.empty(binding.gemm_skinny_workspace_size(N, K, M, fmt=V2), dtype=torch.uint8, device="cuda")
-    Y = [torch.empty((M, N), dtype=torch.float16, device="cuda") for _ in order]
-    Z = [torch.empty((M, N), dtype=torch.float16, device="cuda") for _ in range(2)]
+    X = dev(make_case(n, n, seed=52, M=M)["x"])
+    ws = workspace(n, M)
+    Y = [torch.empty((M, n), dtype=torch.float16, device="cuda") for _ in order]
+    Z = [torch.empty((M, n), dtype=torch.float16, device="cuda") for _ in range(2)]
 
     def chain(ys, sync=False):
         for i, name in enumerate(order):
             fmt, call = FORMS[name]
-            call(layers[i % 2][fmt], X if i == 0 else ys[(i - 1) % len(ys)], ys[i % len(ys)], ws)
+            call(layers[n][i % 2][fmt], X if i == 0 else ys[(i - 1) % len(ys)], ys[i % len(ys)], ws, n)
             if sync:
                 torch.cuda.synchronize()
 
@@ -123,46 +140,46 @@ def test_chain_of_every_kernel_behind_every_kernel(layers, M, level, graph):
     assert binding.ptqtp_kernel_status() == 0
 
 
-@pytest.mark.parametrize("M", [2, 5, 6, 24])
-def test_blob_written_by_a_kernel_directly_ahead_at_level_0(layers, M):
+@pytest.mark.parametrize("n,M", SIZES)
+def test_blob_written_by_a_kernel_directly_ahead_at_level_0(layers, n, M):
     # the blob of every call is rewritten by an elementwise kernel, and the call before that is one that releases its dependents early
-    X = dev(make_case(N, K, seed=53, M=M)["x"])
-    ws = torch.empty(binding.gemm_skinny_workspace_size(N, K, M, fmt=V2), dtype=torch.uint8, device="cuda")
+    X = dev(make_case(n, n, seed=53, M=M)["x"])
+    ws = workspace(n, M)
     for name, (fmt, call) in FORMS.items():
         want = []
-        for lay in layers:
-            y = torch.empty((M, N), dtype=torch.float16, device="cuda")
-            call(lay[fmt], X, y, ws)
+        for lay in layers[n]:
+            y = torch.empty((M, n), dtype=torch.float16, device="cuda")
+            call(lay[fmt], X, y, ws, n)
             want.append(bits(y))
-        blob = torch.empty_like(layers[0][fmt])
-        ys = [torch.empty((M, N), dtype=torch.float16, device="cuda") for _ in range(6)]
+        blob = torch.empty_like(layers[n][0][fmt])
+        ys = [torch.empty((M, n), dtype=torch.float16, device="cuda") for _ in range(6)]
         torch.cuda.synchronize()
         for i, y in enumerate(ys):
-            torch.add(layers[i % 2][fmt], 0, out=blob)
-            call(blob, X, y, ws)
+            torch.add(layers[n][i % 2][fmt], 0, out=blob)
+            call(blob, X, y, ws, n)
         torch.cuda.synchronize()
         for i, y in enumerate(ys):
             assert np.array_equal(bits(y), want[i % 2]), (name, i)
 
 
 @pytest.mark.parametrize("level", [0, 1, 2])
-@pytest.mark.parametrize("M", [2, 5, 6, 24])
-def test_pack_directly_before_a_call(M, level):
+@pytest.mark.parametrize("n,M", SIZES)
+def test_pack_directly_before_a_call(n, M, level):
     # the same blob is packed anew and used by the next call without any synchronisation
-    cs = [make_case(N, K, seed=54 + i, M=M) for i in range(2)]
+    cs = [make_case(n, n, seed=54 + i, M=M) for i in range(2)]
     X = dev(cs[0]["x"])
     planes = [tuple(dev(c[k]) for k in ("T1", "T2", "alpha1", "alpha2")) for c in cs]
-    ws = torch.empty(binding.gemm_skinny_workspace_size(N, K, M, fmt=V2), dtype=torch.uint8, device="cuda")
+    ws = workspace(n, M)
     status = torch.zeros(1, dtype=torch.int32, device="cuda")
     refs = [oracle_y(dict(c, x=cs[0]["x"])) for c in cs]
     binding.ptqtp_set_overlap(level)
     for name, (fmt, call) in FORMS.items():
-        blob = torch.empty(binding.packed_size(N, K, fmt=fmt), dtype=torch.uint8, device="cuda")
-        ys = [torch.empty((M, N), dtype=torch.float16, device="cuda") for _ in range(6)]
+        blob = torch.empty(binding.packed_size(n, n, fmt=fmt), dtype=torch.uint8, device="cuda")
+        ys = [torch.empty((M, n), dtype=torch.float16, device="cuda") for _ in range(6)]
         torch.cuda.synchronize()
         for i, y in enumerate(ys):
             binding.ptqtp_pack(*planes[i % 2], packed=blob, dev_status=status, fmt=fmt)
-            call(blob, X, y, ws)
+            call(blob, X, y, ws, n)
         torch.cuda.synchronize()
         for i, y in enumerate(ys):
             assert_parity(y.cpu().numpy(), refs[i % 2], cs[0]["x"], "%s call %d" % (name, i))
@@ -171,26 +188,26 @@ def test_pack_directly_before_a_call(M, level):
 
 
 @pytest.mark.parametrize("level", [0, 1, 2])
-def test_small_batch_behind_batch_1_and_back(layers, level):
+@pytest.mark.parametrize("n,M", [(N, 6), (SMALL, 24)])
+def test_small_batch_behind_batch_1_and_back(layers, n, M, level):
     # activations of a batch written row by row by batch-1 calls, and a row of a small-batch result read by a batch-1 call
-    M = 6
-    x = dev(make_case(N, K, seed=56, M=M)["x"])
-    ws = torch.empty(binding.gemm_skinny_workspace_size(N, K, M, fmt=V2), dtype=torch.uint8, device="cuda")
+    x = dev(make_case(n, n, seed=56, M=M)["x"])
+    ws = workspace(n, M)
 
     def run(sync):
         out = []
         for name, (fmt, call) in FORMS.items():
-            X = torch.full((M, K), float("nan"), dtype=torch.float16, device="cuda")
-            Y, z = torch.empty((M, N), dtype=torch.float16, device="cuda"), torch.empty(N, dtype=torch.float16, device="cuda")
+            X = torch.full((M, n), float("nan"), dtype=torch.float16, device="cuda")
+            Y, z = torch.empty((M, n), dtype=torch.float16, device="cuda"), torch.empty(n, dtype=torch.float16, device="cuda")
             torch.cuda.synchronize()
             for m in range(M):
-                binding.ptqtp_gemv(layers[0][fmt], N, K, x[m], y=X[m], fmt=fmt)
+                binding.ptqtp_gemv(layers[n][0][fmt], n, n, x[m], y=X[m], fmt=fmt)
                 if sync:
                     torch.cuda.synchronize()
-            call(layers[1][fmt], X, Y, ws)
+            call(layers[n][1][fmt], X, Y, ws, n)
             if sync:
                 torch.cuda.synchronize()
-            binding.ptqtp_gemv(layers[0][fmt], N, K, Y[M - 1], y=z, fmt=fmt)
+            binding.ptqtp_gemv(layers[n][0][fmt], n, n, Y[M - 1], y=z, fmt=fmt)
             torch.cuda.synchronize()
             out.append((name, bits(Y), bits(z)))
         return out
@@ -202,13 +219,13 @@ def test_small_batch_behind_batch_1_and_back(layers, level):
 
 
 @pytest.mark.parametrize("level", [0, 1, 2])
-@pytest.mark.parametrize("M", [2, 5, 6, 24])
-def test_a_call_in_stream_order_releases_the_next_kernel_after_all_that_came_before(layers, neighbours, M, level):
+@pytest.mark.parametrize("n,M", SIZES)
+def test_a_call_in_stream_order_releases_the_next_kernel_after_all_that_came_before(layers, neighbours, n, M, level):
     # level 0, and the call after a pack at levels 1 and 2: a kernel behind the call that reads without waiting sees what a kernel ahead
     # of the call writes late, although that one released its dependents at once
-    X = dev(make_case(N, K, seed=58, M=M)["x"])
-    Y = torch.empty((M, N), dtype=torch.float16, device="cuda")
-    ws = torch.empty(binding.gemm_skinny_workspace_size(N, K, M, fmt=V2), dtype=torch.uint8, device="cuda")
+    X = dev(make_case(n, n, seed=58, M=M)["x"])
+    Y = torch.empty((M, n), dtype=torch.float16, device="cuda")
+    ws = workspace(n, M)
     c = make_case(16, 128, seed=59)
     planes = tuple(dev(c[k]) for k in ("T1", "T2", "alpha1", "alpha2"))
     small = torch.empty(binding.packed_size(16, 128, fmt=V3), dtype=torch.uint8, device="cuda")
@@ -217,14 +234,14 @@ def test_a_call_in_stream_order_releases_the_next_kernel_after_all_that_came_bef
     stream = torch.cuda.Stream()
     for name, (fmt, call) in FORMS.items():
         with torch.cuda.stream(stream):
-            call(layers[0][fmt], X, Y, ws)               # loads the kernels
+            call(layers[n][0][fmt], X, Y, ws, n)               # loads the kernels
             binding.ptqtp_set_overlap(level)
             for i in range(4):
                 stream.synchronize()
                 if level:
                     binding.ptqtp_pack(*planes, packed=small, dev_status=status, fmt=V3)
                 assert neighbours.run_late_writer(word.data_ptr(), i + 1, 200_000, stream.cuda_stream) == 0
-                call(layers[0][fmt], X, Y, ws)
+                call(layers[n][0][fmt], X, Y, ws, n)
                 assert neighbours.run_early_reader(word.data_ptr(), seen.data_ptr() + 4 * i, stream.cuda_stream) == 0
             stream.synchronize()
             binding.ptqtp_set_overlap(0)
@@ -233,31 +250,31 @@ def test_a_call_in_stream_order_releases_the_next_kernel_after_all_that_came_bef
 
 
 @pytest.mark.parametrize("level", [0, 1, 2])
-@pytest.mark.parametrize("M", [5, 24])
-def test_two_blobs_packed_directly_before_two_calls(M, level):
+@pytest.mark.parametrize("n,M", [(N, 5), (N, 24), (SMALL, 24)])
+def test_two_blobs_packed_directly_before_two_calls(n, M, level):
     # the second call reads a blob whose pack is two kernels ahead of it
-    cs = [make_case(N, K, seed=60 + i, M=M) for i in range(2)]
+    cs = [make_case(n, n, seed=60 + i, M=M) for i in range(2)]
     X = dev(cs[0]["x"])
     planes = [tuple(dev(c[k]) for k in ("T1", "T2", "alpha1", "alpha2")) for c in cs]
-    ws = torch.empty(binding.gemm_skinny_workspace_size(N, K, M, fmt=V2), dtype=torch.uint8, device="cuda")
+    ws = workspace(n, M)
     status = torch.zeros(1, dtype=torch.int32, device="cuda")
     want = {}
     for name, (fmt, call) in FORMS.items():
         for i in range(2):
-            y = torch.empty((M, N), dtype=torch.float16, device="cuda")
-            call(binding.ptqtp_pack(*planes[i], fmt=fmt)[0], X, y, ws)
+            y = torch.empty((M, n), dtype=torch.float16, device="cuda")
+            call(binding.ptqtp_pack(*planes[i], fmt=fmt)[0], X, y, ws, n)
             want[name, i] = bits(y)
     binding.ptqtp_set_overlap(level)
     for a, (fmt_a, call_a) in FORMS.items():
         for b, (fmt_b, call_b) in FORMS.items():
-            blobs = [torch.empty(binding.packed_size(N, K, fmt=f), dtype=torch.uint8, device="cuda") for f in (fmt_a, fmt_b)]
-            ys = [torch.empty((M, N), dtype=torch.float16, device="cuda") for _ in range(8)]
+            blobs = [torch.empty(binding.packed_size(n, n, fmt=f), dtype=torch.uint8, device="cuda") for f in (fmt_a, fmt_b)]
+            ys = [torch.empty((M, n), dtype=torch.float16, device="cuda") for _ in range(8)]
             torch.cuda.synchronize()
             for i in range(4):
                 binding.ptqtp_pack(*planes[i % 2], packed=blobs[0], dev_status=status, fmt=fmt_a)
                 binding.ptqtp_pack(*planes[(i + 1) % 2], packed=blobs[1], dev_status=status, fmt=fmt_b)
-                call_a(blobs[0], X, ys[2 * i], ws)
-                call_b(blobs[1], X, ys[2 * i + 1], ws)
+                call_a(blobs[0], X, ys[2 * i], ws, n)
+                call_b(blobs[1], X, ys[2 * i + 1], ws, n)
             torch.cuda.synchronize()
             for i in range(4):
                 assert np.array_equal(bits(ys[2 * i]), want[a, i % 2]), (a, b, i)
