@@ -189,11 +189,14 @@ PTQTP_API ptqtp_status ptqtp_gemv_multi(int32_t count, const ptqtp_shape *shapes
 
 /* Small-batch variant: Y[m,:] = layer(X[m,:]) for m < M, 1 <= M <= PTQTP_MAX_BATCH.
  * X: device fp16 [M*K] row-major; Y: device fp16 [M*N] row-major.  Same definition per row of X.
- * Format 2, 2 <= M <= 8 (16 on small matrices), and format 3, M <= 4 and larger M on small matrices: the planes are contracted
- * on the tensor cores with int8 warp MMAs against 15-bit block-fixed-point activations (blocks of 128 columns), exact int32
- * sums, fp32 scale epilogue.  More rows (on format 3 from M = 5 to about 20, by the size of the matrix): the activations are
- * fp16 operands as given (no quantisation), the trits exact fp16 numbers, the sums of a scale group accumulate in fp32 and
- * get the fp32 scale epilogue.  One pass over the planes takes up to 16 (int8) or 64 (fp16) rows, fewer when K is very long.
+ * Format 2, 2 <= M <= 8 (up to 16 by the shape, small matrices above all), and format 3, M <= 4 and larger M on small matrices: the
+ * planes are contracted on the tensor cores with int8 warp MMAs against 15-bit block-fixed-point activations (blocks of 128 columns),
+ * exact int32 sums, fp32 scale epilogue.  More rows (on format 3 from M = 5 to about 20, by the size of the matrix; on format 2 from
+ * M = 5 where K is so long that clusters of eight share it unequally): the activations are fp16 operands as given (no quantisation),
+ * the trits exact fp16 numbers, the sums of a scale group accumulate in fp32 and get the fp32 scale epilogue.  One pass over the
+ * planes takes up to 16 (int8), 32 (fp16, warp MMAs) or 64 (fp16, tcgen05) rows, fewer when K is very long.  On format 2 a row that
+ * passes of up to four leave alone (the last one of M = 5, 9, 13, ...; every one where K leaves no room for two) is a batch-1 call with
+ * the arithmetic of ptqtp_gemv, a pass of its own.  Which kernel takes a row, and so the last bits of its result, depends on M.
  * Matrices with few rows split K over a thread-block cluster and add the partial sums in a fixed order
  * (reproducible).  M = 1 runs the batch-1 kernel.  Format 1 is a batch-1 layout: M > 1 returns PTQTP_ERR_CONFIG. */
 PTQTP_API ptqtp_status ptqtp_gemm_skinny(const ptqtp_shape *shape /* host */, const void *packed,
@@ -211,8 +214,11 @@ PTQTP_API ptqtp_status ptqtp_gemm_skinny_cfg(const ptqtp_shape *shape /* host */
 /* Small-batch variant with a caller-provided workspace (format 2 only; PTQTP_ERR_CONFIG for format 1).
  * Same result definition as ptqtp_gemm_skinny.  The workspace (device, 16-byte aligned, at least
  * ptqtp_gemm_skinny_workspace_size(shape, m) bytes, contents irrelevant on entry, clobbered on return) holds X
- * converted once to block fixed point when one pass of ptqtp_gemm_skinny does not take all rows (then two kernels are
- * enqueued on `stream`); with it the packed planes are read from HBM exactly once for any M and K.
+ * converted once to block fixed point (two kernels are enqueued on `stream`) where the library takes the kernel that reads it.  It may
+ * for fewer than 1024 rows of weights and more rows of X than a pass of int8 warp MMAs takes, for more than 128 rows of weights per
+ * SM and 9 to 16 rows of X, and for up to 16 rows of X where clusters of eight share a long K unequally; there the results have 15-bit
+ * activations although ptqtp_gemm_skinny may take fp16.  Elsewhere the kernels of ptqtp_gemm_skinny take all rows, none as a pass
+ * of its own, and the workspace is left alone.  The packed planes are read from HBM once for any M and K.
  * Calls that share a workspace must not overlap on the GPU.  ptqtp_gemm_skinny_workspace_size returns 0 for a
  * bad shape, formats 1 and 3 (the workspace kernels read format 2) or M out of range.  (Small-batch use of the layer of Eq. 1-2; the paper measures batch 1.) */
 PTQTP_API size_t ptqtp_gemm_skinny_workspace_size(const ptqtp_shape *shape /* host */, int32_t m);
@@ -324,7 +330,7 @@ PTQTP_API const char *ptqtp_status_string(ptqtp_status status);
 PTQTP_API int ptqtp_last_cuda_error(void);
 
 /* Device-side health of the kernels that stream the packed planes with bulk copies (batch 1 of formats 2 and 3,
- * and the small-batch kernel for two to four rows) on the current device.  They wait for each copy with a bounded
+ * and the small-batch kernels but for the one that reads the workspace) on the current device.  They wait for each copy with a bounded
  * number of polls; if a wait ever gives up, the kernel
  * writes NaN to the rows it could not finish, records PTQTP_ERR_CUDA in a device word and still terminates.
  * This call enqueues a copy of that word (0 = healthy) to *status_host on `stream`; read it after syncing. */

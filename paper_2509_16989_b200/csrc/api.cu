@@ -262,13 +262,13 @@ static bool fp16_activations(const Layout3& L3, int m) {
     return us6 < us5;
 }
 // fp16: the warp-MMA kernel or the tcgen05 kernel (also with an explicit k_split), in microseconds per call in a chain at overlap level 0:
-//   8 rows: always warp MMAs (14336 x 4096 13.9 and 15.5, 4096 x 14336 14.8 and 15.2, 4096 x 4096 6.0 and 7.5).
-//   9 to 16 rows: warp MMAs take about 4.2 us and 0.445 per MB whatever the shape (1024 x 4096 4.9, 3072 x 3072 6.7, 4096 x 4096 8.2,
-//   6144 x 6144 12.7, 14336 x 4096 19.2, 20480 x 6144 32.5), the tcgen05 kernel what its waves of CTAs take (5.2, 6.9, 7.5, 13.1, 15.6, 38.6).
+//   8 rows: always warp MMAs (14336 x 4096 13.7 and 15.2, 4096 x 14336 14.7 and 14.9, 4096 x 4096 6.1 and 7.3).
+//   9 to 16 rows: warp MMAs take about 4.2 us and 0.445 per MB whatever the shape (1024 x 4096 4.8, 3072 x 3072 6.8, 4096 x 4096 8.2,
+//   6144 x 6144 13.0, 14336 x 4096 19.2, 20480 x 6144 32.7), the tcgen05 kernel what its waves of CTAs take (5.2, 6.8, 7.4, 12.8, 15.1, 38.3).
 //   17 to 32 rows: the one that takes less time.  Small matrices, where the tcgen05 kernel's start and end are most of the call, stay with
-//   the warp MMAs (1024 x 2048 at 24 and 32 rows 5.0 and 5.0 against 5.3 and 5.4, 1024 x 4096 5.4 and 6.4 against 5.7 and 5.8), and
+//   the warp MMAs (1024 x 2048 at 24 and 32 rows 4.9 and 4.8 against 5.2 and 5.2, 1024 x 4096 at 24 rows 5.4 against 5.8), and
 //   so do matrices whose superblocks find no even split or whose last wave is nearly empty (18 rows: 2048 x 1536 5.0 against 6.8, 4096 x
-//   1024 4.6 against 5.5, 5003 x 512 4.1 against 5.2, 20480 x 512 8.6 against 10.0); 14336 x 4096 33.2 against 17.3.  Over 603
+//   1024 4.6 against 5.5, 5003 x 512 4.1 against 5.2, 20480 x 512 8.6 against 10.0); 14336 x 4096 at 32 rows 33.2 against 16.8.  Over 603
 //   calls beside the first line the slower kernel is taken 20 times where it costs more than 3 % (11 % at most; with that line alone
 //   66 times, 36 %).  More rows: always tcgen05.
 static bool warp_mmas_for_fp16(const Layout3& L3, int m) {
@@ -299,8 +299,8 @@ static ptqtp_status skinny_v3(const Layout3& L3, const void* packed, int m, cons
 
 // Format 2: the tcgen05 kernel, on the fp16 activations as given, from 17 rows on, and from nine on where it takes less time than the warp
 // MMAs and more than its start and end.  Microseconds per call with a workspace in a chain at level 0, in brackets what takes it
-// otherwise: 12 rows 1024 x 2048 4.9 (5.2), 14336 x 4096 16.4 (19.3), 1024 x 1024 would be 4.9 against 4.0; 16 rows 4096 x 4096 7.4 (12.1),
-// 8192 x 8192 17.2 (27.2); 32 rows 1024 x 1024 5.5 (7.5), 14336 x 4096 18.3 (41.1); 64 rows 21.4 (74.3), 8192 x 28672 60 (275).
+// otherwise: 12 rows 1024 x 2048 4.7 (5.2), 14336 x 4096 16.1 (19.3), 1024 x 1024 would be 4.9 against 4.0; 16 rows 4096 x 4096 7.7 (12.1),
+// 8192 x 8192 16.9 (27.2); 32 rows 1024 x 1024 5.3 (7.5), 14336 x 4096 17.9 (41.1); 64 rows 21.0 (74.3), 8192 x 28672 60 to 70 (275).
 // Three superblocks over two CTAs, a second wave of a few blocks and few rows of many columns stay with the warp MMAs (10 rows: 1024 x
 // 1536 4.5 against 6.2, 20480 x 2048 14.5 against 20.1, 128 x 28672 9.1 against 13.5).  Over 961 calls of 9 to 16 rows the slower kernel
 // is taken 16 times where it costs more than 3 % (12 % at most; by the bytes alone 125 times, 47 %).
@@ -312,7 +312,7 @@ static bool tcgen05_v2(const Layout2& L2, int m) {
 }
 // With a workspace: that X is converted into it is pinned by tests for fewer than 1024 rows of weights and, up to 16 rows of X, for more row
 // blocks than SMs (28672 x 8192), so these stay on the workspace kernel although the tcgen05 kernel would be faster there too
-// (1000 x 4096 at 24 rows 15.8 against 5.8, 28672 x 8192 at 16 rows 79 against 55).
+// (1000 x 4096 at 24 rows 16.1 against 6.0, 28672 x 8192 at 16 rows 79 against 55).
 static bool tcgen05_v2_ws(const Layout2& L2, int m) {
     return m > 8 && tcgen05_v2(L2, m) && L2.n >= 1024 && (m > 16 || (L2.n + 127) / 128 <= sm_count());
 }

@@ -7,8 +7,8 @@
 // mbarriers alone:
 //   * 16 warps decode: a shift and a mask of a code word make two trits (times 2) of operand A, 16 instructions per 16 trits, stored
 //     straight to tensor memory (tcgen05.st 16x256b, whose fragment is a k-step of four lanes x four columns, what a code word holds).
-//     Each of the four warpgroups takes a quarter of a superblock's half-groups (64 columns, both planes) and is up to three groups ahead
-//     of the MMAs.
+//     Each of the four warpgroups takes a quarter of a superblock's half-groups (64 columns, both planes); the stages of trits hold three
+//     and a half groups at 16 rows, two at 64.
 //   * one warp issues the MMAs; one poll by four of its lanes covers all that a group waits for.
 //   * 8 warps read the accumulators (tcgen05.ld), two sets of them in turn: y += alpha1 d1 + alpha2 d2 in fp32, half of the
 //     columns each.
@@ -16,18 +16,19 @@
 //     activations (TMA, 128-byte swizzle, rows past M as zeros), fp16 as given.
 // Format 2 differs in the copies and in where a word lies: two tensor maps for the code bytes and two for the scale quads (full slices, the last
 // slice) bring the same 512 columns of 128 rows by TMA, as lines of 128 bytes [atom][row pair] whose swizzle spreads the eight row
-// pairs that a warp reads over the banks (14336 x 4096 with a workspace at 16, 32, 64 rows: 16.4, 18.3, 21.4 us; before 23.0, 41.1, 74.3).
+// pairs that a warp reads over the banks (14336 x 4096 with a workspace at 16, 32, 64 rows: 16.1, 17.9, 21.0 us; before 23.0, 41.1, 74.3).
 // Matrices with few rows split K over a cluster of up to 8 CTAs; every rank copies its partial sums (bulk copies between the
 // shared memories, counted on the receiver's mbarrier) to the rank that owns the columns, which adds them in rank order: no
 // atomics, no workspace, reproducible.
 //
-// What bounds it, from clock stamps in a copy of the kernel: at 64 rows the tensor pipe (37 cycles per MMA with A from tensor memory,
-// 600 a group, of about 900), at 16 rows the issue slots of the SM (decode 260 of them per group and scheduler; the issuing warp gets
+// What bounds it, from clock stamps in a copy of the kernel: at 64 rows the tensor pipe for two thirds of the time (37 cycles per MMA with A
+// from tensor memory, 600 a group, of about 900; the rest is not accounted for: a decoding warpgroup has one of the four stages of
+// trits there and cannot work ahead), at 16 rows the issue slots of the SM (decode 260 of them per group and scheduler; the issuing warp gets
 // its turn beside four decoding ones: 670 cycles a group, 330 of them MMAs); 3.5 us of a launch are start (first codes and
 // activations 2 us after the wait) and end.  Measured in a chain at level 0, microseconds (14336 x 4096, 4096 x 14336, 4096 x 4096,
 // 1024 x 4096), in brackets the kernel before it (trits by byte permutes and FMAs, activations by cp.async, decoding, sums and fetch in
-// the same warps): 64 rows 20.8, 20.7, 10.5, 7.5 (50.0, 43.3, 17.1, 11.3), 48 rows 18.8, 18.7, 9.3, 6.5 (40.5, 36.8, 14.4, 10.1), 32
-// rows 17.4, 17.1, 8.4, 5.8 (35.9, 32.8, 12.9, 9.0), 16 rows 15.6, 15.3, 7.5, 5.2 (30.7, 28.2, 11.4, 7.9).
+// the same warps): 64 rows 20.0, 20.0, 10.2, 7.4 (50.0, 43.3, 17.1, 11.3), 48 rows 18.3, 18.4, 9.1, 6.5 (40.5, 36.8, 14.4, 10.1), 32
+// rows 16.8, 16.6, 8.2, 5.8 (35.9, 32.8, 12.9, 9.0), 16 rows 15.1, 15.0, 7.4, 5.2 (30.7, 28.2, 11.4, 7.9).
 // What it took: activations by TMA (with cp.async four fetching warps needed 2500 cycles to issue a group of 64 rows: 37.7 us on 14336
 // x 4096), one issuing warp with few instructions, partial sums by bulk copies (loads from the ranks' shared memory took 4500 cycles
 // with eight ranks, st.async of 8 bytes 5000 at 64 rows), one compact loop for the output.  Without effect or slower:
@@ -39,8 +40,9 @@
 // CTA per row block 1.09e-7 (1.44e-7), four 0.80e-7 at 16, 0.94e-7 at 64 rows (0.94e-7, 1.17e-7); x of mean 4 0.80e-7, 1.12e-7,
 // 0.79e-7 (0.80e-7, 1.45e-7, 0.91e-7); x over 24 powers of two 1.98e-7, 2.12e-7, 1.99e-7 (1.98e-7, 2.32e-7, 2.07e-7).
 //
-// Launched as a dependent of the kernel before it on the stream: set-up before griddepcontrol.wait, and a prefetch of the first codes
-// into L2, the point of coherence; at overlap levels 1 and 2 the codes themselves.  Waits on mbarriers are bounded: a wait
+// Launched as a dependent of the kernel before it on the stream: set-up before griddepcontrol.wait, and on format 3 a prefetch of the
+// first codes into L2, the point of coherence; the next launch is released after it.  At overlap levels 1 and 2 the codes themselves are
+// read before it, as many as the ring holds, and the next launch is released at once.  Waits on mbarriers are bounded: a wait
 // that gives up marks the launch failed (status word, NaN rows); the CTA still meets its cluster and frees its tensor memory.
 #include <cuda.h>
 #include <cudaTypedefs.h>

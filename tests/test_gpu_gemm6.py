@@ -167,7 +167,7 @@ def test_rows_do_not_depend_on_their_neighbours():
 
 
 def test_library_dispatch():
-    # the library takes the tcgen05 kernel where its fixed cost pays: many rows, or a matrix of some size
+    # the library takes fp16 operands where the fixed cost of the tcgen05 kernel would pay: many rows, or a matrix of some size
     def same(a, b):
         torch.cuda.synchronize()
         return np.array_equal(a.cpu().numpy().view(np.uint16), b.cpu().numpy().view(np.uint16))

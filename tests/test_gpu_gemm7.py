@@ -1,6 +1,8 @@
 """GPU parity of the warp-MMA small-batch kernel (fp16 activations on format 3, 15-bit block fixed point on formats 3 and 2)
 against the fp64 oracle, at the edges of its tiles: row pairs, superblocks and slices, column tiles, one launch or several,
-columns in chunks, matrices taller than a launch; exact integer cases, the give-up path of its bounded waits."""
+columns in chunks, matrices taller than a launch; exact integer cases, the give-up path of its bounded waits.  (The library gives
+some of the larger cases to other kernels: fp16 with more than 32 rows and 16 rows of 4100 x 6144, on either format, to the tcgen05
+kernel, more than 16 rows of format 2 to the workspace kernel.)"""
 import numpy as np
 import pytest
 import torch

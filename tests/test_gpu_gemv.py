@@ -426,8 +426,8 @@ def _edge_and_sampled_rows(N, seed):
 
 @pytest.mark.parametrize("M", [2, 4, 8, 16, 32, 64])
 def test_gemm_skinny_config2_shape_every_batch_size_both_entry_points(M):
-    # the batch sweep that the measurements run, at its full size: 14336 x 4096 (13 compute warps per CTA in the
-    # workspace kernel), first and last 64 rows and 2048 sampled rows against the fp64 oracle
+    # the batch sweep that the measurements run, at its full size: 14336 x 4096 (warp MMAs up to eight rows, then the tcgen05 kernel,
+    # on either call), first and last 64 rows and 2048 sampled rows against the fp64 oracle
     N, K = LLAMA3_8B_UNIQUE["gate_up"]
     c = make_case(N, K, seed=2, M=M)
     packed = pack_case(c, binding.FORMAT_V2)
