@@ -75,6 +75,12 @@ def test_format_2_with_and_without_a_workspace(K):
             assert_parity(Y, ref, c["x"], "N=%d K=%d M=%d" % (N, K, M))
             assert np.linalg.norm(Y - ref) / np.linalg.norm(ref) < 2.5e-4          # one rounding to fp16: 2.1e-4 (and block fixed point: 2.3e-4)
             assert np.array_equal(Y.view(np.uint16), binding.ptqtp_gemm_skinny(packed, N, K, x, fmt=V2).cpu().numpy().view(np.uint16))
+        # a batch whose last row a batch-1 launch takes when there is no workspace, and this kernel when there is
+        M = (17, 33, 21, 61)[i]
+        c = make_case(N, K, seed=850 + N, M=M)
+        packed, x, ref = pack_case(c, V2), dev(c["x"]), oracle_y(c)
+        assert_parity(binding.ptqtp_gemm_skinny(packed, N, K, x, fmt=V2).cpu().numpy(), ref, c["x"], "N=%d K=%d M=%d" % (N, K, M))
+        assert_parity(binding.ptqtp_gemm_skinny_ws(packed, N, K, x, fmt=V2).cpu().numpy(), ref, c["x"], "N=%d K=%d M=%d workspace" % (N, K, M))
     assert binding.ptqtp_kernel_status() == 0
 
 
