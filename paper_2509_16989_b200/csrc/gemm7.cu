@@ -33,6 +33,7 @@
 // prefetched into L2.  At overlap levels 1 and 2 (where it pays, see launch_nt7) they are read, and the next kernel may start at once.  Waits on mbarriers
 // are bounded: a warp that gives up marks the launch failed (status word) and its rows come out as NaN.
 #include <cuda_fp16.h>
+#include <atomic>
 #include "ptqtp_internal.h"
 
 namespace ptqtp {
@@ -595,18 +596,18 @@ gemm7_kernel(const __grid_constant__ Args7 a) {
     }
 }
 
-// Clusters of csize CTAs that fit on the device at once (one CTA per SM; asked of the runtime once per device and size).
+// Clusters of csize CTAs that fit on the device at once (one CTA per SM; asked of the runtime once per device and size: every plan
+// asks for several sizes, and every call makes a few plans, so what is known is read without a lock).
 template <int FMT, bool INT8, int NT>
 int max_clusters(int csize) {
-    static std::mutex mu;
-    static int known[64][4] = {};
+    static std::atomic<int> known[64][4] = {};
     int dev = 0;
     const int lg = csize == 1 ? 0 : csize == 2 ? 1 : csize == 4 ? 2 : 3;
     if (csize == 1) return sm_count();
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return sm_count() / csize;
-    if (configure_once<gemm7_kernel<FMT, INT8, NT>>() != PTQTP_OK) return sm_count() / csize;
-    std::lock_guard<std::mutex> lock(mu);
-    if (!known[dev][lg]) {
+    int n = known[dev][lg].load(std::memory_order_relaxed);
+    if (!n) {
+        if (configure_once<gemm7_kernel<FMT, INT8, NT>>() != PTQTP_OK) return sm_count() / csize;
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(sm_count() / csize * csize);
         cfg.blockDim = dim3(max_warps7(INT8, NT) * 32);
@@ -617,11 +618,11 @@ int max_clusters(int csize) {
         attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
-        int n = 0;
         if (cudaOccupancyMaxActiveClusters(&n, gemm7_kernel<FMT, INT8, NT>, &cfg) != cudaSuccess || n < 1) { (void)cudaGetLastError(); n = sm_count() / csize; }
-        known[dev][lg] = n < sm_count() / csize ? n : sm_count() / csize;
+        n = n < sm_count() / csize ? n : sm_count() / csize;
+        known[dev][lg].store(n, std::memory_order_relaxed);
     }
-    return known[dev][lg];
+    return n;
 }
 
 // The launch shape of a matrix (rows in tiles of 16, superblocks): clusters, CTAs per cluster, warps that split K.

@@ -629,8 +629,7 @@ ptqtp_status launch_n8(Args8& a, const uint16_t* X, int blocks, cudaStream_t st)
 
 // Clusters of csize CTAs that run at once (one CTA per SM; larger clusters leave SMs of a GPC idle): of 4 and 8 what the runtime said
 // on this device for kernels of this footprint, 33 and 15 of 148 SMs.
-int clusters8(int csize) {
-    const int sms = sm_count();
+int clusters8(int csize, int sms) {
     return csize <= 2 ? sms / csize : csize == 4 ? max(1, sms * 33 / 148) : max(1, sms * 15 / 148);
 }
 
@@ -643,9 +642,10 @@ struct Plan8 {
 };
 Plan8 plan8(int blocks, int sbs, int npad) {
     const double group = npad == 16 ? 0.35 : npad == 32 ? 0.39 : npad == 48 ? 0.46 : 0.53;
+    const int sms = sm_count();
     Plan8 best = {1, 0.0};
     for (int c = 1; c <= 8 && (c == 1 || c <= sbs); c *= 2) {
-        const int waves = (blocks + clusters8(c) - 1) / clusters8(c);
+        const int waves = (blocks + clusters8(c, sms) - 1) / clusters8(c, sms);
         const double us = waves * (4.2 + 4.0 * group * ((sbs + c - 1) / c)) + (c > 1 ? 0.7 : 0.0);
         if (c == 1 || us < best.us) best = {c, us};
     }
@@ -662,7 +662,7 @@ double gemm8_plan_us(const Layout3& L, int m) { return plan8(blocks8(L), L.sbs, 
 // 961 calls on format 2 (9 to 16 rows) and 849 on format 3 (17 to 32), 128 to 28672 rows by 256 to 28672 columns.
 static double gemm8_us(int blocks, int n, int k, int m, size_t total, bool v2) {
     const int sbs = (k + kSuper3 - 1) / kSuper3, split = plan8(blocks, sbs, (m + 15) / 16 * 16).split;
-    const int waves = (blocks + clusters8(split) - 1) / clusters8(split), groups = min(4 * ((sbs + split - 1) / split), k / kGroup);
+    const int clusters = clusters8(split, sm_count()), waves = (blocks + clusters - 1) / clusters, groups = min(4 * ((sbs + split - 1) / split), k / kGroup);
     const bool odd = n % 8 != 0;
     return v2 ? waves * (2.55 + 0.33 * groups + (odd ? 0.27 : 0.0)) + 1.25 * (waves - 1) + (split > 1 ? 0.68 : 0.0) + 0.16e-6 * (double)total
               : waves * (3.35 + 0.28 * groups + (odd ? 0.56 : 0.0)) + 1.0 * (waves - 1) + (split > 1 ? 0.65 : 0.0) + 0.09e-6 * (double)total;
