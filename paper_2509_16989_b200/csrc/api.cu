@@ -318,24 +318,31 @@ static bool tcgen05_v2_ws(const Layout2& L2, int m) {
 }
 
 // Small batch on format 2, m >= 2.  A row that passes of up to four (as many as find room) leave alone keeps the batch-1
-// kernel's 16-bit activations per 64 columns; the other rows have 15 bits per 128 columns, on either of two kernels: two rows, and
-// up to four on small matrices, take the register-stationary kernel, whose launches overlap at level 2 (two rows of 4096 x 4096
-// there 4.4 us against 5.6; at level 0 6.6 against 6.0); the rest the warp-MMA kernel.  For three and four rows the line is
+// kernel's 16-bit activations per 64 columns; the other rows are fp16 operands on the tcgen05 kernel, or have 15 bits per 128 columns, on
+// either of two kernels: two rows, and up to four on small matrices, take the register-stationary kernel, whose launches overlap at
+// level 2 (two rows of 4096 x 4096 there 4.4 us against 5.6; at level 0 6.6 against 6.0); the rest the warp-MMA kernel.  For three and four rows the line is
 // near 1.1 MB at every level (1024 x 2048: 3.4 and 3.6 us against 3.4 and 3.4 at level 0, 3.6 and 3.9 against 3.5 and 3.4 at level
 // 2; 1024 x 1024 3.1 against 3.3 and 3.1; 1536 x 2048 4.0 and 4.2 against 3.6 and 3.5 at level 2).
 static ptqtp_status skinny_v2(const Layout2& L2, const void* packed, int m, const uint16_t* X, uint16_t* Y, cudaStream_t st) {
     const int per_pass = gemv3_rows_per_pass(L2, m), alone = per_pass == 1 ? m : m % per_pass == 1 ? 1 : 0;
     int rows = m - alone;
     // beside whole-SM CTAs of the other kernel a launch that overlaps its neighbours at level 2 pays on small matrices only (five rows of
-    // 2048 x 4096 7.9 us against 9.7 in stream order, 3072 x 3072 11.6 against 8.3, 14336 x 4096 30.3 against 17.5)
-    const bool in_order = rows > 0 && L2.total > 4700000;
+    // 2048 x 4096 7.9 us against 9.7 in stream order, 3072 x 3072 11.6 against 8.3, 14336 x 4096 30.3 against 17.5), and beside the
+    // tcgen05 kernel only where that leaves a third of the SMs (17 rows, 96 CTAs: 6144 x 1024 6.8 against 9.3, 3072 x 2048 6.1 against 8.7;
+    // 112: 14336 x 512 13.7 against 10.1; 128: 8192 x 1024 12.6 against 9.7, 4096 x 2048 10.2 against 9.2)
+    bool tcgen05 = tcgen05_v2(L2, rows);
+    const bool in_order = rows > 0 && (L2.total > 4700000 || (alone && tcgen05 && 3 * gemm8_ctas(L2, rows) > 2 * sm_count()));
     for (int i = rows; i < m; ++i) {
         const ptqtp_status s = launch_gemv2(L2, packed, X + (size_t)i * L2.k, Y + (size_t)i * L2.n, 0, 0, 0, 0, st, false, in_order);
         if (s != PTQTP_OK && (i > rows || s == PTQTP_ERR_CUDA)) return s;
-        if (s != PTQTP_OK) { rows = m; break; }          // K too long for it: nothing launched yet
+        if (s != PTQTP_OK) {                             // K too long for it: nothing launched yet
+            rows = m;
+            tcgen05 = tcgen05_v2(L2, rows);
+            break;
+        }
     }
     if (rows == 0) return PTQTP_OK;
-    if (tcgen05_v2(L2, rows)) return launch_gemm8(L2, packed, rows, X, Y, st);
+    if (tcgen05) return launch_gemm8(L2, packed, rows, X, Y, st);
     if (rows > 4 || (L2.k > 8192 && (rows > 2 || !gemm7_uneven(L2))) || (rows > 2 && L2.total > 1400000)) return launch_gemm7(L2, packed, rows, X, Y, st);
     const ptqtp_status s = launch_gemv3(L2, packed, rows, X, Y, 0, 0, 0, st);
     return s == PTQTP_ERR_SHAPE ? launch_gemm7(L2, packed, rows, X, Y, st) : s;

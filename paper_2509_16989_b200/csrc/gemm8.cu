@@ -669,6 +669,10 @@ static double gemm8_us(int blocks, int n, int k, int m, size_t total, bool v2) {
 }
 double gemm8_us(const Layout3& L, int m) { return gemm8_us(blocks8(L), L.n, L.k, m, L.total, false); }
 double gemm8_us(const Layout2& L, int m) { return gemm8_us((L.nrp + 63) / 64, L.n, L.k, m, L.total, true); }
+int gemm8_ctas(const Layout2& L, int m) {
+    const int blocks = (L.nrp + 63) / 64;
+    return blocks * plan8(blocks, (L.k + kSuper3 - 1) / kSuper3, (m + 15) / 16 * 16).split;
+}
 
 namespace {
 void common8(Args8& a, int n, int k, int m, int nrb, int sbs, int split, uint16_t* Y, cudaStream_t st) {

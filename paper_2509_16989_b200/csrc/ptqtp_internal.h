@@ -165,6 +165,7 @@ ptqtp_status launch_gemm8(const Layout2& L, const void* packed, int m, const uin
 double gemm8_plan_us(const Layout3& L, int m);     // what its plan reckons with
 double gemm8_us(const Layout3& L, int m);     // what these calls take, up to 32 rows
 double gemm8_us(const Layout2& L, int m);
+int gemm8_ctas(const Layout2& L, int m);      // of a launch, one per SM
 // 1 <= m <= 64 rows on formats 3 and 2, warp MMAs on a CTA's share of rows and columns.  int8: 15-bit block fixed-point
 // activations, otherwise fp16 as given.  gemm7_one_launch: all m rows take one pass over the planes.
 ptqtp_status launch_gemm7(const Layout3& L, const void* packed, int m, const uint16_t* X, uint16_t* Y, bool int8, cudaStream_t st);
