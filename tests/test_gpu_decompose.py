@@ -131,6 +131,36 @@ def test_every_sort_width_and_ragged_batches_of_group_rows(G):
             assert_same(run(W, group=G, canonicalize=canonicalize), decompose_c(W, G=G, canonicalize=canonicalize), "%d x %d" % (rows, G))
 
 
+@pytest.mark.parametrize("rows,K,G,kw,okw", [(2048, 4096, 128, {}, {}), (1000, 1536, 24, {"t_max": 12}, {"T_max": 12}),
+                                             (1024, 2048, 32, {"eps": 0.05}, {"eps": 0.05})])
+def test_lanes_that_take_one_group_row_after_the_other(rows, K, G, kw, okw):
+    # more group-rows than the lanes of the device: group-rows of every length of run beside each other in a warp, zeros, constants,
+    # inexact sums, subnormal and huge weights, and errors that are next to nothing among them
+    rng = np.random.default_rng(500 + G)
+    W = (rng.standard_normal((rows, K)) * 0.02).astype(np.float32)
+    W[rng.random(W.shape) < 1e-3] *= 20
+    g = W.reshape(-1, G)
+    n = g.shape[0]
+    pick = lambda share: rng.random(n) < share  # noqa: E731
+    g[pick(0.02)] = 0.0
+    g[pick(0.02)] = np.float32(0.25)
+    m = pick(0.02)
+    g[m] *= np.exp2(rng.integers(-40, 3, g[m].shape)).astype(np.float32)
+    g[pick(0.01)] *= np.float32(1e-41)
+    g[pick(0.01)] *= np.float32(1e30)
+    m = pick(0.02)
+    g[m] = (0.02 * rng.integers(-1, 2, g[m].shape) + 0.0075 * rng.integers(-1, 2, g[m].shape)).astype(np.float32)
+    assert_same(run(W, group=G, **kw), decompose_c(W, G=G, **okw), "%d x %d G=%d" % (rows, K, G))
+
+
+@pytest.mark.parametrize("t_max", [1, 2, 999, 1000])
+def test_histories_with_and_without_room_for_the_records(t_max):
+    # few weights and many sweeps: the records of errors find no room beside the planes
+    for rows, G in ((1, 128), (3, 16), (40, 128)):
+        W = (np.random.default_rng(600 + rows).standard_normal((rows, 2 * G)) * 0.02).astype(np.float32)
+        assert_same(run(W, group=G, t_max=t_max, eps=0.0), decompose_c(W, G=G, T_max=t_max, eps=0.0), "%d %d" % (rows, t_max))
+
+
 @pytest.mark.parametrize("G", [128, 20, 7])
 def test_non_finite_weights_stay_in_their_group_rows(G):
     # a NaN or an infinity makes the scales of its group-row NaN in the first sweep and its planes 0 (no candidate is nearer than
