@@ -1,15 +1,16 @@
 // Pack / unpack kernels of the PTQTP-B200 format 2 (layout described in ptqtp.h).
 // A thread handles 16-byte atoms: 16 columns of one row pair, both planes.  Atoms are numbered along the rows, so that
 // neighbouring lanes read neighbouring columns (numbered in storage order they would read every fourth 16 bytes); two
-// atoms per thread are in flight.  Bound by memory: 14336 x 4096 packs in 28.0 us and unpacks in 25.2 (43.7 and 42.5 with
-// atoms in storage order, a division in 64 bits for each and byte-wise coding).
+// atoms per thread are in flight.  Bound by memory: 14336 x 4096 packs in 27.2 us and unpacks in 24.6 (27.8 and 24.9 with CTAs of
+// 256 threads and plain stores of the blob, 31.1 and 25.6 with 512; 43.7 and 42.5 with atoms in storage order, a division in 64
+// bits for each and byte-wise coding).
 #include "trit_bytes.h"
 
 namespace ptqtp {
 
 namespace {
 
-constexpr int kThreadsP2 = 256;
+constexpr int kThreadsP2 = 128;
 
 __device__ __forceinline__ int active_of(const Layout2& L, int slice) {
     return slice == L.slices - 1 ? L.last_active : 32;
@@ -37,6 +38,7 @@ pack2_kernel(Layout2 L, const int8_t* __restrict__ T1, const int8_t* __restrict_
              const uint16_t* __restrict__ a2, unsigned char* __restrict__ packed, int32_t* dev_status) {
     const size_t stride = (size_t)gridDim.x * blockDim.x;
     const size_t tid = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    in_order();
     unsigned char* codes = packed + L.codes_off;
     bool bad = false;
 
@@ -57,7 +59,7 @@ pack2_kernel(Layout2 L, const int8_t* __restrict__ T1, const int8_t* __restrict_
 #pragma unroll
     for (int n = 0; n < A; ++n)
         if (live[n])
-            *reinterpret_cast<uint4*>(codes + atom_offset(L, rp[n], col[n])) = pair_words(v[n][0], v[n][1], v[n][2], v[n][3], bad);
+            __stcs(reinterpret_cast<uint4*>(codes + atom_offset(L, rp[n], col[n])), pair_words(v[n][0], v[n][1], v[n][2], v[n][3], bad));
 
     // scale quads: one per row pair and 128-column group, after the codes of their slice unit
     const int groups = L.k / kGroup;
@@ -107,6 +109,7 @@ template <class I, int A>
 __global__ void __launch_bounds__(kThreadsP2)
 unpack2_kernel(Layout2 L, const unsigned char* __restrict__ packed, int8_t* __restrict__ T1, int8_t* __restrict__ T2,
                uint16_t* __restrict__ a1, uint16_t* __restrict__ a2, int32_t* dev_status) {
+    in_order();
     if (blockIdx.x == 0 && threadIdx.x == 0 && dev_status) {
         const Header* h = reinterpret_cast<const Header*>(packed);
         const char m[8] = {'P', 'T', 'Q', 'T', 'P', 'B', '2', '\0'};
@@ -163,8 +166,8 @@ unsigned ctas_for2(const Layout2& L, int atoms) {
     const size_t per_cta = (size_t)kThreadsP2 * atoms;
     return (unsigned)(((size_t)L.nrp * (L.k / 16) + per_cta - 1) / per_cta);
 }
-// Two atoms per thread once that still leaves every SM four CTAs (1024 x 1024: 4.2 us with two, 3.5 with one).
-bool two_atoms2(const Layout2& L) { return ctas_for2(L, 2) >= 4u * (unsigned)sm_count(); }
+// Two atoms per thread once that still leaves every SM eight CTAs (1024 x 1024: 4.2 us with two, 3.5 with one).
+bool two_atoms2(const Layout2& L) { return ctas_for2(L, 2) >= 8u * (unsigned)sm_count(); }
 bool index32_2(const Layout2& L) { return (size_t)L.nrp * (L.k / 16) < ((size_t)1 << 32) - 2 * kThreadsP2; }
 
 }  // namespace
@@ -173,16 +176,14 @@ ptqtp_status launch_pack2(const Layout2& L, const int8_t* T1, const int8_t* T2, 
                           const uint16_t* a2, void* packed, int32_t* dev_status, cudaStream_t st) {
     const bool two = two_atoms2(L);
     auto kern = !two ? pack2_kernel<uint32_t, 1> : index32_2(L) ? pack2_kernel<uint32_t, 2> : pack2_kernel<size_t, 2>;
-    kern<<<ctas_for2(L, two ? 2 : 1), kThreadsP2, 0, st>>>(L, T1, T2, a1, a2, static_cast<unsigned char*>(packed), dev_status);
-    return check_launch();
+    return launch_in_order(kern, ctas_for2(L, two ? 2 : 1), kThreadsP2, 0, st, L, T1, T2, a1, a2, static_cast<unsigned char*>(packed), dev_status);
 }
 
 ptqtp_status launch_unpack2(const Layout2& L, const void* packed, int8_t* T1, int8_t* T2, uint16_t* a1,
                             uint16_t* a2, int32_t* dev_status, cudaStream_t st) {
     const bool two = two_atoms2(L);
     auto kern = !two ? unpack2_kernel<uint32_t, 1> : index32_2(L) ? unpack2_kernel<uint32_t, 2> : unpack2_kernel<size_t, 2>;
-    kern<<<ctas_for2(L, two ? 2 : 1), kThreadsP2, 0, st>>>(L, static_cast<const unsigned char*>(packed), T1, T2, a1, a2, dev_status);
-    return check_launch();
+    return launch_in_order(kern, ctas_for2(L, two ? 2 : 1), kThreadsP2, 0, st, L, static_cast<const unsigned char*>(packed), T1, T2, a1, a2, dev_status);
 }
 
 }  // namespace ptqtp

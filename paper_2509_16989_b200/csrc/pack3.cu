@@ -2,14 +2,18 @@
 // A run of 16 columns of one scale group is two words of each of two neighbouring lane entries, so a thread takes a row pair,
 // chunk and group pair of a tile: eight 16-byte loads (two rows, two planes, the two groups of the pair), 32
 // contiguous bytes of the blob.  Eight lanes cover 128 contiguous bytes of a row.  Bound by memory: 14336 x 4096
-// packs in 27.8 us and unpacks in 25.9 (5.4 and 5.7 TB/s; 61.9 and 112 with four-byte accesses and byte-wise coding).
+// packs in 26.2 us and unpacks in 25.6 (5.7 and 5.9 TB/s; 61.9 and 112 with four-byte accesses and byte-wise coding).  Packing takes a
+// tile per CTA and streams the blob out past L2 (two tiles, plain stores 27.5; four tiles 32.9; a loop of CTAs that stay, the
+// next tile's loads in flight, 41); unpacking two (one tile: 25.4 there, but 4.2 against 3.9 on 1024 x 4096).
+// Launched as dependents that wait first: call after call of the binding 26.9 us packing and 26.9 unpacking 14336 x 4096 (28.8 and 28.7 with
+// plain launches).
 #include "trit_bytes.h"
 
 namespace ptqtp {
 
 namespace {
 
-constexpr int kThreadsP3 = 256, kTileThreads3 = 128;   // a CTA takes two tiles
+constexpr int kTileThreads3 = 128, kThreadsPack3 = 128, kThreadsUnpack3 = 256;
 
 // Thread -> tile (row block by row block, so that neighbours read the same rows), chunk, row pair, group pair.
 struct Run3 {
@@ -18,7 +22,7 @@ struct Run3 {
     bool live;
 };
 __device__ __forceinline__ Run3 run_of(const Layout3& L) {
-    const size_t tile = (size_t)blockIdx.x * (kThreadsP3 / kTileThreads3) + threadIdx.x / kTileThreads3;
+    const size_t tile = (size_t)blockIdx.x * (blockDim.x / kTileThreads3) + threadIdx.x / kTileThreads3;
     const int r = threadIdx.x % kTileThreads3;
     Run3 p;
     p.rb = (int)(tile / L.sbs);
@@ -31,9 +35,10 @@ __device__ __forceinline__ Run3 run_of(const Layout3& L) {
     return p;
 }
 
-__global__ void __launch_bounds__(kThreadsP3)
+__global__ void __launch_bounds__(kThreadsPack3)
 pack3_kernel(Layout3 L, const int8_t* __restrict__ T1, const int8_t* __restrict__ T2, const uint16_t* __restrict__ a1,
              const uint16_t* __restrict__ a2, unsigned char* __restrict__ packed, int32_t* dev_status) {
+    in_order();
     unsigned char* codes = packed + L.codes_off;
     bool bad = false;
     const Run3 p = run_of(L);
@@ -54,8 +59,8 @@ pack3_kernel(Layout3 L, const int8_t* __restrict__ T1, const int8_t* __restrict_
         const uint4 lo = pair_words(v[0][0], v[0][1], v[0][2], v[0][3], bad), hi = pair_words(v[1][0], v[1][1], v[1][2], v[1][3], bad);
         // entry t = 2 u: columns 0-3 and 8-11 of the run, t = 2 u + 1: columns 4-7 and 12-15; words (s, h)
         uint4* dst = reinterpret_cast<uint4*>(codes + p.tile_off + (p.c * 32 + 4 * p.g + 2 * p.u) * 16);
-        dst[0] = make_uint4(lo.x, hi.x, lo.z, hi.z);
-        dst[1] = make_uint4(lo.y, hi.y, lo.w, hi.w);
+        __stcs(dst, make_uint4(lo.x, hi.x, lo.z, hi.z));
+        __stcs(dst + 1, make_uint4(lo.y, hi.y, lo.w, hi.w));
     }
 
     // scale quads: 32 per tile, quad 4 g + t = row pair g of the tile, group t of the superblock
@@ -89,9 +94,10 @@ pack3_kernel(Layout3 L, const int8_t* __restrict__ T1, const int8_t* __restrict_
     if (bad && dev_status) atomicExch(dev_status, (int)PTQTP_ERR_TRIT);
 }
 
-__global__ void __launch_bounds__(kThreadsP3)
+__global__ void __launch_bounds__(kThreadsUnpack3)
 unpack3_kernel(Layout3 L, const unsigned char* __restrict__ packed, int8_t* __restrict__ T1, int8_t* __restrict__ T2,
                uint16_t* __restrict__ a1, uint16_t* __restrict__ a2, int32_t* dev_status) {
+    in_order();
     if (blockIdx.x == 0 && threadIdx.x == 0 && dev_status) {
         const Header* h = reinterpret_cast<const Header*>(packed);
         const char m[8] = {'P', 'T', 'Q', 'T', 'P', 'B', '2', '\0'};
@@ -136,8 +142,8 @@ unpack3_kernel(Layout3 L, const unsigned char* __restrict__ packed, int8_t* __re
     }
 }
 
-unsigned grid_for3(const Layout3& L) {
-    constexpr size_t per_cta = kThreadsP3 / kTileThreads3;
+unsigned grid_for3(const Layout3& L, int threads) {
+    const size_t per_cta = threads / kTileThreads3;
     return (unsigned)(((size_t)L.nrb * L.sbs + per_cta - 1) / per_cta);
 }
 
@@ -145,16 +151,13 @@ unsigned grid_for3(const Layout3& L) {
 
 ptqtp_status launch_pack3(const Layout3& L, const int8_t* T1, const int8_t* T2, const uint16_t* a1,
                           const uint16_t* a2, void* packed, int32_t* dev_status, cudaStream_t st) {
-    pack3_kernel<<<grid_for3(L), kThreadsP3, 0, st>>>(L, T1, T2, a1, a2, static_cast<unsigned char*>(packed),
-                                                        dev_status);
-    return check_launch();
+    return launch_in_order(pack3_kernel, grid_for3(L, kThreadsPack3), kThreadsPack3, 0, st, L, T1, T2, a1, a2, static_cast<unsigned char*>(packed), dev_status);
 }
 
 ptqtp_status launch_unpack3(const Layout3& L, const void* packed, int8_t* T1, int8_t* T2, uint16_t* a1,
                             uint16_t* a2, int32_t* dev_status, cudaStream_t st) {
-    unpack3_kernel<<<grid_for3(L), kThreadsP3, 0, st>>>(L, static_cast<const unsigned char*>(packed), T1, T2,
-                                                          a1, a2, dev_status);
-    return check_launch();
+    return launch_in_order(unpack3_kernel, grid_for3(L, kThreadsUnpack3), kThreadsUnpack3, 0, st, L, static_cast<const unsigned char*>(packed), T1, T2, a1, a2,
+                           dev_status);
 }
 
 }  // namespace ptqtp

@@ -220,4 +220,28 @@ inline ptqtp_status configure_once(bool with_carveout = true) {
 }
 
 
+// A launch in stream order whose set-up overlaps the end of the kernel before it: a dependent launch of a kernel that executes in_order()
+// before it touches any memory that others see.
+template <class... P, class... A>
+ptqtp_status launch_in_order(void (*kernel)(P...), unsigned grid, int threads, size_t smem, cudaStream_t st, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+    if (e != cudaSuccess) { set_last_cuda_error(e); (void)cudaGetLastError(); return PTQTP_ERR_CUDA; }
+    return PTQTP_OK;
+}
+// Waits until everything before this kernel on the stream is complete, then lets the next launch begin its own set-up.
+__device__ __forceinline__ void in_order() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;");
+}
+
 }  // namespace ptqtp

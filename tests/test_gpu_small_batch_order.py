@@ -320,3 +320,40 @@ def test_polls_of_the_tcgen05_kernel_do_not_count_the_time_of_the_kernel_ahead(n
     binding.ptqtp_kernel_status_clear()
     assert status == 0 and np.array_equal(bits(Y), want)
     assert_parity(Y.cpu().numpy(), oracle_y(c), c["x"], form)
+
+
+@pytest.mark.parametrize("fmt", [V2, V3])
+@pytest.mark.parametrize("form", ["pack", "unpack", "decompose"])
+def test_conversions_follow_stream_order_between_dependent_launches(neighbours, form, fmt):
+    # a kernel ahead that releases its dependents at once and writes late what the call reads; a kernel behind that reads without waiting sees
+    # what that kernel wrote
+    n, k = 48, 1152
+    c = make_case(n, k, seed=62)
+    planes = [dev(c[v]) for v in ("T1", "T2", "alpha1", "alpha2")]
+    blob = binding.ptqtp_pack(*planes, fmt=fmt)[0]
+    W, status = torch.randn((n, k), generator=torch.Generator().manual_seed(5)).cuda(), torch.zeros(1, dtype=torch.int32, device="cuda")
+    source = {"pack": planes[0], "unpack": blob, "decompose": W}[form]
+
+    def call():
+        if form == "pack":
+            return binding.ptqtp_pack(*planes, packed=torch.empty_like(blob), dev_status=status, fmt=fmt)[0]
+        return binding.ptqtp_unpack(blob, n, k, dev_status=status, fmt=fmt)[0] if form == "unpack" else binding.ptqtp_decompose(W)[0]
+
+    # the late word: four trits, the bytes of four columns, or a weight
+    words = source.view(torch.uint8).flatten()[256:256 + 4 * 64].view(torch.int32) if form == "unpack" else source.flatten().view(torch.int32)
+    old = int(words[0].item())
+    new = {"pack": 0x0100ff01, "unpack": 0x55555555, "decompose": 0x3f800000}[form]
+    stream, seen = torch.cuda.Stream(), torch.zeros(8, dtype=torch.int32, device="cuda")
+    with torch.cuda.stream(stream):
+        for i in range(4):
+            value = new if i % 2 == 0 else old
+            words[0] = value
+            want = call().clone()
+            words[0] = old if i % 2 == 0 else new
+            stream.synchronize()
+            assert neighbours.run_late_writer(words.data_ptr(), value, 200_000, stream.cuda_stream) == 0
+            got = call()
+            assert neighbours.run_early_reader(words.data_ptr(), seen.data_ptr() + 4 * i, stream.cuda_stream) == 0
+            stream.synchronize()
+            assert torch.equal(got, want), (form, i)
+            assert int(seen[i].item()) == value
