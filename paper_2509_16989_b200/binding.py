@@ -1,4 +1,5 @@
-"""ctypes binding of libptqtp.so: argument marshalling only; every step runs in the CUDA kernels.
+"""Binding of libptqtp.so: argument marshalling only; every step runs in the CUDA kernels.  ctypes, and for the plain arguments of
+a decode loop the extension of marshal.cpp, which checks tensors and calls the library in a third of the time.
 
 torch supplies device memory and streams.  Function names mirror the C ABI (include/ptqtp.h).
 There is no CPU path: if the shared library is missing or a call fails, a PtqtpError is raised.
@@ -48,6 +49,21 @@ class Shape(ctypes.Structure):
 
 
 _lib = None
+# the functions of the extension, or None: its library is not there or was built for another torch
+_gemv_plain = _gemv_host_plain = _gemm_skinny_plain = _gemm_skinny_ws_plain = None
+
+
+def _bind_plain(L):
+    global _gemv_plain, _gemv_host_plain, _gemm_skinny_plain, _gemm_skinny_ws_plain
+    try:
+        from . import _marshal as m
+    except ImportError:
+        return
+    if m.torch_version != torch.__version__.split("+")[0]:
+        return
+    m.bind(*[ctypes.cast(f, ctypes.c_void_p).value
+             for f in (L.ptqtp_gemv, L.ptqtp_gemv_host, L.ptqtp_gemm_skinny, L.ptqtp_gemm_skinny_ws)])
+    _gemv_plain, _gemv_host_plain, _gemm_skinny_plain, _gemm_skinny_ws_plain = m.gemv, m.gemv_host, m.gemm_skinny, m.gemm_skinny_ws
 
 
 def lib():
@@ -108,6 +124,7 @@ def lib():
         L.ptqtp_set_wait_limit.argtypes = [ctypes.c_int]
         L.ptqtp_test_fail_next_wait.restype = None
         L.ptqtp_test_fail_next_wait.argtypes = [ctypes.c_int]
+        _bind_plain(L)
         _lib = L
     return _lib
 
@@ -197,6 +214,11 @@ def ptqtp_unpack(packed, N, K, dev_status=None, stream=None, fmt=None):
 
 def ptqtp_gemv(packed, N, K, x, y=None, stream=None, fmt=None):
     """y[N] = layer(x[K]) from a packed blob; fp16 CUDA tensors."""
+    if _gemv_plain is not None and y is not None and stream is None:
+        st = _gemv_plain(packed, x, y, N, K, DEFAULT_FORMAT if fmt is None else fmt)
+        if st is not None:
+            _check(st, "ptqtp_gemv")
+            return y
     shape = _shape_ref(N, K, fmt)
     if y is None:
         y = torch.empty(N, dtype=torch.float16, device=x.device)
@@ -286,6 +308,11 @@ def ptqtp_gemv_multi(packed_list, N_list, K, x, ys=None, epilogue=EPILOGUE_NONE,
 
 def ptqtp_gemm_skinny(packed, N, K, X, Y=None, stream=None, fmt=None):
     """Y[M,N] = layer applied to each row of X[M,K]; fp16 CUDA tensors, 1 <= M <= 64."""
+    if _gemm_skinny_plain is not None and Y is not None and stream is None:
+        st = _gemm_skinny_plain(packed, X, Y, N, K, DEFAULT_FORMAT if fmt is None else fmt)
+        if st is not None:
+            _check(st, "ptqtp_gemm_skinny")
+            return Y
     shape = _shape_ref(N, K, fmt)
     M = X.shape[0]
     if Y is None:
@@ -316,6 +343,11 @@ def gemm_skinny_workspace_size(N, K, M, fmt=None):
 
 def ptqtp_gemm_skinny_ws(packed, N, K, X, Y=None, workspace=None, stream=None, fmt=None):
     """ptqtp_gemm_skinny with a caller-provided workspace (uint8 CUDA tensor; allocated here if None)."""
+    if _gemm_skinny_ws_plain is not None and Y is not None and workspace is not None and stream is None:
+        st = _gemm_skinny_ws_plain(packed, X, Y, workspace, N, K, DEFAULT_FORMAT if fmt is None else fmt)
+        if st is not None:
+            _check(st, "ptqtp_gemm_skinny_ws")
+            return Y
     shape = _shape_ref(N, K, fmt)
     M = X.shape[0]
     if Y is None:
@@ -348,6 +380,11 @@ def ptqtp_gemm_skinny_static(packed, N, K, X, Y, stream=None, fmt=None):
 
 def ptqtp_gemv_host(packed, N, K, x_host, y_host, x_dev, y_dev, stream=None, fmt=None):
     """Host-buffer call: H2D copy of x, GEMV, D2H copy of y, all on `stream` (no sync)."""
+    if _gemv_host_plain is not None and stream is None:
+        st = _gemv_host_plain(packed, x_host, y_host, x_dev, y_dev, N, K, DEFAULT_FORMAT if fmt is None else fmt)
+        if st is not None:
+            _check(st, "ptqtp_gemv_host")
+            return y_host
     shape = _shape_ref(N, K, fmt)
     for t, what in ((x_host, "x_host"), (y_host, "y_host")):
         if t.is_cuda or t.dtype != torch.float16 or not t.is_contiguous():

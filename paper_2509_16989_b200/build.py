@@ -1,12 +1,15 @@
-"""Build libptqtp.so in-tree with nvcc for sm_100a (no JIT cache, no torch extension machinery)."""
+"""Build libptqtp.so in-tree with nvcc for sm_100a and the marshalling extension of the binding with the host compiler (no JIT cache, no
+torch extension machinery)."""
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libptqtp.so")
+MARSHAL = os.path.join(HERE, "_marshal.so")
 SOURCES = ["api.cu", "pack.cu", "pack2.cu", "gemv.cu", "gemv2.cu", "gemv3.cu", "pack3.cu", "gemv4.cu", "gemv5.cu", "gemm7.cu", "gemm8.cu", "skinny3.cu", "decompose.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "-Xcompiler", "-fvisibility=hidden", "--shared", "-cudart", "shared"]
@@ -20,15 +23,31 @@ def _nvcc():
 
 
 def needs_build():
-    if not os.path.exists(LIB):
+    if not os.path.exists(LIB) or not os.path.exists(MARSHAL):
         return True
-    t = os.path.getmtime(LIB)
+    t = min(os.path.getmtime(LIB), os.path.getmtime(MARSHAL))
     deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)] + [os.path.join(ROOT, "include", "ptqtp.h")]
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+def build_marshal():
+    """Compile csrc/marshal.cpp into paper_2509_16989_b200/_marshal.so against the torch that is installed."""
+    import torch
+    root = os.path.dirname(torch.__file__)
+    cuda = os.path.dirname(os.path.dirname(_nvcc())) if os.path.isabs(_nvcc()) else "/usr/local/cuda"
+    cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
+           "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI), "-I", os.path.join(ROOT, "include"),
+           "-I", sysconfig.get_paths()["include"], "-isystem", os.path.join(cuda, "include"), "-isystem", os.path.join(root, "include"),
+           "-isystem", os.path.join(root, "include", "torch", "csrc", "api", "include"), os.path.join(CSRC, "marshal.cpp"),
+           "-L", os.path.join(root, "lib"), "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python", "-o", MARSHAL]
+    res = subprocess.run(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)
+    if res.returncode != 0:
+        sys.stderr.write(res.stdout)
+        raise RuntimeError("building _marshal.so failed")
+
+
 def build(force=False, verbose=False, extra=()):
-    """Compile every CUDA source into paper_2509_16989_b200/libptqtp.so; returns its path."""
+    """Compile every CUDA source into paper_2509_16989_b200/libptqtp.so and the marshalling extension; returns the library's path."""
     if not force and not needs_build():
         return LIB
     cmd = [_nvcc()] + NVCC_FLAGS + list(extra) + ["-I", os.path.join(ROOT, "include"), "-I", CSRC]
@@ -40,6 +59,7 @@ def build(force=False, verbose=False, extra=()):
         sys.stderr.write(res.stdout)
     if res.returncode != 0:
         raise RuntimeError("nvcc failed building libptqtp.so")
+    build_marshal()
     return LIB
 
 
