@@ -1,9 +1,10 @@
 // Pack / unpack kernels of the PTQTP-B200 format 2 (layout described in ptqtp.h).
 // A thread handles 16-byte atoms: 16 columns of one row pair, both planes.  Atoms are numbered along the rows, so that
 // neighbouring lanes read neighbouring columns (numbered in storage order they would read every fourth 16 bytes); two
-// atoms per thread are in flight.  Bound by memory: 14336 x 4096 packs in 27.2 us and unpacks in 24.6 (27.8 and 24.9 with CTAs of
-// 256 threads and plain stores of the blob, 31.1 and 25.6 with 512; 43.7 and 42.5 with atoms in storage order, a division in 64
-// bits for each and byte-wise coding).
+// atoms per thread are in flight.  Bound by memory: 14336 x 4096 packs in 27.7 us and unpacks in 24.6 (27.8 and 24.9 with CTAs of
+// 256 threads, 31.1 and 25.6 with 512; 43.7 and 42.5 with atoms in storage order, a division in 64 bits for each and byte-wise
+// coding).  Streaming stores of the blob would bring 27.2, but who reads it next finds it in L2 without them (a call of ptqtp_unpack right
+// after 55 us with the host's part, 61 from memory).
 #include "trit_bytes.h"
 
 namespace ptqtp {
@@ -59,7 +60,7 @@ pack2_kernel(Layout2 L, const int8_t* __restrict__ T1, const int8_t* __restrict_
 #pragma unroll
     for (int n = 0; n < A; ++n)
         if (live[n])
-            __stcs(reinterpret_cast<uint4*>(codes + atom_offset(L, rp[n], col[n])), pair_words(v[n][0], v[n][1], v[n][2], v[n][3], bad));
+            *reinterpret_cast<uint4*>(codes + atom_offset(L, rp[n], col[n])) = pair_words(v[n][0], v[n][1], v[n][2], v[n][3], bad);
 
     // scale quads: one per row pair and 128-column group, after the codes of their slice unit
     const int groups = L.k / kGroup;

@@ -2,10 +2,10 @@
 // A run of 16 columns of one scale group is two words of each of two neighbouring lane entries, so a thread takes a row pair,
 // chunk and group pair of a tile: eight 16-byte loads (two rows, two planes, the two groups of the pair), 32
 // contiguous bytes of the blob.  Eight lanes cover 128 contiguous bytes of a row.  Bound by memory: 14336 x 4096
-// packs in 26.2 us and unpacks in 25.6 (5.7 and 5.9 TB/s; 61.9 and 112 with four-byte accesses and byte-wise coding).  Packing takes a
-// tile per CTA and streams the blob out past L2 (two tiles, plain stores 27.5; four tiles 32.9; a loop of CTAs that stay, the
-// next tile's loads in flight, 41); unpacking two (one tile: 25.4 there, but 4.2 against 3.9 on 1024 x 4096).
-// Launched as dependents that wait first: call after call of the binding 26.9 us packing and 26.9 unpacking 14336 x 4096 (28.8 and 28.7 with
+// packs in 26.7 us and unpacks in 25.6 (5.6 and 5.9 TB/s; 61.9 and 112 with four-byte accesses and byte-wise coding).  Packing takes a
+// tile per CTA (two tiles 27.5; four 32.9; a loop of CTAs that stay, the next tile's loads in flight, 41; streaming stores of the blob
+// 26.2, but who reads it next finds it in L2 without them); unpacking two (one tile: 25.4 there, but 4.2 against 3.9 on 1024 x 4096).
+// Launched as dependents that wait first: call after call of the binding 27.1 us packing and 26.9 unpacking 14336 x 4096 (28.8 and 28.7 with
 // plain launches).
 #include "trit_bytes.h"
 
@@ -59,8 +59,8 @@ pack3_kernel(Layout3 L, const int8_t* __restrict__ T1, const int8_t* __restrict_
         const uint4 lo = pair_words(v[0][0], v[0][1], v[0][2], v[0][3], bad), hi = pair_words(v[1][0], v[1][1], v[1][2], v[1][3], bad);
         // entry t = 2 u: columns 0-3 and 8-11 of the run, t = 2 u + 1: columns 4-7 and 12-15; words (s, h)
         uint4* dst = reinterpret_cast<uint4*>(codes + p.tile_off + (p.c * 32 + 4 * p.g + 2 * p.u) * 16);
-        __stcs(dst, make_uint4(lo.x, hi.x, lo.z, hi.z));
-        __stcs(dst + 1, make_uint4(lo.y, hi.y, lo.w, hi.w));
+        dst[0] = make_uint4(lo.x, hi.x, lo.z, hi.z);
+        dst[1] = make_uint4(lo.y, hi.y, lo.w, hi.w);
     }
 
     // scale quads: 32 per tile, quad 4 g + t = row pair g of the tile, group t of the superblock
