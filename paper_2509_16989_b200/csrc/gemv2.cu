@@ -476,14 +476,20 @@ ptqtp_status launch_gemv2(const Layout2& L, const void* packed, const uint16_t* 
     const int max_warps = kMaxWarps2 / per_sm;
     const size_t budget = (size_t)(228 / per_sm - 1) * 1024;          // 228 KB per SM, 1 KB of it reserved per CTA
     const int grid = min(per_sm * sm_count(), L.nrp);
-    if (warps == 0 && (!overlap_enabled() || in_order)) warps = -1;   // nothing to gain from sharing an SM with the next launch
+    const long units_per_cta = (long)((L.nrp + grid - 1) / grid) * S;
+    if (warps == 0 && (!overlap_enabled() || in_order)) {
+        // Nothing to gain from sharing an SM with the next launch: as many warps as fit, but on one or two slices fewer where 16 would have
+        // less than two units each: starting them takes longer than they save.  In a chain at level 0, 16, 8 and 4 warps: 1000 x 1024
+        // (4 units per CTA) 2.58, 2.38, 2.30 us, 2048 x 2048 (7) 2.80, 2.66, 2.59, 1000 x 4096 (8) 2.87, 2.61, 2.95, 3072 x 1024 (11) 2.95, 2.84,
+        // 2.94, 4096 x 4096 (28) 4.18, 4.10, 4.83, 6144 x 3072 (42) 4.91, 5.11; three slices 2048 x 6144 (21) 3.90, 4.36 (six warps).
+        warps = per_sm == 1 && S <= 2 && units_per_cta <= 28 ? (S == 1 && units_per_cta <= 7 ? 4 : 8) : -1;
+    }
     if (warps == -1) {
         // the caller knows that the call runs alone (copies on both sides of it): one CTA takes the whole SM
         warps = S >= max_warps ? max_warps : S * (max_warps / S);
     } else if (warps == 0) {
         // a multiple of the slice count (every slice lane gets as many warps): at least 4, at least 8 when a CTA
         // streams many units, and all 16 when that is what it takes to give every slice a warp
-        const long units_per_cta = (long)((L.nrp + grid - 1) / grid) * S;
         const int target = units_per_cta >= 160 ? 8 : 4;  // (a long launch with 4 warps holds up the short ones behind it)
         warps = S >= max_warps ? max_warps : S * ((target + S - 1) / S);
         if (warps > max_warps) warps = S * (max_warps / S);

@@ -706,3 +706,17 @@ def test_kernel_status_is_healthy():
     c = make_case(64, 4096, seed=60)
     run_gemv(c, binding.FORMAT_V2)
     assert binding.ptqtp_kernel_status() == 0
+
+
+@pytest.mark.parametrize("N,K", [(2, 128), (2072, 2048), (2074, 2048), (8288, 1152), (8290, 1152), (4144, 4096), (4146, 4096), (301, 3200)])
+def test_fewer_warps_on_small_matrices_give_the_same_bits(N, K):
+    # format 2 in stream order, either side of the lines between 4, 8 and 16 warps (7 and 28 units per CTA of 148; one and two slices)
+    c = make_case(N, K, seed=900 + K)
+    packed = pack_case(c, binding.FORMAT_V2)
+    x = dev(c["x"])
+    y = binding.ptqtp_gemv(packed, N, K, x, fmt=binding.FORMAT_V2)
+    all_warps = binding.ptqtp_gemv_cfg(packed, N, K, x, k_split=-1, fmt=binding.FORMAT_V2)
+    torch.cuda.synchronize()
+    assert torch.equal(y, all_warps)
+    rows = np.unique(np.concatenate([np.arange(min(N, 64)), np.arange(max(0, N - 64), N)]))
+    assert_parity(y.cpu().numpy()[rows], oracle_y(c, rows), c["x"], "%d x %d" % (N, K))
