@@ -265,7 +265,8 @@ PTQTP_API ptqtp_status ptqtp_gemm_skinny_static(const ptqtp_shape *shape /* host
  * workspace: device, 16-byte aligned, ptqtp_decompose_workspace_size bytes, contents irrelevant on entry.  On
  * return (after syncing) it holds, at the offsets given by ptqtp_decompose_layout: int32 sweeps run; per sweep
  * t = 1..sweeps the largest change of a scale pair (f64 at delta_offset + 8 t) and the total squared error after the
- * sweep (f64 at error_offset + 8 (t - 1)); per group-row the unrounded scales and lambda (f64).
+ * sweep (f64 at error_offset + 8 (t - 1); the error of a group-row is held to twice the precision and rounded once, their sum in double);
+ * per group-row the unrounded scales and lambda (f64).
  * Four or five kernels are enqueued on `stream`; no synchronisation.  T1, T2, alpha1 and alpha2 hold other values until the last of them. */
 #define PTQTP_DECOMPOSE_MAX_GROUP 256
 #define PTQTP_DECOMPOSE_MAX_SWEEPS 1000

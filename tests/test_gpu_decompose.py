@@ -161,6 +161,32 @@ def test_histories_with_and_without_room_for_the_records(t_max):
         assert_same(run(W, group=G, t_max=t_max, eps=0.0), decompose_c(W, G=G, T_max=t_max, eps=0.0), "%d %d" % (rows, t_max))
 
 
+def _total_error(W, T1, T2, a1, a2, G):
+    # the levels rounded once, as the T-step forms them; an fp32 weight minus such a level fits into the 64 bits of an extended double
+    level = a1.reshape(-1, 1) * T1.reshape(-1, G) + a2.reshape(-1, 1) * T2.reshape(-1, G)
+    d = W.reshape(-1, G).astype(np.longdouble) - level.astype(np.longdouble)
+    return (d * d).sum()
+
+
+@pytest.mark.parametrize("G", [128, 256, 100, 64, 20, 16])
+def test_error_of_a_group_row_in_full_precision(G):
+    # one group-row at a time, from weights that two planes hardly describe to ones that they describe to 2^-30 of the sum of the squares:
+    # the error after a sweep is that sum minus what the planes explain, and what is left is good to its own last bit.  Bound: the parts are
+    # held to twice the precision, so one rounding, 2^-53; twice that, because the parts below it were rounded as well.
+    rng = np.random.default_rng(800 + G)
+    left = []
+    for noise in (1.0, 0.3, 0.1, 0.05, 0.03, 0.02, 0.01, 1e-3, 1e-4):
+        for most in (1, 2) * 3:                          # around 0 and one or two levels of either sign
+            W = (np.copysign(0.01, rng.standard_normal((1, G))) * rng.integers(0, most + 1, (1, G)) +
+                 rng.standard_normal((1, G)) * 0.01 * noise).astype(np.float32)
+            for t_max in (1, 2, 7, 20):
+                got = run(W, group=G, t_max=t_max, eps=0.0, canonicalize=False)
+                want = _total_error(W, got["T1"], got["T2"], got["alpha1"], got["alpha2"], G)
+                assert abs(np.longdouble(got["err_history"][-1]) - want) <= 2.0 ** -52 * want, (noise, t_max)
+                left.append(float(want) / float((W.astype(np.float64) ** 2).sum()))
+    assert min(left) < 2.0 ** -20 and max(left) > 2.0 ** -6 and sum(2.0 ** -11 < v < 2.0 ** -9 for v in left) > 3
+
+
 @pytest.mark.parametrize("G", [128, 20, 7])
 def test_non_finite_weights_stay_in_their_group_rows(G):
     # a NaN or an infinity makes the scales of its group-row NaN in the first sweep and its planes 0 (no candidate is nearer than
