@@ -187,6 +187,15 @@ def test_error_of_a_group_row_in_full_precision(G):
     assert min(left) < 2.0 ** -20 and max(left) > 2.0 ** -6 and sum(2.0 ** -11 < v < 2.0 ** -9 for v in left) > 3
 
 
+@pytest.mark.parametrize("t_max", [2, 30, 31, 32, 33, 62, 63, 64, 65, 100])
+def test_histories_past_the_sweep_at_which_the_last_group_row_repeats(t_max):
+    # eps = 0 goes on to t_max; a warp per sweep, 32 at a time, sweep 0 among them
+    rng = np.random.default_rng(700 + t_max)
+    W = (rng.standard_normal((256, 1024)) * 0.02).astype(np.float32)
+    for w in (W, np.sign(W) * np.float32(0.25), np.zeros_like(W)):
+        assert_same(run(w, t_max=t_max, eps=0.0), decompose_c(w, T_max=t_max, eps=0.0))
+
+
 @pytest.mark.parametrize("G", [128, 20, 7])
 def test_non_finite_weights_stay_in_their_group_rows(G):
     # a NaN or an infinity makes the scales of its group-row NaN in the first sweep and its planes 0 (no candidate is nearer than
