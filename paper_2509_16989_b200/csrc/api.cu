@@ -333,7 +333,7 @@ static ptqtp_status skinny_v2(const Layout2& L2, const void* packed, int m, cons
     bool tcgen05 = tcgen05_v2(L2, rows);
     const bool in_order = rows > 0 && (L2.total > 4700000 || (alone && tcgen05 && 3 * gemm8_ctas(L2, rows) > 2 * sm_count()));
     for (int i = rows; i < m; ++i) {
-        const ptqtp_status s = launch_gemv2(L2, packed, X + (size_t)i * L2.k, Y + (size_t)i * L2.n, 0, 0, 0, 0, st, false, in_order);
+        const ptqtp_status s = launch_gemv2(L2, packed, X + (size_t)i * L2.k, Y + (size_t)i * L2.n, 0, 0, 0, 0, st, false, in_order, rows > 0);
         if (s != PTQTP_OK && (i > rows || s == PTQTP_ERR_CUDA)) return s;
         if (s != PTQTP_OK) {                             // K too long for it: nothing launched yet
             rows = m;

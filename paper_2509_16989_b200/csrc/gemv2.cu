@@ -458,7 +458,8 @@ ptqtp_status copy_gemv2_status(int32_t* status_host, cudaStream_t st) {
     return PTQTP_OK;
 }
 
-// gated: y[i] = silu(row 2i) * row 2i+1 instead of the rows themselves (N even).  in_order: as at overlap level 0.
+// gated: y[i] = silu(row 2i) * row 2i+1 instead of the rows themselves (N even).  in_order: as at overlap level 0.  beside: a small-batch
+// kernel for the other rows of the call follows.
 // warps: per CTA, 0 = the default below, -1 = as many as fit (for a call that is known to run alone).
 // ctas_per_sm: CTAs of this launch per SM (0 = one).  units: slice units per bulk copy (1, 2 or 4; 0 = 2).
 // The defaults keep a CTA small (4 to 8 warps, two ring slots of two units per warp) so that the CTAs of several
@@ -466,7 +467,7 @@ ptqtp_status copy_gemv2_status(int32_t* status_host, cudaStream_t st) {
 // execution the head of one launch (fetching x) and the tail of another (verifying x, reducing) then overlap the
 // streaming of a third.  Measured on the LLaMA-3-8B shapes, 4 warps beat 8 and 16.
 ptqtp_status launch_gemv2(const Layout2& L, const void* packed, const uint16_t* x, uint16_t* y, int warps,
-                          int ctas_per_sm, int depth, int units, cudaStream_t st, bool gated, bool in_order) {
+                          int ctas_per_sm, int depth, int units, cudaStream_t st, bool gated, bool in_order, bool beside) {
     const int S = L.slices;
     const int speculate = speculation_enabled() && !in_order ? 1 : 0;
     if (ctas_per_sm < 0 || ctas_per_sm > 4) return PTQTP_ERR_CONFIG;
@@ -481,8 +482,13 @@ ptqtp_status launch_gemv2(const Layout2& L, const void* packed, const uint16_t* 
         // Nothing to gain from sharing an SM with the next launch: as many warps as fit, but on one or two slices fewer where 16 would have
         // less than two units each: starting them takes longer than they save.  In a chain at level 0, 16, 8 and 4 warps: 1000 x 1024
         // (4 units per CTA) 2.58, 2.38, 2.30 us, 2048 x 2048 (7) 2.80, 2.66, 2.59, 1000 x 4096 (8) 2.87, 2.61, 2.95, 3072 x 1024 (11) 2.95, 2.84,
-        // 2.94, 4096 x 4096 (28) 4.18, 4.10, 4.83, 6144 x 3072 (42) 4.91, 5.11; three slices 2048 x 6144 (21) 3.90, 4.36 (six warps).
-        warps = per_sm == 1 && S <= 2 && units_per_cta <= 28 ? (S == 1 && units_per_cta <= 7 ? 4 : 8) : -1;
+        // 2.94, 4096 x 4096 (28) 4.18, 4.10, 4.83, 6144 x 3072 (42) 4.91, 5.11; three slices 2048 x 6144 (21) 3.90, 4.36 (six warps).  Over 260
+        // shapes of up to 28 units 0.85 to 1.02 of the time with 16, 0.95 on average in every range; of 29 to 45 units 0.99 to 1.02.
+        // Beside a small-batch kernel the line lies lower (the row left alone of 5 to 61 at level 0, against 16 warps: one slice, up to four
+        // units 0.87 to 1.03, five 0.97 to 1.00, six to 28 0.89 to 1.14, mostly above 1.02; two slices, up to 14 units 0.86 to 1.03, 22 units
+        // at level 2 1.05 to 1.09).
+        const long most = !beside ? 28 : S == 1 ? 4 : 14;
+        warps = per_sm == 1 && S <= 2 && units_per_cta <= most ? (S == 1 && units_per_cta <= 7 ? 4 : 8) : -1;
     }
     if (warps == -1) {
         // the caller knows that the call runs alone (copies on both sides of it): one CTA takes the whole SM

@@ -136,7 +136,7 @@ ptqtp_status launch_pack2(const Layout2& L, const int8_t* T1, const int8_t* T2, 
 ptqtp_status launch_unpack2(const Layout2& L, const void* packed, int8_t* T1, int8_t* T2, uint16_t* a1,
                             uint16_t* a2, int32_t* dev_status, cudaStream_t st);
 ptqtp_status launch_gemv2(const Layout2& L, const void* packed, const uint16_t* x, uint16_t* y, int warps,
-                          int ctas_per_sm, int depth, int units, cudaStream_t st, bool gated = false, bool in_order = false);
+                          int ctas_per_sm, int depth, int units, cudaStream_t st, bool gated = false, bool in_order = false, bool beside = false);
 ptqtp_status launch_pack3(const Layout3& L, const int8_t* T1, const int8_t* T2, const uint16_t* a1,
                           const uint16_t* a2, void* packed, int32_t* dev_status, cudaStream_t st);
 ptqtp_status launch_unpack3(const Layout3& L, const void* packed, int8_t* T1, int8_t* T2, uint16_t* a1,
