@@ -39,7 +39,7 @@ pack2_kernel(Layout2 L, const int8_t* __restrict__ T1, const int8_t* __restrict_
              const uint16_t* __restrict__ a2, unsigned char* __restrict__ packed, int32_t* dev_status) {
     const size_t stride = (size_t)gridDim.x * blockDim.x;
     const size_t tid = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    in_order();
+    in_order(T1, T2, a1, a2);
     unsigned char* codes = packed + L.codes_off;
     bool bad = false;
 
@@ -74,8 +74,8 @@ pack2_kernel(Layout2 L, const int8_t* __restrict__ T1, const int8_t* __restrict_
         for (int r = 0; r < 2; ++r) {
             const int row = 2 * rp + r;
             if (row < L.n) {
-                s[2 * r] = a1[(size_t)row * groups + g];
-                s[2 * r + 1] = a2[(size_t)row * groups + g];
+                s[2 * r] = __ldcg(a1 + (size_t)row * groups + g);
+                s[2 * r + 1] = __ldcg(a2 + (size_t)row * groups + g);
             }
         }
         unsigned char* dst = codes + unit_offset(L, rp, slice) + (size_t)active * 64 + gl * 8;
@@ -110,7 +110,7 @@ template <class I, int A>
 __global__ void __launch_bounds__(kThreadsP2)
 unpack2_kernel(Layout2 L, const unsigned char* __restrict__ packed, int8_t* __restrict__ T1, int8_t* __restrict__ T2,
                uint16_t* __restrict__ a1, uint16_t* __restrict__ a2, int32_t* dev_status) {
-    in_order();
+    in_order(packed);
     if (blockIdx.x == 0 && threadIdx.x == 0 && dev_status) {
         const Header* h = reinterpret_cast<const Header*>(packed);
         const char m[8] = {'P', 'T', 'Q', 'T', 'P', 'B', '2', '\0'};
@@ -148,8 +148,7 @@ unpack2_kernel(Layout2 L, const unsigned char* __restrict__ packed, int8_t* __re
         const int rp = (int)(q / groups), g = (int)(q % groups);
         const int slice = g / 16, gl = g % 16;
         const int active = active_of(L, slice);
-        const uint2 s = *reinterpret_cast<const uint2*>(codes + unit_offset(L, rp, slice) +
-                                                        (size_t)active * 64 + gl * 8);
+        const uint2 s = __ldcg(reinterpret_cast<const uint2*>(codes + unit_offset(L, rp, slice) + (size_t)active * 64 + gl * 8));
         const uint32_t v[2] = {s.x, s.y};
 #pragma unroll
         for (int r = 0; r < 2; ++r) {

@@ -38,7 +38,7 @@ __device__ __forceinline__ Run3 run_of(const Layout3& L) {
 __global__ void __launch_bounds__(kThreadsPack3)
 pack3_kernel(Layout3 L, const int8_t* __restrict__ T1, const int8_t* __restrict__ T2, const uint16_t* __restrict__ a1,
              const uint16_t* __restrict__ a2, unsigned char* __restrict__ packed, int32_t* dev_status) {
-    in_order();
+    in_order(T1, T2, a1, a2);
     unsigned char* codes = packed + L.codes_off;
     bool bad = false;
     const Run3 p = run_of(L);
@@ -72,8 +72,8 @@ pack3_kernel(Layout3 L, const int8_t* __restrict__ T1, const int8_t* __restrict_
         for (int r = 0; r < 2; ++r) {
             const int row = 2 * (p.rb * kTileRp3 + g) + r;
             if (row < L.n && grp < groups) {
-                s[2 * r] = a1[(size_t)row * groups + grp];
-                s[2 * r + 1] = a2[(size_t)row * groups + grp];
+                s[2 * r] = __ldcg(a1 + (size_t)row * groups + grp);
+                s[2 * r + 1] = __ldcg(a2 + (size_t)row * groups + grp);
             }
         }
         *reinterpret_cast<uint2*>(codes + p.tile_off + kTileCodes3 + l * 8) =
@@ -97,7 +97,7 @@ pack3_kernel(Layout3 L, const int8_t* __restrict__ T1, const int8_t* __restrict_
 __global__ void __launch_bounds__(kThreadsUnpack3)
 unpack3_kernel(Layout3 L, const unsigned char* __restrict__ packed, int8_t* __restrict__ T1, int8_t* __restrict__ T2,
                uint16_t* __restrict__ a1, uint16_t* __restrict__ a2, int32_t* dev_status) {
-    in_order();
+    in_order(packed);
     if (blockIdx.x == 0 && threadIdx.x == 0 && dev_status) {
         const Header* h = reinterpret_cast<const Header*>(packed);
         const char m[8] = {'P', 'T', 'Q', 'T', 'P', 'B', '2', '\0'};
@@ -129,7 +129,7 @@ unpack3_kernel(Layout3 L, const unsigned char* __restrict__ packed, int8_t* __re
 
     const int groups = L.k / kGroup, l = threadIdx.x % kTileThreads3, grp = 4 * p.sb + (l & 3);
     if (p.live && l < 32 && grp < groups) {
-        const uint2 s = *reinterpret_cast<const uint2*>(codes + p.tile_off + kTileCodes3 + l * 8);
+        const uint2 s = __ldcg(reinterpret_cast<const uint2*>(codes + p.tile_off + kTileCodes3 + l * 8));
         const uint32_t v[2] = {s.x, s.y};
 #pragma unroll
         for (int r = 0; r < 2; ++r) {

@@ -238,9 +238,14 @@ ptqtp_status launch_in_order(void (*kernel)(P...), unsigned grid, int threads, s
     if (e != cudaSuccess) { set_last_cuda_error(e); (void)cudaGetLastError(); return PTQTP_ERR_CUDA; }
     return PTQTP_OK;
 }
-// Waits until everything before this kernel on the stream is complete, then lets the next launch begin its own set-up.
-__device__ __forceinline__ void in_order() {
+// Waits until everything before this kernel on the stream is complete, then lets the next launch begin its own set-up.  reads: the pointers
+// to what others wrote.  A kernel that is resident before its inputs are complete must not take them for constant, as the compiler
+// may with a `const __restrict__` parameter (a load ahead of the wait, or through the non-coherent cache): the pointers come out of an
+// assembly statement behind the wait, and what is read through them is read by coherent loads (__ldcg, __ldcs).
+template <class... P>
+__device__ __forceinline__ void in_order(P&... reads) {
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    (..., [](P& p) { asm volatile("" : "+l"(p)::"memory"); }(reads));
     asm volatile("griddepcontrol.launch_dependents;");
 }
 

@@ -323,37 +323,52 @@ def test_polls_of_the_tcgen05_kernel_do_not_count_the_time_of_the_kernel_ahead(n
 
 
 @pytest.mark.parametrize("fmt", [V2, V3])
-@pytest.mark.parametrize("form", ["pack", "unpack", "decompose"])
-def test_conversions_follow_stream_order_between_dependent_launches(neighbours, form, fmt):
-    # a kernel ahead that releases its dependents at once and writes late what the call reads; a kernel behind that reads without waiting sees
-    # what that kernel wrote
+@pytest.mark.parametrize("late", ["pack T1", "pack T2", "pack alpha1", "pack alpha2", "unpack codes", "unpack scales", "unpack header", "decompose W"])
+def test_conversions_follow_stream_order_between_dependent_launches(neighbours, late, fmt):
+    # a kernel ahead that releases its dependents at once and writes late what the call reads, each operand in turn; a kernel behind that reads
+    # without waiting sees what that kernel wrote
     n, k = 48, 1152
     c = make_case(n, k, seed=62)
-    planes = [dev(c[v]) for v in ("T1", "T2", "alpha1", "alpha2")]
-    blob = binding.ptqtp_pack(*planes, fmt=fmt)[0]
+    form, what = late.split()
+    planes = dict((v, dev(c[v])) for v in ("T1", "T2", "alpha1", "alpha2"))
+    blob = binding.ptqtp_pack(*planes.values(), fmt=fmt)[0]
     W, status = torch.randn((n, k), generator=torch.Generator().manual_seed(5)).cuda(), torch.zeros(1, dtype=torch.int32, device="cuda")
-    source = {"pack": planes[0], "unpack": blob, "decompose": W}[form]
 
     def call():
         if form == "pack":
-            return binding.ptqtp_pack(*planes, packed=torch.empty_like(blob), dev_status=status, fmt=fmt)[0]
-        return binding.ptqtp_unpack(blob, n, k, dev_status=status, fmt=fmt)[0] if form == "unpack" else binding.ptqtp_decompose(W)[0]
+            return binding.ptqtp_pack(*planes.values(), packed=torch.empty_like(blob), dev_status=status, fmt=fmt)
+        return binding.ptqtp_unpack(blob, n, k, dev_status=status, fmt=fmt) if form == "unpack" else binding.ptqtp_decompose(W)
 
-    # the late word: four trits, the bytes of four columns, or a weight
-    words = source.view(torch.uint8).flatten()[256:256 + 4 * 64].view(torch.int32) if form == "unpack" else source.flatten().view(torch.int32)
+    # the late word: four trits, two scales, the bytes of four columns, the scales of a row pair, the version of the format, or a weight
+    word = 0
+    if form == "unpack":
+        other = planes["alpha1"].clone()
+        other[0, 0] += 1
+        scales = int((binding.ptqtp_pack(planes["T1"], planes["T2"], other, planes["alpha2"], fmt=fmt)[0] != blob).nonzero()[0])
+        word = {"codes": 64, "scales": scales // 4, "header": 2}[what]
+    source = blob if form == "unpack" else W if form == "decompose" else planes[what]
+    words = source.flatten().view(torch.int32)[word:]
     old = int(words[0].item())
-    new = {"pack": 0x0100ff01, "unpack": 0x55555555, "decompose": 0x3f800000}[form]
+    new = {"T1": 0x0100ff01, "T2": 0x0100ff01, "alpha1": 0x3c003800, "alpha2": 0x3c003800, "codes": 0x55555555, "scales": 0x3c003800, "header": 99,
+           "W": 0x3f800000}[what]
+    assert old != new
     stream, seen = torch.cuda.Stream(), torch.zeros(8, dtype=torch.int32, device="cuda")
+    kept = []
     with torch.cuda.stream(stream):
         for i in range(4):
             value = new if i % 2 == 0 else old
+            status.zero_()
             words[0] = value
-            want = call().clone()
+            want = [t.clone() for t in call()]
             words[0] = old if i % 2 == 0 else new
+            status.zero_()
             stream.synchronize()
             assert neighbours.run_late_writer(words.data_ptr(), value, 200_000, stream.cuda_stream) == 0
             got = call()
             assert neighbours.run_early_reader(words.data_ptr(), seen.data_ptr() + 4 * i, stream.cuda_stream) == 0
             stream.synchronize()
-            assert torch.equal(got, want), (form, i)
+            assert all(torch.equal(g, w) for g, w in zip(got, want)), i
             assert int(seen[i].item()) == value
+            kept.append(want)
+    # the word matters
+    assert any(not torch.equal(a, b) for a, b in zip(kept[0], kept[1]))
