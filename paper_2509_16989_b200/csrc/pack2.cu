@@ -1,10 +1,10 @@
 // Pack / unpack kernels of the PTQTP-B200 format 2 (layout described in ptqtp.h).
 // A thread handles 16-byte atoms: 16 columns of one row pair, both planes.  Atoms are numbered along the rows, so that
-// neighbouring lanes read neighbouring columns (numbered in storage order they would read every fourth 16 bytes); two
-// atoms per thread are in flight.  Bound by memory: 14336 x 4096 packs in 27.7 us and unpacks in 24.6 (27.8 and 24.9 with CTAs of
-// 256 threads, 31.1 and 25.6 with 512; 43.7 and 42.5 with atoms in storage order, a division in 64 bits for each and byte-wise
-// coding).  Streaming stores of the blob would bring 27.2, but who reads it next finds it in L2 without them (a call of ptqtp_unpack right
-// after 55 us with the host's part, 61 from memory).
+// neighbouring lanes read neighbouring columns (numbered in storage order they would read every fourth 16 bytes).  Bound by memory: in a
+// chain of calls 13506 x 4096 packs in 23.0 us and unpacks in 22.9 (24.8 and 22.9 with two atoms per packing thread, 24.6 and 22.9 with
+// that, CTAs of 256 threads and plain launches; 43.7 and 42.5 for 14336 x 4096 with atoms in storage order, a division in 64 bits for each and
+// byte-wise coding).  Streaming stores of the blob would bring 2 %, but who reads it next finds it in L2 without them (a call of
+// ptqtp_unpack right after 55 us with the host's part, 61 from memory).
 #include "trit_bytes.h"
 
 namespace ptqtp {
@@ -33,7 +33,7 @@ __device__ __forceinline__ size_t atom_offset(const Layout2& L, int rp, int col)
     return unit_offset(L, rp, slice) + (size_t)((c / 16 % 4) * active_of(L, slice) + c / kLane2) * 16;
 }
 
-template <class I, int A>
+template <class I>
 __global__ void __launch_bounds__(kThreadsP2)
 pack2_kernel(Layout2 L, const int8_t* __restrict__ T1, const int8_t* __restrict__ T2, const uint16_t* __restrict__ a1,
              const uint16_t* __restrict__ a2, unsigned char* __restrict__ packed, int32_t* dev_status) {
@@ -43,24 +43,18 @@ pack2_kernel(Layout2 L, const int8_t* __restrict__ T1, const int8_t* __restrict_
     unsigned char* codes = packed + L.codes_off;
     bool bad = false;
 
-    int rp[A], col[A];
-    bool live[A];
-    uint4 v[A][4];                                 // (row, plane 1), (row, plane 2), (row + 1, plane 1), (row + 1, plane 2)
-#pragma unroll
-    for (int n = 0; n < A; ++n) {
-        live[n] = atom_of<I, A>(L, n, rp[n], col[n]);
+    int rp, col;
+    if (atom_of<I, 1>(L, 0, rp, col)) {
+        uint4 v[4];                                // (row, plane 1), (row, plane 2), (row + 1, plane 1), (row + 1, plane 2)
 #pragma unroll
         for (int r = 0; r < 2; ++r) {
-            const bool in = live[n] && 2 * rp[n] + r < L.n;
-            const size_t at = (size_t)(2 * rp[n] + r) * L.k + col[n];
-            v[n][2 * r] = in ? __ldcs(reinterpret_cast<const uint4*>(T1 + at)) : make_uint4(0u, 0u, 0u, 0u);
-            v[n][2 * r + 1] = in ? __ldcs(reinterpret_cast<const uint4*>(T2 + at)) : make_uint4(0u, 0u, 0u, 0u);
+            const bool in = 2 * rp + r < L.n;
+            const size_t at = (size_t)(2 * rp + r) * L.k + col;
+            v[2 * r] = in ? __ldcs(reinterpret_cast<const uint4*>(T1 + at)) : make_uint4(0u, 0u, 0u, 0u);
+            v[2 * r + 1] = in ? __ldcs(reinterpret_cast<const uint4*>(T2 + at)) : make_uint4(0u, 0u, 0u, 0u);
         }
+        *reinterpret_cast<uint4*>(codes + atom_offset(L, rp, col)) = pair_words(v[0], v[1], v[2], v[3], bad);
     }
-#pragma unroll
-    for (int n = 0; n < A; ++n)
-        if (live[n])
-            *reinterpret_cast<uint4*>(codes + atom_offset(L, rp[n], col[n])) = pair_words(v[n][0], v[n][1], v[n][2], v[n][3], bad);
 
     // scale quads: one per row pair and 128-column group, after the codes of their slice unit
     const int groups = L.k / kGroup;
@@ -166,17 +160,32 @@ unsigned ctas_for2(const Layout2& L, int atoms) {
     const size_t per_cta = (size_t)kThreadsP2 * atoms;
     return (unsigned)(((size_t)L.nrp * (L.k / 16) + per_cta - 1) / per_cta);
 }
-// Two atoms per thread once that still leaves every SM eight CTAs (1024 x 1024: 4.2 us with two, 3.5 with one).
-bool two_atoms2(const Layout2& L) { return ctas_for2(L, 2) >= 8u * (unsigned)sm_count(); }
 bool index32_2(const Layout2& L) { return (size_t)L.nrp * (L.k / 16) < ((size_t)1 << 32) - 2 * kThreadsP2; }
+constexpr unsigned kResident2 = 16;                // CTAs per SM: 128 threads of 32 registers at most
+
+// Packing as a dependent launch: where the CTAs of two launches find room beside each other (468 x 4096 2.7 us instead of 3.1), and from three
+// waves on (8054 x 4096 13.6 instead of 14.0).  In between the next launch's CTAs leave no room for the rest of this one's
+// or start unevenly: 1438 x 4096 4.8 us against 4.1 with plain launches, 9195 x 640 6.3 and 4.6, 28195 x 640 11.9 and 8.9 (with K a
+// multiple of 2048 dependent launches would be the better ones again from one wave on, 3708 x 4096 7.0 and 7.4).
+bool pack_dependent2(unsigned ctas) {
+    const unsigned wave = kResident2 * (unsigned)sm_count();
+    return 2 * ctas <= wave || ctas >= 3 * wave;
+}
+// Unpacking: two atoms per thread where each SM gets two CTAs or more and the CTAs of two launches find room beside each other (860 x 6272
+// 3.8 us instead of 4.2), and from a wave and a half on (8778 x 4096 11.8 and 12.2); one in between (2410 x 4096 4.5, with two atoms 5.6)
+// and below (191 x 1024 2.6 and 2.9).  (Packing takes one everywhere: 1860 x 4096 4.6 with one, 5.4 with two, 13506 x 4096 23.0 and 24.8.)
+bool two_atoms2(const Layout2& L) {
+    const unsigned sms = (unsigned)sm_count(), wave = kResident2 * sms, ctas = ctas_for2(L, 2);
+    return ctas >= 2 * sms && (2 * ctas <= wave || 2 * ctas >= 3 * wave);
+}
 
 }  // namespace
 
 ptqtp_status launch_pack2(const Layout2& L, const int8_t* T1, const int8_t* T2, const uint16_t* a1,
                           const uint16_t* a2, void* packed, int32_t* dev_status, cudaStream_t st) {
-    const bool two = two_atoms2(L);
-    auto kern = !two ? pack2_kernel<uint32_t, 1> : index32_2(L) ? pack2_kernel<uint32_t, 2> : pack2_kernel<size_t, 2>;
-    return launch_in_order(kern, ctas_for2(L, two ? 2 : 1), kThreadsP2, 0, st, L, T1, T2, a1, a2, static_cast<unsigned char*>(packed), dev_status);
+    const unsigned ctas = ctas_for2(L, 1);
+    return launch_in_order_if(pack_dependent2(ctas), index32_2(L) ? pack2_kernel<uint32_t> : pack2_kernel<size_t>, ctas, kThreadsP2, 0, st, L, T1, T2, a1, a2,
+                              static_cast<unsigned char*>(packed), dev_status);
 }
 
 ptqtp_status launch_unpack2(const Layout2& L, const void* packed, int8_t* T1, int8_t* T2, uint16_t* a1,

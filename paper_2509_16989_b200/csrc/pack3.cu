@@ -5,7 +5,7 @@
 // packs in 26.7 us and unpacks in 25.6 (5.6 and 5.9 TB/s; 61.9 and 112 with four-byte accesses and byte-wise coding).  Packing takes a
 // tile per CTA (two tiles 27.5; four 32.9; a loop of CTAs that stay, the next tile's loads in flight, 41; streaming stores of the blob
 // 26.2, but who reads it next finds it in L2 without them); unpacking two (one tile: 25.4 there, but 4.2 against 3.9 on 1024 x 4096).
-// Launched as dependents that wait first: call after call of the binding 27.1 us packing and 26.9 unpacking 14336 x 4096 (28.8 and 28.7 with
+// Launched as dependents that wait first, mostly: call after call of the binding 27.1 us packing and 26.9 unpacking 14336 x 4096 (28.8 and 28.7 with
 // plain launches).
 #include "trit_bytes.h"
 
@@ -142,6 +142,15 @@ unpack3_kernel(Layout3 L, const unsigned char* __restrict__ packed, int8_t* __re
     }
 }
 
+// A plain launch where the CTAs of this launch fill between a half and three quarters of the device's places, so that only some of the
+// next launch's find room beside them: packing 1708 x 4096 4.8 to 5.0 us, 5.2 as a dependent launch (469 x 4096 3.5 instead of 4.0, 2410 x 4096
+// 5.4 instead of 5.6, 13506 x 4096 23.1 instead of 23.4), unpacking 2410 x 4096 5.2 and 6.6, 11196 x 640 4.4 and 5.4 (1860 x 4096 4.6
+// instead of 4.8, 4042 x 4096 7.3 instead of 7.4, 13506 x 4096 23.2 instead of 23.6).  resident: CTAs per SM, by the registers.
+bool dependent3(unsigned ctas, unsigned resident) {
+    const unsigned wave = resident * (unsigned)sm_count();
+    return 2 * ctas <= wave || 4 * ctas > 3 * wave;
+}
+constexpr unsigned kResidentPack3 = 10, kResidentUnpack3 = 8;      // 48 and 32 registers a thread
 unsigned grid_for3(const Layout3& L, int threads) {
     const size_t per_cta = threads / kTileThreads3;
     return (unsigned)(((size_t)L.nrb * L.sbs + per_cta - 1) / per_cta);
@@ -151,13 +160,16 @@ unsigned grid_for3(const Layout3& L, int threads) {
 
 ptqtp_status launch_pack3(const Layout3& L, const int8_t* T1, const int8_t* T2, const uint16_t* a1,
                           const uint16_t* a2, void* packed, int32_t* dev_status, cudaStream_t st) {
-    return launch_in_order(pack3_kernel, grid_for3(L, kThreadsPack3), kThreadsPack3, 0, st, L, T1, T2, a1, a2, static_cast<unsigned char*>(packed), dev_status);
+    const unsigned grid = grid_for3(L, kThreadsPack3);
+    return launch_in_order_if(dependent3(grid, kResidentPack3), pack3_kernel, grid, kThreadsPack3, 0, st, L, T1, T2, a1, a2, static_cast<unsigned char*>(packed),
+                              dev_status);
 }
 
 ptqtp_status launch_unpack3(const Layout3& L, const void* packed, int8_t* T1, int8_t* T2, uint16_t* a1,
                             uint16_t* a2, int32_t* dev_status, cudaStream_t st) {
-    return launch_in_order(unpack3_kernel, grid_for3(L, kThreadsUnpack3), kThreadsUnpack3, 0, st, L, static_cast<const unsigned char*>(packed), T1, T2, a1, a2,
-                           dev_status);
+    const unsigned grid = grid_for3(L, kThreadsUnpack3);
+    return launch_in_order_if(dependent3(grid, kResidentUnpack3), unpack3_kernel, grid, kThreadsUnpack3, 0, st, L, static_cast<const unsigned char*>(packed), T1, T2,
+                              a1, a2, dev_status);
 }
 
 }  // namespace ptqtp

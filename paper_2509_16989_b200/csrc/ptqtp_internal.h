@@ -221,9 +221,9 @@ inline ptqtp_status configure_once(bool with_carveout = true) {
 
 
 // A launch in stream order whose set-up overlaps the end of the kernel before it: a dependent launch of a kernel that executes in_order()
-// before it touches any memory that others see.
+// before it touches any memory that others see.  dependent = false: a plain launch of such a kernel.
 template <class... P, class... A>
-ptqtp_status launch_in_order(void (*kernel)(P...), unsigned grid, int threads, size_t smem, cudaStream_t st, A... args) {
+ptqtp_status launch_in_order_if(bool dependent, void (*kernel)(P...), unsigned grid, int threads, size_t smem, cudaStream_t st, A... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(threads);
@@ -233,10 +233,14 @@ ptqtp_status launch_in_order(void (*kernel)(P...), unsigned grid, int threads, s
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = dependent ? 1 : 0;
     const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
     if (e != cudaSuccess) { set_last_cuda_error(e); (void)cudaGetLastError(); return PTQTP_ERR_CUDA; }
     return PTQTP_OK;
+}
+template <class... P, class... A>
+ptqtp_status launch_in_order(void (*kernel)(P...), unsigned grid, int threads, size_t smem, cudaStream_t st, A... args) {
+    return launch_in_order_if(true, kernel, grid, threads, smem, st, args...);
 }
 // Waits until everything before this kernel on the stream is complete, then lets the next launch begin its own set-up.  reads: the pointers
 // to what others wrote.  A kernel that is resident before its inputs are complete must not take them for constant, as the compiler

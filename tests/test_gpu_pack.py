@@ -165,3 +165,18 @@ def test_every_byte_value_next_to_valid_trits(fmt, N, K):
         assert np.array_equal(U.cpu().numpy(), np.where(np.abs(T.astype(np.int32)) <= 1, T, 0))
     assert np.array_equal(b1.cpu().numpy().view(np.uint16), a[0].view(np.uint16))
     assert np.array_equal(b2.cpu().numpy().view(np.uint16), a[1].view(np.uint16))
+
+
+@pytest.mark.parametrize("fmt", [binding.FORMAT_V2, binding.FORMAT_V3])
+@pytest.mark.parametrize("ctas", [295, 296, 592, 593, 740, 741, 888, 889, 1110, 1111, 1184, 1185, 3552, 7104])
+@pytest.mark.parametrize("K", [640, 2048])
+def test_either_side_of_the_lines_between_forms_of_launch(K, ctas, fmt):
+    # what is launched how, and with how many atoms per thread, goes by the number of CTAs (128 or 256 atoms of 16 columns of a row pair; on
+    # format 3 one or two tiles): rows for about that many, the last pair cut short
+    for atoms in (128, 256) if ctas < 2000 else (128,):
+        N = 2 * (ctas * atoms // (K // 16)) - 1
+        g = torch.Generator(device="cuda").manual_seed(ctas)
+        planes = [torch.randint(-1, 2, (N, K), generator=g, device="cuda", dtype=torch.int8).cpu().numpy() for _ in range(2)]
+        scales = [torch.rand((N, K // 128), generator=g, device="cuda").half().cpu().numpy() for _ in range(2)]
+        c = dict(zip(("T1", "T2", "alpha1", "alpha2"), planes + scales), N=N, K=K)
+        assert np.array_equal(roundtrip(c, fmt), reference_blob(c, fmt))
