@@ -22,12 +22,23 @@ def _nvcc():
     return "nvcc"
 
 
-def needs_build():
-    if not os.path.exists(LIB) or not os.path.exists(MARSHAL):
+def _stale(target, sources):
+    if not os.path.exists(target):
         return True
-    t = min(os.path.getmtime(LIB), os.path.getmtime(MARSHAL))
-    deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)] + [os.path.join(ROOT, "include", "ptqtp.h")]
-    return any(os.path.getmtime(d) > t for d in deps)
+    t = os.path.getmtime(target)
+    return any(os.path.getmtime(d) > t for d in sources + [os.path.join(ROOT, "include", "ptqtp.h")])
+
+
+def library_stale():
+    return _stale(LIB, [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith((".cu", ".h"))])
+
+
+def marshal_stale():
+    return _stale(MARSHAL, [os.path.join(CSRC, "marshal.cpp")])
+
+
+def needs_build():
+    return library_stale() or marshal_stale()
 
 
 def build_marshal():
@@ -42,24 +53,30 @@ def build_marshal():
            "-L", os.path.join(root, "lib"), "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python", "-o", MARSHAL]
     res = subprocess.run(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)
     if res.returncode != 0:
-        sys.stderr.write(res.stdout)
-        raise RuntimeError("building _marshal.so failed")
+        raise RuntimeError("%s failed\n%s" % (cmd[0], res.stdout))
 
 
 def build(force=False, verbose=False, extra=()):
-    """Compile every CUDA source into paper_2509_16989_b200/libptqtp.so and the marshalling extension; returns the library's path."""
-    if not force and not needs_build():
-        return LIB
-    cmd = [_nvcc()] + NVCC_FLAGS + list(extra) + ["-I", os.path.join(ROOT, "include"), "-I", CSRC]
-    if verbose:
-        cmd += ["-Xptxas", "-v"]
-    cmd += [os.path.join(CSRC, s) for s in SOURCES] + ["-o", LIB]
-    res = subprocess.run(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)
-    if verbose or res.returncode != 0:
-        sys.stderr.write(res.stdout)
-    if res.returncode != 0:
-        raise RuntimeError("nvcc failed building libptqtp.so")
-    build_marshal()
+    """Compile every CUDA source into paper_2509_16989_b200/libptqtp.so and the marshalling extension, what is not up to date of the two;
+    returns the library's path.  The library needs no torch; the binding runs without the extension, only slower, so where that cannot be
+    built (no host compiler, no torch or Python headers) a message is printed."""
+    if force or library_stale():
+        cmd = [_nvcc()] + NVCC_FLAGS + list(extra) + ["-I", os.path.join(ROOT, "include"), "-I", CSRC]
+        if verbose:
+            cmd += ["-Xptxas", "-v"]
+        cmd += [os.path.join(CSRC, s) for s in SOURCES] + ["-o", LIB]
+        res = subprocess.run(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)
+        if verbose or res.returncode != 0:
+            sys.stderr.write(res.stdout)
+        if res.returncode != 0:
+            raise RuntimeError("nvcc failed building libptqtp.so")
+    if force or marshal_stale():
+        try:
+            build_marshal()
+        except (ImportError, OSError, RuntimeError) as e:
+            if os.path.exists(MARSHAL):                  # of older sources
+                os.remove(MARSHAL)
+            sys.stderr.write("the marshalling extension was not built, plain calls of the binding take the slower way: %s\n" % e)
     return LIB
 
 
