@@ -9,7 +9,6 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libptqtp.so")
-MARSHAL = os.path.join(HERE, "_marshal.so")
 SOURCES = ["api.cu", "pack.cu", "pack2.cu", "gemv.cu", "gemv2.cu", "gemv3.cu", "pack3.cu", "gemv4.cu", "gemv5.cu", "gemm7.cu", "gemm8.cu", "skinny3.cu", "decompose.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "-Xcompiler", "-fvisibility=hidden", "--shared", "-cudart", "shared"]
@@ -20,6 +19,12 @@ def _nvcc():
         if cand and (os.path.isabs(cand) and os.path.exists(cand) or not os.path.isabs(cand)):
             return cand
     return "nvcc"
+
+
+def marshal_path():
+    """The extension's file, which belongs to one Python and one torch: it is made of the headers of both."""
+    import torch
+    return os.path.join(HERE, "_marshal-%s%s" % (torch.__version__, sysconfig.get_config_var("EXT_SUFFIX")))
 
 
 def _stale(target, sources):
@@ -34,7 +39,10 @@ def library_stale():
 
 
 def marshal_stale():
-    return _stale(MARSHAL, [os.path.join(CSRC, "marshal.cpp")])
+    try:
+        return _stale(marshal_path(), [os.path.join(CSRC, "marshal.cpp")])
+    except ImportError:
+        return False                                     # without torch nobody calls it
 
 
 def needs_build():
@@ -42,15 +50,15 @@ def needs_build():
 
 
 def build_marshal():
-    """Compile csrc/marshal.cpp into paper_2509_16989_b200/_marshal.so against the torch that is installed."""
+    """Compile csrc/marshal.cpp against the torch that is installed."""
     import torch
     root = os.path.dirname(torch.__file__)
     cuda = os.path.dirname(os.path.dirname(_nvcc())) if os.path.isabs(_nvcc()) else "/usr/local/cuda"
     cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
-           "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI), "-I", os.path.join(ROOT, "include"),
+           "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI), '-DPTQTP_TORCH_VERSION="%s"' % torch.__version__, "-I", os.path.join(ROOT, "include"),
            "-I", sysconfig.get_paths()["include"], "-isystem", os.path.join(cuda, "include"), "-isystem", os.path.join(root, "include"),
            "-isystem", os.path.join(root, "include", "torch", "csrc", "api", "include"), os.path.join(CSRC, "marshal.cpp"),
-           "-L", os.path.join(root, "lib"), "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python", "-o", MARSHAL]
+           "-L", os.path.join(root, "lib"), "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python", "-o", marshal_path()]
     res = subprocess.run(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)
     if res.returncode != 0:
         raise RuntimeError("%s failed\n%s" % (cmd[0], res.stdout))
@@ -74,8 +82,8 @@ def build(force=False, verbose=False, extra=()):
         try:
             build_marshal()
         except (ImportError, OSError, RuntimeError) as e:
-            if os.path.exists(MARSHAL):                  # of older sources
-                os.remove(MARSHAL)
+            if not isinstance(e, ImportError) and os.path.exists(marshal_path()):           # of older sources
+                os.remove(marshal_path())
             sys.stderr.write("the marshalling extension was not built, plain calls of the binding take the slower way: %s\n" % e)
     return LIB
 

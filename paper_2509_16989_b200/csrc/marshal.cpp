@@ -8,7 +8,6 @@
 #include <c10/core/impl/TorchDispatchModeTLS.h>
 #include <c10/cuda/CUDAStream.h>
 #include <torch/csrc/autograd/python_variable.h>
-#include <torch/version.h>
 #include "ptqtp.h"
 
 namespace {
@@ -131,6 +130,6 @@ PyModuleDef g_module = {PyModuleDef_HEAD_INIT, "_marshal", nullptr, -1, g_method
 
 extern "C" __attribute__((visibility("default"))) PyObject* PyInit__marshal() {
     PyObject* m = PyModule_Create(&g_module);
-    if (m && PyModule_AddStringConstant(m, "torch_version", TORCH_VERSION) != 0) { Py_DECREF(m); return nullptr; }
+    if (m && PyModule_AddStringConstant(m, "torch_version", PTQTP_TORCH_VERSION) != 0) { Py_DECREF(m); return nullptr; }
     return m;
 }

@@ -1,11 +1,15 @@
 """The binding's extension for plain arguments: what is not plain is left to the Python marshalling, and both do the same."""
+import os
+import sys
+import warnings
+
 import numpy as np
 import pytest
 import torch
 from torch.overrides import TorchFunctionMode
 from torch.utils._python_dispatch import TorchDispatchMode
 
-from paper_2509_16989_b200 import binding
+from paper_2509_16989_b200 import binding, build
 
 
 class Sub(torch.Tensor):
@@ -13,9 +17,42 @@ class Sub(torch.Tensor):
 
 
 def functions():
+    # an extension that was built and is not in use is a failure; none only where it cannot be built
+    if not os.path.exists(build.marshal_path()):
+        try:
+            build.build_marshal()
+        except (OSError, RuntimeError) as e:
+            pytest.skip("the extension cannot be built here: %s" % e)
+        binding._bind_plain(binding.lib())
     binding.lib()
-    m = pytest.importorskip("paper_2509_16989_b200._marshal")
-    return m
+    assert binding._gemv_plain is not None
+    return sys.modules["paper_2509_16989_b200._marshal"]
+
+
+@pytest.mark.parametrize("kind", ["missing", "broken", "another torch"])
+def test_an_extension_that_cannot_serve_is_reported(kind, tmp_path, monkeypatch):
+    functions()
+    for name in ("_gemv_plain", "_gemv_host_plain", "_gemm_skinny_plain", "_gemm_skinny_ws_plain"):
+        monkeypatch.setattr(binding, name, None)
+    path = tmp_path / "_marshal.so"
+    if kind == "broken":
+        path.write_bytes(b"no library")
+    if kind == "another torch":
+        real = build.marshal_path()
+        monkeypatch.setattr(torch, "__version__", "0.0.0+none")
+        assert not os.path.exists(build.marshal_path())  # it looks for a file of its own name
+        path = real
+    monkeypatch.setattr(build, "marshal_path", lambda: str(path))
+    with pytest.warns(RuntimeWarning, match={"missing": "not there", "broken": "does not load", "another torch": "built for torch"}[kind]):
+        binding._bind_plain(binding.lib())
+    assert binding._gemv_plain is None
+
+
+def test_a_usable_extension_is_not_reported():
+    functions()
+    with warnings.catch_warnings():
+        warnings.simplefilter("error")
+        binding._bind_plain(binding.lib())
 
 
 def test_left_alone_on_the_cpu():
