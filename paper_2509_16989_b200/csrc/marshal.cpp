@@ -22,6 +22,7 @@ struct Functions {
     Skinny skinny;
     SkinnyWs skinny_ws;
 } g_fn = {};
+bool g_bound = false;              // until bind() the functions leave every call to binding.py
 
 const c10::DispatchKeySet kWrapped({c10::DispatchKey::FuncTorchBatched, c10::DispatchKey::FuncTorchVmapMode, c10::DispatchKey::FuncTorchGradWrapper,
                                     c10::DispatchKey::Functionalize, c10::DispatchKey::Python, c10::DispatchKey::Batched});
@@ -59,7 +60,7 @@ bool modes() { return at::impl::torch_function_mode_enabled() || c10::impl::Torc
 // (packed, x, y, N, K, format)
 PyObject* gemv(PyObject*, PyObject* const* a, Py_ssize_t n) {
     ptqtp_shape s;
-    if (n != 6 || modes() || !plain_shape(a + 3, s)) PTQTP_NOT_PLAIN();
+    if (n != 6 || !g_bound || modes() || !plain_shape(a + 3, s)) PTQTP_NOT_PLAIN();
     const at::Tensor *p = plain(a[0], at::kByte), *x = plain(a[1], at::kHalf), *y = plain(a[2], at::kHalf);
     if (!p || !x || !y) PTQTP_NOT_PLAIN();
     void *pp = p->data_ptr(), *xp = x->data_ptr(), *yp = y->data_ptr();
@@ -69,7 +70,7 @@ PyObject* gemv(PyObject*, PyObject* const* a, Py_ssize_t n) {
 // (packed, x_host, y_host, x_dev, y_dev, N, K, format)
 PyObject* gemv_host(PyObject*, PyObject* const* a, Py_ssize_t n) {
     ptqtp_shape s;
-    if (n != 8 || modes() || !plain_shape(a + 5, s)) PTQTP_NOT_PLAIN();
+    if (n != 8 || !g_bound || modes() || !plain_shape(a + 5, s)) PTQTP_NOT_PLAIN();
     const at::Tensor *p = plain(a[0], at::kByte), *xh = plain(a[1], at::kHalf, true), *yh = plain(a[2], at::kHalf, true), *xd = plain(a[3], at::kHalf),
                      *yd = plain(a[4], at::kHalf);
     if (!p || !xh || !yh || !xd || !yd) PTQTP_NOT_PLAIN();
@@ -81,7 +82,7 @@ PyObject* gemv_host(PyObject*, PyObject* const* a, Py_ssize_t n) {
 // (packed, X, Y, N, K, format)
 PyObject* gemm_skinny(PyObject*, PyObject* const* a, Py_ssize_t n) {
     ptqtp_shape s;
-    if (n != 6 || modes() || !plain_shape(a + 3, s)) PTQTP_NOT_PLAIN();
+    if (n != 6 || !g_bound || modes() || !plain_shape(a + 3, s)) PTQTP_NOT_PLAIN();
     const at::Tensor *p = plain(a[0], at::kByte), *x = plain(a[1], at::kHalf), *y = plain(a[2], at::kHalf);
     if (!p || !x || !y || x->dim() < 1 || x->size(0) > 0x7fffffffL) PTQTP_NOT_PLAIN();
     void *pp = p->data_ptr(), *xp = x->data_ptr(), *yp = y->data_ptr();
@@ -92,7 +93,7 @@ PyObject* gemm_skinny(PyObject*, PyObject* const* a, Py_ssize_t n) {
 // (packed, X, Y, workspace, N, K, format)
 PyObject* gemm_skinny_ws(PyObject*, PyObject* const* a, Py_ssize_t n) {
     ptqtp_shape s;
-    if (n != 7 || modes() || !plain_shape(a + 4, s)) PTQTP_NOT_PLAIN();
+    if (n != 7 || !g_bound || modes() || !plain_shape(a + 4, s)) PTQTP_NOT_PLAIN();
     const at::Tensor *p = plain(a[0], at::kByte), *x = plain(a[1], at::kHalf), *y = plain(a[2], at::kHalf), *w = plain(a[3], at::kByte);
     if (!p || !x || !y || !w || x->dim() < 1 || x->size(0) > 0x7fffffffL) PTQTP_NOT_PLAIN();
     void *pp = p->data_ptr(), *xp = x->data_ptr(), *yp = y->data_ptr(), *wp = w->data_ptr();
@@ -107,8 +108,10 @@ PyObject* bind(PyObject*, PyObject* const* a, Py_ssize_t n) {
     for (int i = 0; i < 4; ++i) {
         f[i] = PyLong_AsVoidPtr(a[i]);
         if (PyErr_Occurred()) return nullptr;
+        if (!f[i]) { PyErr_SetString(PyExc_ValueError, "a null address"); return nullptr; }
     }
     g_fn = {reinterpret_cast<Gemv>(f[0]), reinterpret_cast<GemvHost>(f[1]), reinterpret_cast<Skinny>(f[2]), reinterpret_cast<SkinnyWs>(f[3])};
+    g_bound = true;
     Py_RETURN_NONE;
 }
 

@@ -1,5 +1,6 @@
 """The binding's extension for plain arguments: what is not plain is left to the Python marshalling, and both do the same."""
 import os
+import subprocess
 import sys
 import warnings
 
@@ -71,6 +72,30 @@ def test_what_was_refused_stays_refused_on_the_cpu():
         binding.ptqtp_gemv(b, 16, 256, h, y=h, fmt=3)
     with pytest.raises(TypeError):
         binding.ptqtp_gemm_skinny(b, 16, 256, h.reshape(1, 256), Y=h, fmt=3)
+
+
+def test_addresses_are_four_and_not_null():
+    m = functions()
+    for args, error in (((1, 2, 3), TypeError), ((0, 0, 0, 0), ValueError), ((None, 1, 2, 3), TypeError)):
+        with pytest.raises(error):
+            m.bind(*args)
+
+
+@pytest.mark.gpu
+def test_nothing_is_called_before_there_are_addresses():
+    # in a process of its own, where nothing has given them
+    functions()
+    code = """
+import importlib.util, torch
+spec = importlib.util.spec_from_file_location("_marshal", %r)
+m = importlib.util.module_from_spec(spec)
+spec.loader.exec_module(m)
+b, h = torch.zeros(1 << 20, dtype=torch.uint8, device="cuda"), torch.zeros(1152, dtype=torch.float16, device="cuda")
+p = h.cpu()
+assert m.gemv(b, h, h, 40, 1152, 3) is None and m.gemm_skinny(b, h, h, 40, 1152, 3) is None
+assert m.gemm_skinny_ws(b, h, h, b, 40, 1152, 2) is None and m.gemv_host(b, p, p, h, h, 40, 1152, 3) is None
+""" % build.marshal_path()
+    subprocess.run([sys.executable, "-c", code], check=True, timeout=300)
 
 
 @pytest.mark.gpu
