@@ -1,5 +1,8 @@
 """GPU trit-plane decomposition (ptqtp_decompose) against the CPU oracle: identical planes, scales to 1e-12, the
 same number of sweeps and the same error and change histories; the hand-worked 2 x 4 example; degenerate groups."""
+import ctypes
+import os
+import subprocess
 from fractions import Fraction
 
 import numpy as np
@@ -9,7 +12,7 @@ import torch
 from golden_io import load_worked_2x4
 from oracle.c_oracle import decompose_c
 from oracle.decompose import decompose, reconstruction_error
-from paper_2509_16989_b200 import binding
+from paper_2509_16989_b200 import binding, build
 from paper_2509_16989_b200.inputs import make_activations, make_weights
 from gpu_util import assert_parity, dev, oracle_y
 
@@ -159,6 +162,54 @@ def test_histories_with_and_without_room_for_the_records(t_max):
     for rows, G in ((1, 128), (3, 16), (40, 128)):
         W = (np.random.default_rng(600 + rows).standard_normal((rows, 2 * G)) * 0.02).astype(np.float32)
         assert_same(run(W, group=G, t_max=t_max, eps=0.0), decompose_c(W, G=G, T_max=t_max, eps=0.0), "%d %d" % (rows, t_max))
+
+
+@pytest.mark.parametrize("kind", ["normal", "few values", "short mantissas", "one plane", "planes", "extremes", "inexact sums"])
+@pytest.mark.parametrize("G", [128, 64, 20, 256])
+def test_scales_bit_for_bit(kind, G):
+    # every operation of the solve is rounded on its own, so the unrounded scales are the oracle's to the last bit, sweep by sweep
+    W = _special(kind, np.random.default_rng(900 + G))[:, :2 * G]
+    for t_max in (1, 2, 3, 9, 50):
+        got, ref = run(W, group=G, t_max=t_max, canonicalize=False), decompose_c(W, G=G, T_max=t_max, canonicalize=False)
+        for k in ("alpha1", "alpha2"):
+            assert np.array_equal(got[k].view(np.uint64), ref[k].view(np.uint64)), (t_max, k)
+
+
+def test_one_reciprocal_serves_both_divisions(tmp_path):
+    # the shared reciprocal with two corrections per quotient against IEEE divisions, and both against numpy: sums as they occur, counts of
+    # 0 to 256 weights, determinants from that of lambda alone (1e-16) on, weights from subnormal to huge, sums of zero
+    src = os.path.join(os.path.dirname(os.path.abspath(__file__)), "alpha_step.cu")
+    out = str(tmp_path / "alpha_step.so")
+    subprocess.run([build._nvcc()] + build.NVCC_FLAGS + ["-I", build.CSRC, src, "-o", out], check=True)
+    lib = ctypes.CDLL(out)
+    lib.run_compare.argtypes = [ctypes.c_void_p, ctypes.c_int, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p]
+    rng = np.random.default_rng(11)
+    n = 4_000_000
+    n11, n22 = rng.integers(0, 257, n), rng.integers(0, 257, n)
+    n11[::50], n22[::70] = 0, 0
+    n12 = np.rint((2 * rng.random(n) - 1) * np.minimum(n11, n22)).astype(np.int64)
+    n12[::9] = np.minimum(n11, n22)[::9]
+    same = rng.random(n) < 0.05                          # both planes alike: singular but for lambda
+    n22, n12 = np.where(same, n11, n22), np.where(same, n11, n12)
+    unit = np.exp2(rng.integers(-149, 105, n).astype(np.float64))
+    b1, b2 = (np.rint((2 * rng.random(n) - 1) * 2.0 ** rng.integers(0, 30, n)) * unit for _ in range(2))
+    b2 = np.where(same, b1, b2)
+    lam = np.where(rng.random(n) < 0.7, 1e-8, 10.0 ** (-8 * rng.random(n)))
+    v = np.stack([n11, n22, n12, b1 + 0.0, b2 + 0.0, lam], axis=1).astype(np.float64)
+    d_in, d_out, differ = dev(v), torch.empty((n, 3), dtype=torch.float64, device="cuda"), torch.zeros(1, dtype=torch.int32, device="cuda")
+    assert lib.run_compare(d_in.data_ptr(), n, d_out.data_ptr(), differ.data_ptr(), torch.cuda.current_stream().cuda_stream) == 0
+    got = d_out.cpu().numpy()
+    assert int(differ.item()) == 0
+    n11, n22, n12, b1, b2, lam = v.T
+    with np.errstate(all="ignore"):
+        A11, A22 = n11 + lam, n22 + lam
+        det = A11 * A22 - n12 * n12
+        kappa = ((A11 * A11 + A22 * A22) + (2.0 * n12) * n12) / np.abs(det)
+        grown = np.maximum(np.where(kappa >= 1e6, np.minimum(lam * np.sqrt(kappa / 1e6), 1.0), lam), 1e-8)
+        A11, A22 = n11 + grown, n22 + grown
+        det = A11 * A22 - n12 * n12
+        want = np.stack([(A22 * b1 - n12 * b2) / det, (A11 * b2 - n12 * b1) / det, grown], axis=1)
+    assert np.isfinite(want).all() and np.array_equal(got.view(np.uint64), want.view(np.uint64))
 
 
 def _total_error(W, T1, T2, a1, a2, G):
