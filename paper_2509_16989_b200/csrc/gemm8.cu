@@ -23,9 +23,10 @@
 //
 // What bounds it, from clock stamps in a copy of the kernel: at 64 rows the tensor pipe for two thirds of the time (37 cycles per MMA with A
 // from tensor memory, 600 a group, of about 900; the rest is not accounted for: a decoding warpgroup has one of the four stages of
-// trits there and cannot work ahead), at 16 rows the issue slots of the SM (decode 260 of them per group and scheduler; the issuing warp gets
-// its turn beside four decoding ones: 670 cycles a group, 330 of them MMAs); 3.5 us of a launch are start (first codes and
-// activations 2 us after the wait) and end.  Measured in a chain at level 0, microseconds (14336 x 4096, 4096 x 14336, 4096 x 4096,
+// trits there and cannot work ahead), at 16 rows the issue slots of the SM (670 cycles a group, 330 of them MMAs; by the counters 528
+// instructions per group and scheduler, start and end of the launch among them, three of four slots of the SMs that have a CTA; 260 of
+// them are the shifts, masks and stores of decoding, the others, loads, sums, polls and the issuing warp, have not been told apart);
+// 3.5 us of a launch are start (first codes and activations 2 us after the wait) and end.  Measured in a chain at level 0, microseconds (14336 x 4096, 4096 x 14336, 4096 x 4096,
 // 1024 x 4096), in brackets the kernel before it (trits by byte permutes and FMAs, activations by cp.async, decoding, sums and fetch in
 // the same warps): 64 rows 20.0, 20.0, 10.2, 7.4 (50.0, 43.3, 17.1, 11.3), 48 rows 18.3, 18.4, 9.1, 6.5 (40.5, 36.8, 14.4, 10.1), 32
 // rows 16.8, 16.6, 8.2, 5.8 (35.9, 32.8, 12.9, 9.0), 16 rows 15.1, 15.0, 7.4, 5.2 (30.7, 28.2, 11.4, 7.9).
